@@ -16,6 +16,8 @@
 //                       attention output and one block scores the visual rows, radix-selects the rows
 //                       to keep (ties toward the lower original index) and fills the holes among the
 //                       first n_new rows with the kept rows of the tail.
+// A prompt (prefill) is attended in the caller's tensors; a third launch, st3_gather_kernel, then copies the text and
+// the kept visual rows to the cache.
 // A step's finish launch overlaps the next step's attention launch (programmatic dependent launch,
 // ordered by per-(layer, sequence) flags).  The work decomposition is computed on the host from the
 // schedule (row counts are a pure function of layer and step), so no table is uploaded per step.
@@ -206,21 +208,40 @@ struct st3_ctx {
 
 namespace {
 
+// Launches `kernel`; `programmatic`: it may be set up (and start) while the launch ahead of it is still running.
+template <typename... A>
+cudaError_t launch(void (*kernel)(A...), unsigned grid_x, unsigned grid_y, int threads, int smem, bool programmatic,
+                   cudaStream_t st, const StepParams& p) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid_x, grid_y);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = programmatic ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, p);
+}
+
+// prefill: the layers' prompt rows stand in p.k_in / p.v_in; select_first: prune by the caller's scores, then attend.
 template <typename T, int D>
-st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, int total_items, cudaStream_t st, const void* pk,
-                         const void* pv, bool ingest, const StepParams* select_first) {
+st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, bool prefill, const StepParams* select_first) {
   const st3_config& c = ctx->cfg;
-  if (ingest) {
-    dim3 grid(8, (unsigned)(c.num_heads * c.batch * p.layer_count));
-    st3_ingest_kernel<T, D><<<grid, kThreads, 0, st>>>(p, reinterpret_cast<const T*>(pk),
-                                                       reinterpret_cast<const T*>(pv),
-                                                       c.sys_len + c.num_visual + c.max_text_len);
+  const int units = p.layer_count * c.batch;
+  const bool pdl = !ctx->profiling;  // the events between the launches want each one to end before the next begins
+  // the kept rows and the text go to the cache once the selection is known
+  auto gather = [&]() {
     ctx->launches++;
-  }
+    return launch(st3_gather_kernel<T, D>, kGatherBlocks, (unsigned)(c.num_heads * units), kThreads, 0, pdl, st,
+                  select_first ? *select_first : p) == cudaSuccess;
+  };
   if (select_first) {  // prune by the caller's scores before the layer attends
-    st3_finish_kernel<T, D, kFinishThreads><<<(unsigned)(2 * p.layer_count * c.batch), kFinishThreads, ctx->finish_smem, st>>>(
-        *select_first);
     ctx->launches++;
+    if (launch(st3_finish_kernel<T, D, kFinishThreads>, (unsigned)(2 * units), 1, kFinishThreads, ctx->finish_smem, false,
+               st, *select_first) != cudaSuccess || !gather())
+      return ST3_ERR_CUDA;
   }
   cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr;
   if (ctx->profiling) {
@@ -233,60 +254,43 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, int total_items, cud
     ctx->ev_used += 3;
     cudaEventRecord(e0, st);
   }
-  (void)total_items;
   {
     // With st3_set_overlap(ctx, 1) this is a programmatic dependent launch: it may start while the previous
     // step's finish launch is still running (that kernel allows it at its start); p.flags orders what the two
     // share.  The kernel reads the step's inputs without waiting for the launch ahead of it, which is only
     // right when those inputs were complete before that launch began - hence off unless the caller says so.
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(p.first_dynamic / kSlots));
-    cfg.blockDim = dim3(kAttendThreads);
-    cfg.dynamicSmemBytes = (size_t)ctx->attend_smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = (!ctx->overlap || ctx->profiling || ingest || ctx->serialize_next) ? 0 : 1;
+    const bool direct = prefill && !select_first;
+    const bool early = ctx->overlap && pdl && !prefill && !ctx->serialize_next;
     bool fat = false;  // some item carries lazy layers (QK heredity): the instantiation that streams their values
     for (int i = 0; i < p.layer_count; ++i) fat = fat || p.nfol[i] != 0;
-    if ((fat ? cudaLaunchKernelEx(&cfg, st3_attend_kernel<T, D, true>, p)
-             : cudaLaunchKernelEx(&cfg, st3_attend_kernel<T, D, false>, p)) != cudaSuccess)
+    auto kernel = direct ? (fat ? st3_attend_kernel<T, D, true, true> : st3_attend_kernel<T, D, false, true>)
+                         : (fat ? st3_attend_kernel<T, D, true, false> : st3_attend_kernel<T, D, false, false>);
+    if (launch(kernel, (unsigned)(p.first_dynamic / kSlots), 1, kAttendThreads, ctx->attend_smem, early, st, p) != cudaSuccess)
       return ST3_ERR_CUDA;
   }
   if (e1) cudaEventRecord(e1, st);
   {
     // Also a programmatic dependent launch: the attention kernel allows it at its start, the blocks become
     // resident as that grid drains and their first instruction waits for all of it.
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * p.layer_count * c.batch));
     // half-size blocks, two per SM, once the units outnumber the blocks the GPU holds (see st3_finish.cuh)
-    const bool half = 2 * p.layer_count * c.batch > 2 * ctx->num_sms && 2 * ctx->finish_smem <= 200 * 1024;
-    cfg.blockDim = dim3(half ? kFinishThreads / 2 : kFinishThreads);
-    cfg.dynamicSmemBytes = (size_t)ctx->finish_smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = ctx->profiling ? 0 : 1;
-    if ((half ? cudaLaunchKernelEx(&cfg, st3_finish_kernel<T, D, kFinishThreads / 2>, p)
-              : cudaLaunchKernelEx(&cfg, st3_finish_kernel<T, D, kFinishThreads>, p)) != cudaSuccess)
+    const bool half = 2 * units > 2 * ctx->num_sms && 2 * ctx->finish_smem <= 200 * 1024;
+    auto kernel = half ? st3_finish_kernel<T, D, kFinishThreads / 2> : st3_finish_kernel<T, D, kFinishThreads>;
+    if (launch(kernel, (unsigned)(2 * units), 1, half ? kFinishThreads / 2 : kFinishThreads, ctx->finish_smem, pdl, st, p) !=
+        cudaSuccess)
       return ST3_ERR_CUDA;
   }
   if (e2) cudaEventRecord(e2, st);
   ctx->launches += 2;
+  if (prefill && !select_first && !gather()) return ST3_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? ST3_OK : ST3_ERR_CUDA;
 }
 
 template <typename T, int D>
 st3_status set_attrs_t(st3_ctx* ctx) {
-  if (cudaFuncSetAttribute(st3_attend_kernel<T, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           ctx->attend_smem) != cudaSuccess ||
-      cudaFuncSetAttribute(st3_attend_kernel<T, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           ctx->attend_smem) != cudaSuccess)
-    return ST3_ERR_CUDA;
+  for (auto kernel : {st3_attend_kernel<T, D, false, false>, st3_attend_kernel<T, D, true, false>,
+                      st3_attend_kernel<T, D, false, true>, st3_attend_kernel<T, D, true, true>})
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->attend_smem) != cudaSuccess)
+      return ST3_ERR_CUDA;
   if (cudaFuncSetAttribute(st3_finish_kernel<T, D, kFinishThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            ctx->finish_smem) != cudaSuccess ||
       cudaFuncSetAttribute(st3_finish_kernel<T, D, kFinishThreads / 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -302,7 +306,7 @@ st3_status set_attrs_t(st3_ctx* ctx) {
 
 bool aligned16(const void* p) { return p && (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// Common body of prefill (step 0, ingest, no append) and decode (step >= 1, append).
+// Common body of prefill (step 0, no append) and decode (step >= 1, append).
 st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, const void* q, const void* k,
                     const void* v, void* out, cudaStream_t st, bool prefill, const float* ext_scores = nullptr) {
   const st3_config& c = ctx->cfg;
@@ -331,6 +335,7 @@ st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, co
   p.sys_len = c.sys_len; p.Nv = c.num_visual; p.cap_txt = L.cap_txt; p.step = step; p.append = prefill ? 0 : 1;
   p.chunk_rows = L.chunk_rows;
   p.static_rank = c.static_rank ? 1 : 0;
+  p.fresh = prefill && !ext_scores;
   p.k_in = prefill ? k : nullptr; p.v_in = prefill ? v : nullptr;
   p.t0_max = c.sys_len + c.num_visual + c.max_text_len;
   const int R = L.chunk_rows;
@@ -343,7 +348,7 @@ st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, co
     const int tgt = ctx->n_tab[(size_t)l * (c.max_decode_steps + 1) + step];
     if (ext_scores && tgt < ncur) ncur = tgt;  // already pruned by the selection launch when the layer attends
     p.nold[i] = ncur;
-    p.req[i] = prefill ? 0 : ctx->flag_req[l];  // prefill follows the ingest launch in stream order
+    p.req[i] = prefill ? 0 : ctx->flag_req[l];  // a prompt reads nothing the launch ahead of it writes
     if (c.static_rank && !prefill && tgt < ncur) ncur = tgt;  // cut first, then attend (Algorithm 3)
     p.ncur[i] = ncur;
     p.ntgt[i] = tgt < ncur ? tgt : ncur;
@@ -415,12 +420,13 @@ st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, co
   if (ext_scores) {  // parameters of the selection-only launch: all Nv rows held, cut to the schedule
     psel = p;
     psel.ext_scores = ext_scores;
+    psel.fresh = 1;
     for (int i = 0; i < layer_count; ++i) {
       psel.ncur[i] = psel.nold[i] = c.num_visual;
       psel.ntgt[i] = p.ncur[i];
     }
   }
-#define ST3_LAUNCH(T, D) launch_step_t<T, D>(ctx, p, (int)total_items, st, k, v, prefill, ext_scores ? &psel : nullptr)
+#define ST3_LAUNCH(T, D) launch_step_t<T, D>(ctx, p, st, prefill, ext_scores ? &psel : nullptr)
   const st3_status s = ST3_DISPATCH(ctx, ST3_LAUNCH);
 #undef ST3_LAUNCH
   if (s != ST3_OK) {
@@ -439,8 +445,9 @@ st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, co
     }
   }
   // Those logits are protected by no flag, so the launch that may overwrite them must not overlap this
-  // call's finish launch: it is launched without the programmatic attribute.
-  ctx->serialize_next = reads_older;
+  // call's finish launch: it is launched without the programmatic attribute.  Nor may it overlap the launch that
+  // copies a prompt's rows to the cache.
+  ctx->serialize_next = reads_older || prefill;
   ctx->seq++;
   ctx->counter_base += (unsigned)p.total_work;  // one fetch per work item (the first of each manager is fixed)
   ctx->last_stream = st;
@@ -673,7 +680,7 @@ st3_status st3_prefill_select_host(st3_ctx* ctx, int32_t layer_begin, int32_t la
     const int slot = (int)(ctx->pseq & 1);
     unsigned char* dk = ctx->ws + L.stage_prompt + (size_t)slot * 2 * L.prompt_bytes;
     unsigned char* dv = dk + L.prompt_bytes;
-    // layer i's rows move while the layer before it is ingested, attended and trimmed
+    // layer i's rows move while the layer before it is attended, trimmed and copied to the cache
     if (ctx->rec_pk[slot] && cudaStreamWaitEvent(ctx->s_h2d, ctx->ev_pk[slot], 0) != cudaSuccess) return ST3_ERR_CUDA;
     if (cudaMemcpyAsync(dk, static_cast<const unsigned char*>(k_host) + (size_t)i * lp, lp, cudaMemcpyHostToDevice,
                         ctx->s_h2d) != cudaSuccess ||

@@ -131,7 +131,20 @@ __device__ __forceinline__ void store_acc(float* dst, const u64 (&acc2)[DPL / 2]
 struct Chain {
   const unsigned char* srcV;  // first value row of the chunk in the item's own layer
   int oidx, lb, l_rel, nrows, has_new, is_vis;
+  int nrows1;                 // rows up to the break in the prompt tensors (see rows_g2s)
 };
+
+// Copies the rows of a chunk to a tile area.  In the prompt's tensors the visual rows stand between the system and
+// the text rows, so a text chunk may come in two pieces: `bytes1` bytes, then the rest `gap` bytes further on.
+__device__ __forceinline__ void rows_g2s(unsigned char* dst, const unsigned char* src, uint32_t bytes, uint32_t bytes1,
+                                         size_t gap, uint64_t* bar) {
+  if (bytes1 < bytes) {
+    bulk_g2s(dst, src, bytes1, bar);
+    bulk_g2s(dst + bytes1, src + bytes1 + gap, bytes - bytes1, bar);
+  } else {
+    bulk_g2s(dst, src, bytes, bar);
+  }
+}
 
 // A consumer warp's part of a value-only use (QK heredity): area A (and B when vonly == 2) of the slot holds
 // the value rows of a lazy layer; the probabilities were left in `prob` by the item's own use (another group's
@@ -167,14 +180,16 @@ __device__ __noinline__ bool consume_values(const unsigned char* areaA, const un
 
 // The manager's part of a value-only use: the value rows of the item's chunk (`c`) in lazy layers f0 .. f0+n-1
 // (n = 1 or 2) go to tile areas A and B of the slot.  Out of line for the same reason.
-template <typename T, int D>
+template <typename T, int D, bool PRE>
 __device__ __noinline__ void issue_values(const StepParams& p, const Chain* chain, ItemDesc* desc, unsigned char* areaA,
                                           unsigned char* areaB, uint64_t* barA, uint64_t* barB, int f0, int n, int lane,
                                           volatile int* abort_flag) {
   constexpr int ROWB = D * (int)sizeof(T), VPR = ROWB / 16, LN = VPR <= 16 ? VPR : 16, NV = VPR / LN;
   const Chain c = *chain;
   const int H = p.H;
-  const size_t layer_bytes = (size_t)p.B * H * (size_t)p.lbh_stride * sizeof(T);  // one layer of cache blocks
+  // one layer of cache blocks, or of the prompt's tensor
+  const size_t layer_bytes = (size_t)p.B * H * (PRE ? (size_t)p.t0_max * D : (size_t)p.lbh_stride) * sizeof(T);
+  const size_t gap = PRE ? (size_t)p.Nv * ROWB : 0;
   if (c.is_vis) {  // rows the previous step's selection may still be moving
     for (int j = 0; j < n; ++j)
       if (p.req[c.l_rel + f0 + j] &&
@@ -199,17 +214,18 @@ __device__ __noinline__ void issue_values(const StepParams& p, const Chain* chai
   if (lane == 0) {
     desc->info = pack_info(c.nrows, 0, n, 0);
     const uint32_t kb = (uint32_t)(c.nrows - (c.has_new ? 1 : 0)) * ROWB;
+    const uint32_t kb1 = PRE ? (uint32_t)c.nrows1 * ROWB : kb;
     if (n == 2) {
       if (kb) {
         mbar_expect_tx(barB, kb);
-        bulk_g2s(areaB, c.srcV + (f0 + 1) * layer_bytes, kb, barB);
+        rows_g2s(areaB, c.srcV + (f0 + 1) * layer_bytes, kb, kb1, gap, barB);
       } else {
         mbar_arrive(barB);
       }
     }
     if (kb) {
       mbar_expect_tx(barA, kb);
-      bulk_g2s(areaA, c.srcV + f0 * layer_bytes, kb, barA);
+      rows_g2s(areaA, c.srcV + f0 * layer_bytes, kb, kb1, gap, barA);
     } else {
       mbar_arrive(barA);
     }
@@ -218,7 +234,11 @@ __device__ __noinline__ void issue_values(const StepParams& p, const Chain* chai
 
 // FAT: the launch has items that carry lazy layers.  The host picks the plain instantiation when no layer of
 // the call is lazy, so that path pays nothing (registers, code size) for the other.
-template <typename T, int D, bool FAT>
+// PRE: the rows come from the prompt's own tensors ([layer][sequence][head][S | V | I]) and not from the cache; nothing
+// is appended.  Attending in place and copying only the kept rows afterwards (st3_gather_kernel) replaced a copy of
+// every row into the cache ahead of this launch, a second read of all of them here and moves inside the cache: a
+// prompt row that is not kept now crosses the memory bus once instead of three times.
+template <typename T, int D, bool FAT, bool PRE>
 __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __grid_constant__ StepParams p) {
   constexpr int EPL = 16 / sizeof(T);      // elements per 16-byte chunk
   constexpr int ROWB = D * sizeof(T);      // bytes per row
@@ -285,6 +305,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       int slot;          // index of the item's partial: item * H + h
       int oidx, lb;      // (relative layer, sequence, head) and (layer, sequence) indices
       const unsigned char *srcK, *srcV;  // first key / value row of the chunk
+      int nrows1;        // PRE: rows up to the break in the prompt tensors
       const T* srcQ;
       long long glog;  // offset into p.logits of this chunk's first row
       uint4 nv[NV];  // the newest row (key lanes and value lanes), fetched ahead of the slot becoming free
@@ -300,6 +321,9 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
     auto oidx_of = [&](int lr, int b, int h) { return ((long long)lr * p.B + b) * H + h; };
     // first key (kv = 0) or value (kv = 1) row of the region an item of relative layer lr reads
     auto region_of = [&](int lr, int b, int h, bool is_vis, int kv) {
+      if constexpr (PRE)
+        return const_cast<T*>(reinterpret_cast<const T*>(kv ? p.v_in : p.k_in)) +
+               (oidx_of(lr, b, h) * p.t0_max + (is_vis ? p.sys_len : 0)) * D;
       T* blk = reinterpret_cast<T*>(p.cache) + lbh_of(lr, b, h) * p.lbh_stride;
       if (is_vis) return blk + (long long)kv * p.Nv * D;
       return blk + 2LL * p.Nv * D + (long long)kv * p.cap_txt * D;
@@ -367,8 +391,14 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       const int lk = ls < 0 ? l_rel : ls;  // whose keys and query
       d.lazy = ls >= 0;
       d.wait_for_k = is_vis && ls >= 0 ? p.req[ls] : 0;  // the source's rows as well
-      d.srcK = reinterpret_cast<const unsigned char*>(region_of(lk, b, h, is_vis, 0)) + (size_t)r0 * ROWB;
-      d.srcV = reinterpret_cast<const unsigned char*>(region_of(l_rel, b, h, is_vis, 1)) + (size_t)r0 * ROWB;
+      int row0 = r0;  // the chunk's first row in its source
+      if constexpr (PRE) {
+        const bool whole = is_vis || r0 >= p.sys_len || r0 + nrows <= p.sys_len;  // all of it on one side of the break
+        d.nrows1 = whole ? nrows : p.sys_len - r0;
+        if (!is_vis && r0 >= p.sys_len) row0 += p.Nv;
+      }
+      d.srcK = reinterpret_cast<const unsigned char*>(region_of(lk, b, h, is_vis, 0)) + (size_t)row0 * ROWB;
+      d.srcV = reinterpret_cast<const unsigned char*>(region_of(l_rel, b, h, is_vis, 1)) + (size_t)row0 * ROWB;
       d.srcQ = reinterpret_cast<const T*>(p.q) + oidx_of(lk, b, h) * D;
       d.glog = lbh_of(l_rel, b, h) * p.Nv + r0;
       if (d.has_new && lane < 2 * LN) {
@@ -409,18 +439,21 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
             Chain& c = s_chain[s];
             c.srcV = d.srcV; c.oidx = d.oidx; c.lb = d.lb; c.l_rel = d.l_rel; c.nrows = d.nrows;
             c.has_new = d.has_new; c.is_vis = d.is_vis;
+            if constexpr (PRE) c.nrows1 = d.nrows1;
           }
         }
         ItemDesc& sd = s_desc[s];
         sd.info = pack_info(d.nrows, d.nfol, 0, d.want_logits);
         sd.glog = d.glog;
         const uint32_t kb = (uint32_t)(d.nrows - (d.has_new ? 1 : 0)) * ROWB;
+        const uint32_t kb1 = PRE ? (uint32_t)d.nrows1 * ROWB : kb;
+        const size_t gap = PRE ? (size_t)p.Nv * ROWB : 0;
         mbar_expect_tx(&s_fullK[s][g], kb + ROWB);  // K rows + the query (D elements = ROWB bytes)
         bulk_g2s(sQ, d.srcQ, ROWB, &s_fullK[s][g]);
         if (kb) {
-          bulk_g2s(sK, d.srcK, kb, &s_fullK[s][g]);
+          rows_g2s(sK, d.srcK, kb, kb1, gap, &s_fullK[s][g]);
           mbar_expect_tx(&s_fullV[s][g], kb);
-          bulk_g2s(sV, d.srcV, kb, &s_fullV[s][g]);
+          rows_g2s(sV, d.srcV, kb, kb1, gap, &s_fullV[s][g]);
         } else {
           mbar_arrive(&s_fullV[s][g]);
         }
@@ -484,7 +517,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
         if constexpr (FAT) {
           const int gn = (use + 1 + s) % kGroups;
           __syncwarp();
-          issue_values<T, D>(p, &s_chain[s], &s_desc[s], sK, sV, &s_fullK[s][gn], &s_fullV[s][gn], fnext, nn, lane,
+          issue_values<T, D, PRE>(p, &s_chain[s], &s_desc[s], sK, sV, &s_fullK[s][gn], &s_fullV[s][gn], fnext, nn, lane,
                              abort_flag);
         }
         f0 = fnext; fn = nn;

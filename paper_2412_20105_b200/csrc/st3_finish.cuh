@@ -124,8 +124,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
   const int k = min(n_host, p.ntgt[l_rel]);
   const bool evicts = k < n_host;  // same answer in every thread
   const int n_dev = p.n_cur[lb];
+  const bool fresh = p.fresh;  // a new prompt: row i is visual token i, whatever the bookkeeping says
   if (!evicts) {
-    if (tt == 0) {
+    if (fresh) {
+      for (int i = tt; i < n_host; i += kFinishThreads) { p.ids[lb * Nv + i] = i; p.mass_by_id[lb * Nv + i] = 0.f; }
+      if (tt == 0) p.n_cur[lb] = n_host;
+    } else if (tt == 0) {
       if (n_dev != p.nold[l_rel]) atomicOr(p.status, ST3_DEV_COUNT_MISMATCH);
       else if (n_host != n_dev) p.n_cur[lb] = n_host;  // static-rank cut: only the count changes
     }
@@ -154,7 +158,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
   const bool own_scores = p.ext_scores == nullptr;
   if (own_scores) {
     if (ri < n_cur) {
-      if (hg == 0) id0 = ids[ri];
+      if (hg == 0) id0 = fresh ? ri : ids[ri];
 #pragma unroll
       for (int j = 0; j < kHeadBatch; ++j) {
         const int h = hg * kHeadBatch + j;
@@ -181,7 +185,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
     }
   }
   __syncthreads();
-  if (n_dev != n_host) {  // host bookkeeping and device state disagree: flag, do not touch
+  if (!fresh && n_dev != n_host) {  // host bookkeeping and device state disagree: flag, do not touch
     if (tt == 0) atomicOr(p.status, ST3_DEV_COUNT_MISMATCH);
     done();
     return;
@@ -193,7 +197,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
     // scores supplied by the caller (any finite float): order-preserving map of the bits to unsigned
     const float* ext = p.ext_scores + ((long long)l_rel * B + b) * Nv;
     for (int i = tt; i < n_cur; i += kFinishThreads) {
-      const int id = ids[i];
+      const int id = fresh ? i : ids[i];
       float sc = ext[id];
       if (!(fabsf(sc) <= 3.0e38f)) { bad = true; sc = -3.0e38f; }
       mass_by_id[id] = sc;
@@ -208,7 +212,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
     float pm = 0.f;
     int id = id0;
     if (i < n_cur) {
-      if (i0 && hg == 0) id = ids[i];
+      if (i0 && hg == 0) id = fresh ? i : ids[i];
       for (int h0 = hg * kHeadBatch; h0 < H; h0 += 2 * kHeadBatch) {
         float v[kHeadBatch];
         if (i0 == 0 && h0 == hg * kHeadBatch) {
@@ -277,34 +281,16 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
     prefix = ~0ull;  // keep nothing (ids are < 2^31, so no key reaches this value)
   }
 
-  if (p.static_rank) {
-    // ---- top-index order: the kept row with r larger keys goes to position r, copied from the
-    // caller's prompt tensors (the cache rows are only written, so nothing is read after being moved)
-    for (int i = tt; i < n_cur; i += kFinishThreads) s_mover[i] = ids[i];
+  if (fresh && p.static_rank) {
+    // ---- top-index order: the kept token with r larger keys comes r-th.  st3_gather_kernel copies the rows.
     for (int i = tt; i < n_cur; i += kFinishThreads) {
       const unsigned long long key = s_key[i];
       if (key >= prefix) {
         int r = 0;
         for (int j = 0; j < n_cur; ++j) r += s_key[j] > key;
-        s_hole[r] = i;
+        ids[r] = i;
       }
     }
-    __syncthreads();
-    unsigned char* blk0 = reinterpret_cast<unsigned char*>(p.cache) + (size_t)(lb * H) * p.lbh_stride * sizeof(T);
-    const long long nvec = (long long)k * H * 2 * VPR;
-    for (long long v = tt; v < nvec; v += kFinishThreads) {
-      const int c = (int)(v % VPR);
-      long long r = v / VPR;
-      const int kv = (int)(r % 2); r /= 2;
-      const int h = (int)(r % H);
-      const int j = (int)(r / H);
-      const unsigned char* src = reinterpret_cast<const unsigned char*>(kv ? p.v_in : p.k_in) +
-                                 ((((size_t)l_rel * B + b) * H + h) * p.t0_max + p.sys_len + s_mover[s_hole[j]]) * ROWB;
-      unsigned char* dst = blk0 + (size_t)h * p.lbh_stride * sizeof(T) + (size_t)kv * Nv * ROWB + (size_t)j * ROWB;
-      *reinterpret_cast<uint4*>(dst + c * 16) = *reinterpret_cast<const uint4*>(src + c * 16);
-    }
-    __syncthreads();  // every thread has read the old ids it needs
-    for (int j = tt; j < k; j += kFinishThreads) ids[j] = s_mover[s_hole[j]];
     if (tt == 0) p.n_cur[lb] = k;
     done();
     return;
@@ -316,8 +302,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
   int nh = 0, nm = 0;
   for (int i = i0; i < i1; ++i) {
     const bool keep = s_key[i] >= prefix;
-    nh += (i < k && !keep);
-    nm += (i >= k && keep);
+    nh += fresh ? keep : (i < k && !keep);
+    nm += !fresh && i >= k && keep;
   }
   const int packed = nh | (nm << 16);
   int incl = packed;
@@ -336,6 +322,16 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
   }
   const int excl = woff + incl - packed;
   int ph = excl & 0xffff, pm = excl >> 16;
+  if (fresh) {  // the kept tokens in the prompt's order; st3_gather_kernel copies the rows
+    for (int i = i0; i < i1; ++i)
+      if (s_key[i] >= prefix) ids[ph++] = i;
+    if (tt == 0) {
+      p.n_cur[lb] = k;
+      if ((total & 0xffff) != k) atomicOr(p.status, ST3_DEV_RANGE);  // cannot happen: exactly k keys pass the threshold
+    }
+    done();
+    return;
+  }
   for (int i = i0; i < i1; ++i) {
     const bool keep = s_key[i] >= prefix;
     if (i < k && !keep) s_hole[ph++] = i;
@@ -370,48 +366,56 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
 }
 
 // ------------------------------------------------------------------------------------------
-// Prompt ingest: rows [S | V | I] of the caller's tensors -> cache regions
+// Prompt rows -> cache regions: [S | I] to the text region, the kept visual rows (ids) to the visual region
 // ------------------------------------------------------------------------------------------
+// Runs after the selection and copies what it kept, spread over the whole GPU: bound by memory bandwidth for a batch,
+// by one round trip for ids and one for the rows for a single layer.  The selection blocks used to move the kept rows
+// inside the cache, one block per (layer, sequence): 105-118 us for 32 heads and 576 visual tokens, 515 us for 2880.
+// st3_prefill_select of one 7B layer, one sequence: 105 -> 28 us; 32 layers in one call: 298 -> 137 us; a 13B layer of
+// 16 sequences: 269 -> 104 us; three NeXT layers of 8 sequences that prune: 1099 -> 415 us, that keep all: 589 -> 577 us.
+constexpr int kGatherBlocks = 16;  // per (layer, sequence, head); 4, 8, 16 and 32 blocks and 1, 2 or 4 vectors in flight
+                                   // per thread are within 3 % of one another on a batch, 16 or more best for one layer
+
 template <typename T, int D>
-__global__ void __launch_bounds__(kThreads) st3_ingest_kernel(const StepParams p, const T* __restrict__ k,
-                                                              const T* __restrict__ v, int t0_max) {
+__global__ void __launch_bounds__(kThreads) st3_gather_kernel(const __grid_constant__ StepParams p) {
   constexpr int VPR = D * sizeof(T) / 16;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int H = p.H, B = p.B, Nv = p.Nv;
   int y = blockIdx.y;
   const int h = y % H; y /= H;
   const int b = y % B;
   const int l_rel = y / B;
-  const int l = p.layer_begin + l_rel;
-  const int text = __ldg(p.text_len + b);
-  const int t0 = p.sys_len + Nv + text;
-  const long long lbh_in = ((long long)l_rel * B + b) * H + h;
-  const long long lbh = ((long long)l * B + b) * H + h;
-  const uint4* srcK = reinterpret_cast<const uint4*>(k + lbh_in * t0_max * D);
-  const uint4* srcV = reinterpret_cast<const uint4*>(v + lbh_in * t0_max * D);
-  T* blk = reinterpret_cast<T*>(p.cache) + lbh * p.lbh_stride;
-  uint4* dKv = reinterpret_cast<uint4*>(blk);
-  uint4* dVv = reinterpret_cast<uint4*>(blk + (long long)Nv * D);
-  uint4* dKt = reinterpret_cast<uint4*>(blk + 2LL * Nv * D);
-  uint4* dVt = reinterpret_cast<uint4*>(blk + 2LL * Nv * D + (long long)p.cap_txt * D);
-  const int total = t0 * VPR;
-  for (int i = blockIdx.x * kThreads + threadIdx.x; i < total; i += gridDim.x * kThreads) {
+  const long long lb = (long long)(p.layer_begin + l_rel) * B + b;
+  const int n_txt = p.sys_len + __ldg(p.text_len + b);
+  const int n_vis = p.ntgt[l_rel];
+  const bool all = n_vis == Nv;
+  const int* ids = p.ids + lb * Nv;
+  const long long in0 = (((long long)l_rel * B + b) * H + h) * p.t0_max * VPR;
+  const uint4* srcK = reinterpret_cast<const uint4*>(p.k_in) + in0;
+  const uint4* srcV = reinterpret_cast<const uint4*>(p.v_in) + in0;
+  uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<T*>(p.cache) + (lb * H + h) * p.lbh_stride);
+  const int total = (n_vis + n_txt) * VPR;
+  for (int i = blockIdx.x * kThreads + threadIdx.x; i < total; i += kGatherBlocks * kThreads) {
     const int row = i / VPR, c = i % VPR;
-    const uint4 kk = __ldg(srcK + i), vv = __ldg(srcV + i);
-    if (row >= p.sys_len && row < p.sys_len + Nv) {
-      const int d = (row - p.sys_len) * VPR + c;
-      dKv[d] = kk; dVv[d] = vv;
+    const bool vis = row < n_vis;
+    int src;  // row of the prompt
+    if (vis) {
+      const int id = all ? row : ids[row];
+      if ((unsigned)id >= (unsigned)Nv) {  // a selection that failed: reported, not used
+        atomicOr(p.status, ST3_DEV_RANGE);
+        continue;
+      }
+      src = p.sys_len + id;
     } else {
-      const int d = (row < p.sys_len ? row : row - Nv) * VPR + c;
-      dKt[d] = kk; dVt[d] = vv;
+      src = row - n_vis < p.sys_len ? row - n_vis : row - n_vis + Nv;
     }
-  }
-  if (h == 0 && blockIdx.x == 0) {
-    const long long lb = (long long)l * B + b;
-    for (int i = threadIdx.x; i < Nv; i += kThreads) { p.ids[lb * Nv + i] = i; p.mass_by_id[lb * Nv + i] = 0.f; }
-    if (threadIdx.x == 0) p.n_cur[lb] = Nv;
+    const uint4 kk = __ldg(srcK + src * VPR + c), vv = __ldg(srcV + src * VPR + c);
+    // K_vis | V_vis | K_txt | V_txt
+    const long long d = vis ? i : 2LL * Nv * VPR + (i - n_vis * VPR);
+    dst[d] = kk;
+    dst[d + (long long)(vis ? Nv : p.cap_txt) * VPR] = vv;
   }
 }
-
 
 }  // namespace
 
