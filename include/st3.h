@@ -174,8 +174,9 @@ st3_status st3_decode_step(st3_ctx* ctx, int32_t step, int32_t layer_begin, int3
  * sequence) flags order the rest.  The price is a promise by the caller: q, k_new and v_new of a step are
  * complete in device memory BEFORE the launch ahead of st3_decode_step in the stream begins; in particular
  * the kernel that produces them must not signal programmatic completion (griddepcontrol.launch_dependents,
- * cudaTriggerProgrammaticLaunchCompletion) before its last write to them.  Off by default: every kernel of
- * a call then starts only after all earlier work of the stream has finished. */
+ * cudaTriggerProgrammaticLaunchCompletion) before its last write to them.  Off by default: a kernel of a call
+ * may then be set up, and read rows that the library itself cached, while the launch ahead of it ends, but it
+ * reads no input before all earlier work of the stream has finished. */
 st3_status st3_set_overlap(st3_ctx* ctx, int32_t on);
 
 /* Same step with HOST buffers (pinned memory, else the copies do not overlap anything): the library copies

@@ -47,6 +47,10 @@ __device__ __forceinline__ int pack_info(int nrows, int nfol, int vonly, int wan
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// announces bytes of a phase that another arrival completes
+__device__ __forceinline__ void mbar_expect_more(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ unsigned fast_div(unsigned n, unsigned mul, unsigned shift) {
   return (__umulhi(n, mul) + n) >> shift;  // exact for n < 2^31 (host: make_fast_div)
 }
@@ -310,6 +314,14 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       long long glog;  // offset into p.logits of this chunk's first row
       uint4 nv[NV];  // the newest row (key lanes and value lanes), fetched ahead of the slot becoming free
     };
+    // Whether the step's inputs may be read.  In plain stream order this launch may have been started before the launch
+    // ahead of it ended (p.order): each manager first requests its item's cached rows, which only launches of this
+    // library write (flags order the visual ones), and waits before it touches an input.
+    bool inputs_ready = p.order == 0;
+    if constexpr (PRE) {  // the prompt's rows are inputs too
+      if (!inputs_ready) asm volatile("griddepcontrol.wait;" ::: "memory");
+      inputs_ready = true;
+    }
     int wcur = 0;  // working layer of the previous visual item: this warp's items arrive in increasing order
     int lb_ready = -1;  // the (l, b) whose visual rows were last seen released by the previous finish launch
     // the first item of every manager is fixed (no round trip to the counter before the first copy);
@@ -329,6 +341,15 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       return blk + 2LL * p.Nv * D + (long long)kv * p.cap_txt * D;
     };
 
+    auto fetch_new = [&](Dec& d) {  // newest row, key and value lanes: from the step's inputs; stored when the slot is free
+      if (d.has_new && lane < 2 * LN) {
+        const int ls = p.lazy_src[d.l_rel];
+        const T* src = lane / LN ? reinterpret_cast<const T*>(p.v_new) + (long long)d.oidx * D
+                                 : reinterpret_cast<const T*>(p.k_new) + (long long)(d.oidx + (ls < 0 ? 0 : ls - d.l_rel) * p.B * H) * D;
+#pragma unroll
+        for (int i = 0; i < NV; ++i) d.nv[i] = __ldg(reinterpret_cast<const uint4*>(src) + (lane % LN) + i * LN);
+      }
+    };
     auto decode = [&](Dec& d) {
       const int x = __shfl_sync(0xffffffffu, x_next, 0);
       d.valid = (unsigned)x < (unsigned)total;
@@ -401,16 +422,10 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       d.srcV = reinterpret_cast<const unsigned char*>(region_of(l_rel, b, h, is_vis, 1)) + (size_t)row0 * ROWB;
       d.srcQ = reinterpret_cast<const T*>(p.q) + oidx_of(lk, b, h) * D;
       d.glog = lbh_of(l_rel, b, h) * p.Nv + r0;
-      if (d.has_new && lane < 2 * LN) {
-        // newest row: fetched from the step's inputs now, stored when the slot is free
-        const T* src = lane / LN ? reinterpret_cast<const T*>(p.v_new) + oidx_of(l_rel, b, h) * D
-                                 : reinterpret_cast<const T*>(p.k_new) + oidx_of(ls < 0 ? l_rel : ls, b, h) * D;
-#pragma unroll
-        for (int i = 0; i < NV; ++i) d.nv[i] = __ldg(reinterpret_cast<const uint4*>(src) + (lane % LN) + i * LN);
-      }
+      if (inputs_ready) fetch_new(d);
     };
     // Starts the copies of a decoded item into this (free) slot.
-    auto issue = [&](const Dec& d, int g) {  // g: the consumer group this use of the slot belongs to
+    auto issue = [&](Dec& d, int g) {  // g: the consumer group this use of the slot belongs to
       if (d.wait_for) {
         if (!flag_wait(p.flags + d.lb, d.wait_for, abort_flag, p.status)) return;
         lb_ready = d.lb;
@@ -418,6 +433,22 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       if (d.wait_for_k &&  // the source layer's (l, b): the same sequence, lazy_src layers lower
           !flag_wait(p.flags + d.lb + (p.lazy_src[d.l_rel] - d.l_rel) * p.B, d.wait_for_k, abort_flag, p.status))
         return;
+      const uint32_t kb = (uint32_t)(d.nrows - (d.has_new ? 1 : 0)) * ROWB;
+      const uint32_t kb1 = PRE ? (uint32_t)d.nrows1 * ROWB : kb;
+      const size_t gap = PRE ? (size_t)p.Nv * ROWB : 0;
+      const bool ahead = !inputs_ready;  // the rows go ahead of the inputs
+      if (ahead) {
+        if (lane == 0 && kb) {
+          mbar_expect_more(&s_fullK[s][g], kb);
+          bulk_g2s(sK, d.srcK, kb, &s_fullK[s][g]);
+          mbar_expect_more(&s_fullV[s][g], kb);
+          bulk_g2s(sV, d.srcV, kb, &s_fullV[s][g]);
+        }
+        __syncwarp();
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        inputs_ready = true;
+        fetch_new(d);
+      }
       if (d.has_new) {
         if (lane < 2 * LN) {
           const int kv = lane / LN;
@@ -445,17 +476,14 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
         ItemDesc& sd = s_desc[s];
         sd.info = pack_info(d.nrows, d.nfol, 0, d.want_logits);
         sd.glog = d.glog;
-        const uint32_t kb = (uint32_t)(d.nrows - (d.has_new ? 1 : 0)) * ROWB;
-        const uint32_t kb1 = PRE ? (uint32_t)d.nrows1 * ROWB : kb;
-        const size_t gap = PRE ? (size_t)p.Nv * ROWB : 0;
-        mbar_expect_tx(&s_fullK[s][g], kb + ROWB);  // K rows + the query (D elements = ROWB bytes)
+        mbar_expect_tx(&s_fullK[s][g], ahead ? ROWB : kb + ROWB);  // K rows + the query (D elements = ROWB bytes)
         bulk_g2s(sQ, d.srcQ, ROWB, &s_fullK[s][g]);
-        if (kb) {
+        if (ahead || !kb) {
+          mbar_arrive(&s_fullV[s][g]);
+        } else {
           rows_g2s(sK, d.srcK, kb, kb1, gap, &s_fullK[s][g]);
           mbar_expect_tx(&s_fullV[s][g], kb);
           rows_g2s(sV, d.srcV, kb, kb1, gap, &s_fullV[s][g]);
-        } else {
-          mbar_arrive(&s_fullV[s][g]);
         }
       }
     };
@@ -683,7 +711,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       if (lane == 0) mbar_arrive(&s_done[s][grp]);
     }
   }
-  // This grid started without waiting for the launch before it (flags order what they share).  It must not
+  // This grid may have started without waiting for the launch before it (flags order what they share).  It must not
   // *complete* before that launch has, though: the finish launch after this one waits for this grid only.
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }

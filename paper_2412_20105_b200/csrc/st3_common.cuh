@@ -61,6 +61,7 @@ struct StepParams {
   int ncur[kMaxLayers];     // visual rows held before this step (host's schedule bookkeeping)
   int ntgt[kMaxLayers];     // visual rows to hold after this step
   int nold[kMaxLayers];     // visual rows the device should report before this step
+  int order;                // 1: the launch may start before the launch ahead of it ends, and waits before it reads inputs
   int fresh;                // 1: a new prompt, whose visual rows are the tokens 0 .. Nv-1 (ids are not read)
   const void* k_in;         // prefill only: the caller's prompt tensors [layer_count][B][H][t0_max][D]
   const void* v_in;

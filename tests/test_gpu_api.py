@@ -353,3 +353,46 @@ def test_a_new_generation_starts_at_layer_zero():
         assert run.ctx.status() == 0
     finally:
         run.close()
+
+
+@pytest.mark.parametrize("captured", [False, True])
+def test_layer_calls_behind_a_copy_and_an_early_producer(captured):
+    """Plain stream order, a call per layer: each layer's inputs are written by a kernel that allows its dependents to
+    launch 20 us before it writes, the next layer's by a copy.  `captured`: the calls of a step are captured in a
+    graph, which is launched once."""
+    import native
+    lib = native.load()
+    wl = _small(num_layers=4)
+    a, b = GpuRun(wl), GpuRun(wl)
+    try:
+        a.prefill(); b.prefill()
+        for t in range(1, 4):
+            a.decode(t)
+            q, kn, vn = b.inputs(t)
+            src = torch.stack([q, kn, vn], dim=1).contiguous()       # [layer][q | k | v]
+            dst = torch.zeros_like(src)
+            torch.cuda.synchronize()
+
+            def step():
+                st = torch.cuda.current_stream().cuda_stream
+                for l in range(wl.num_layers):
+                    if l % 2:
+                        dst[l].copy_(src[l])
+                    else:
+                        n16 = src[l].numel() * src.element_size() // 16
+                        assert lib.st3_test_early_trigger_copy(dst[l].data_ptr(), src[l].data_ptr(), n16, 20, st) == 0
+                    b.ctx.decode_step(t, dst[l, 0:1], dst[l, 1:2], dst[l, 2:3], b.out[l:l + 1], layer_begin=l)
+
+            if captured:
+                graph = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(graph):
+                    step()
+                graph.replay()
+            else:
+                step()
+            torch.cuda.synchronize()
+            assert torch.equal(a.out, b.out), t
+            b.check_rows_unit(0, 1, 0, t)
+        assert a.ctx.status() == 0 and b.ctx.status() == 0
+    finally:
+        a.close(); b.close()
