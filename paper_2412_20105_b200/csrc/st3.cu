@@ -24,6 +24,7 @@
 // This file holds the host logic and the C ABI.
 #include "st3.h"
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -854,15 +855,18 @@ st3_status st3_destroy(st3_ctx* ctx) {
 }  // extern "C"
 
 // ------------------------------------------------------------------------------------------
-// st3_attend_noalloc: one-shot attention whose split partials live in a static device array
+// st3_attend_noalloc: one-shot attention without a workspace
 // ------------------------------------------------------------------------------------------
 // Some callers cannot hand this library a workspace: code that runs where cudaMalloc is off
 // limits (inside a framework's allocator-owned region, in a plugin that was given only its
 // input and output tensors, late in a process whose memory is fully committed).  For them the
-// chunk partials of the attention go into the fixed array below instead of caller memory.
+// partials of the attention stay in shared memory, or, for a few heads of very many rows, go
+// into the fixed array below instead of caller memory.
 // The array is part of the loaded module: every GPU that loads the library holds these bytes
 // until the process exits, which is why the limit is kept small.
 constexpr int kNaChunkRows = 128;
+constexpr int kNaMaxCluster = 8;  // blocks that share a head in the one-launch form (the portable limit)
+constexpr int kNaLongRows = 8192;  // rows above which a few heads take the two-launch form
 constexpr int kNaMaxSlots = 8192;  // heads x row chunks of one call
 constexpr size_t kNaScratchBytes = (size_t)kNaMaxSlots * (2 + 128) * sizeof(float);  // 4 259 840 bytes
 static __device__ __align__(256) unsigned char st3_static_scratch[kNaScratchBytes];
@@ -975,6 +979,140 @@ __global__ void st3_na_merge_kernel(T* __restrict__ out, int nchunk, const float
   store_out(out + (long long)h * D + d, o / L);
 }
 
+// One launch and no scratch: a cluster of blocks shares a head, every warp streams its own rows (K and V of
+// kNaBatch groups in flight at once, softmax relative to the warp's running maximum), the warps' results meet in
+// shared memory and the blocks' results in that of the cluster's first block.
+// One latency for the loads and one cluster barrier bound it at 7B size (32 x 675 rows).
+constexpr int kNaBatch = 8;
+template <typename T, int D>
+__global__ void __launch_bounds__(kThreads, 2) st3_na_cluster_kernel(const T* __restrict__ q, const T* __restrict__ K,
+                                                                     const T* __restrict__ V, T* __restrict__ out,
+                                                                     int num_rows) {
+  constexpr int EPL = 16 / sizeof(T), LPR = D / EPL, RPW = 32 / LPR;
+  __shared__ float s_m[kWarps], s_l[kWarps];
+  __shared__ float s_acc[kWarps][D];
+  __shared__ float s_blk[2 + D];  // this block's (maximum, sum, un-normalised output)
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  // may have been set up while the launch ahead was still running
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nblk = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), h = blockIdx.y;
+  const int per = (num_rows + nblk - 1) / nblk;
+  const int r0 = min(num_rows, rank * per), r1 = min(num_rows, r0 + per);
+  const int sub = lane / LPR, lir = lane % LPR;
+  const uint4* gK = reinterpret_cast<const uint4*>(K + (long long)h * num_rows * D) + lir;
+  const uint4* gV = reinterpret_cast<const uint4*>(V + (long long)h * num_rows * D) + lir;
+  float qf[EPL];
+  unpack16(__ldg(reinterpret_cast<const uint4*>(q + (long long)h * D) + lir), qf);
+  const float sc = 1.4426950408889634f * rsqrtf((float)D);
+#pragma unroll
+  for (int e = 0; e < EPL; ++e) qf[e] *= sc;
+  float m = -INFINITY, l = 0.f, acc[EPL];
+#pragma unroll
+  for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
+  for (int rb = r0 + warp * RPW; rb < r1; rb += kNaBatch * kWarps * RPW) {  // the same trips for the whole warp
+    uint4 kk[kNaBatch], vv[kNaBatch];
+#pragma unroll
+    for (int u = 0; u < kNaBatch; ++u) {
+      const int r = rb + u * kWarps * RPW + sub;
+      if (r < r1) { kk[u] = __ldg(gK + (long long)r * LPR); vv[u] = __ldg(gV + (long long)r * LPR); }
+    }
+    float s[kNaBatch], mx = m;
+#pragma unroll
+    for (int u = 0; u < kNaBatch; ++u) {
+      float kf[EPL], a = 0.f;
+      unpack16(kk[u], kf);
+#pragma unroll
+      for (int e = 0; e < EPL; ++e) a = fmaf(qf[e], kf[e], a);
+#pragma unroll
+      for (int o = LPR / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      s[u] = rb + u * kWarps * RPW + sub < r1 ? a : -INFINITY;
+      mx = fmaxf(mx, s[u]);
+    }
+    const float ref = mx > -INFINITY ? mx : 0.f;  // lanes without a row yet keep zeros
+    const float f = fast_exp2(m - ref);
+    m = mx;
+    float lb = 0.f, ab[EPL];  // the batch's own sums: short chains of additions
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) ab[e] = 0.f;
+#pragma unroll
+    for (int u = 0; u < kNaBatch; ++u) {
+      if (rb + u * kWarps * RPW + sub < r1) {
+        const float pr = fast_exp2(s[u] - ref);
+        float vf[EPL];
+        unpack16(vv[u], vf);
+        lb += pr;
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) ab[e] = fmaf(pr, vf[e], ab[e]);
+      }
+    }
+    l = fmaf(l, f, lb);
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) acc[e] = fmaf(acc[e], f, ab[e]);
+  }
+  // the RPW row groups of the warp, then the warps, then the blocks of the cluster
+#pragma unroll
+  for (int o = LPR; o < 32; o <<= 1) {
+    const float mo = __shfl_xor_sync(0xffffffffu, m, o);
+    const float mx = fmaxf(m, mo), ref = mx > -INFINITY ? mx : 0.f;
+    const float f = fast_exp2(m - ref);
+    m = mx;
+    l *= f;
+    l += __shfl_xor_sync(0xffffffffu, l, o);
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) {
+      acc[e] *= f;
+      acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
+    }
+  }
+  if (lane == 0) { s_m[warp] = m; s_l[warp] = l; }
+  if (lane < LPR) {
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) s_acc[warp][lir * EPL + e] = acc[e];
+  }
+  __syncthreads();
+  if (tid < D) {
+    float M = s_m[0];
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) M = fmaxf(M, s_m[w]);
+    const float ref = M > -INFINITY ? M : 0.f;  // a block without rows
+    float L = 0.f, o = 0.f;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      const float f = fast_exp2(s_m[w] - ref);
+      L = fmaf(s_l[w], f, L);
+      o = fmaf(s_acc[w][tid], f, o);
+    }
+    s_blk[2 + tid] = o;
+    if (tid == 0) { s_blk[0] = M; s_blk[1] = L; }
+  }
+  cluster.sync();
+  if (rank == 0 && tid < D) {
+    float mb[kNaMaxCluster], lb[kNaMaxCluster], ob[kNaMaxCluster], M = -INFINITY;
+#pragma unroll
+    for (int c = 0; c < kNaMaxCluster; ++c) {
+      mb[c] = -INFINITY; lb[c] = ob[c] = 0.f;
+      if (c < nblk) {
+        const float* r = cluster.map_shared_rank(s_blk, c);
+        mb[c] = r[0]; lb[c] = r[1]; ob[c] = r[2 + tid];
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < kNaMaxCluster; ++c) M = fmaxf(M, mb[c]);
+    float L = 0.f, o = 0.f;
+#pragma unroll
+    for (int c = 0; c < kNaMaxCluster; ++c) {
+      const float f = fast_exp2(mb[c] - M);
+      L = fmaf(lb[c], f, L);
+      o = fmaf(ob[c], f, o);
+    }
+    store_out(out + (long long)h * D + tid, o / L);
+  }
+  cluster.sync();  // the other blocks' shared memory stays until it has been read
+}
+
 // Device address of st3_static_scratch, looked up once per device.  In host code the array's
 // name is only a handle for the runtime, never an address a kernel may be given.
 constexpr int kNaMaxDevices = 64;
@@ -995,6 +1133,25 @@ st3_status na_scratch(float** ml, float** acc) {
 
 template <typename T, int D>
 st3_status na_launch(const void* q, const void* k, const void* v, void* out, int H, int rows, cudaStream_t st) {
+  // The one-launch form, unless a few heads of very many rows would leave most of the GPU idle: eight blocks a head keep
+  // 16 heads on 128 SMs.  GPU time a call, two launches against one: 32 x 675 rows (bf16, D = 128) 17.2 / 5.6 us,
+  // 40 x 1500 18.5 / 14.9, 4 x 8000 21.3 / 16.8, 64 x 8000 67.8 / 46.8; 1 x 100000 74.6 / 161.6.
+  if (rows <= kNaLongRows || H >= 16) {
+    const int nblk = rows >= kNaMaxCluster * 64 ? kNaMaxCluster : ceil_div(rows, 64);  // 32 to 128 rows: no difference
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nblk, (unsigned)H);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)nblk; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, st3_na_cluster_kernel<T, D>, static_cast<const T*>(q), static_cast<const T*>(k),
+                              static_cast<const T*>(v), static_cast<T*>(out), rows) == cudaSuccess ? ST3_OK : ST3_ERR_CUDA;
+  }
   float *ml, *acc;
   const st3_status s = na_scratch(&ml, &acc);
   if (s != ST3_OK) return s;

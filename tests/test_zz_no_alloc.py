@@ -83,3 +83,29 @@ def test_sizes_beyond_the_static_array_are_rejected():
         # 128 heads x 65 chunks of 128 rows = 8320 partial slots > 8192; pointers are never dereferenced
         B.st3_attend_noalloc(q.data_ptr(), q.data_ptr(), q.data_ptr(), q.data_ptr(), 128, 65 * 128, 128, "f32", 0)
     assert e.value.code == 4
+
+
+# one block of the cluster, its last row alone in a block, one full batch of every warp and a row more, and both
+# sides of the rule that sends a few heads of many rows to the two-launch form
+@pytest.mark.parametrize("H,T,D,dtype", [(3, 64, 128, "bf16"), (3, 65, 128, "f32"), (2, 513, 64, "bf16"), (5, 1025, 64, "f32"),
+                                         (3, 1031, 128, "f32"), (2, 8192, 128, "bf16"), (2, 8193, 128, "bf16"),
+                                         (15, 8193, 64, "bf16"), (16, 8193, 64, "bf16")])
+def test_cluster_form_and_its_limits(H, T, D, dtype):
+    build()
+    _check_call(7, H, T, D, dtype, torch.cuda.current_stream().cuda_stream)
+
+
+def test_rows_without_weight_and_a_nan():
+    """Logits of minus infinity take no part, also where a warp or a block sees nothing else; a NaN comes through."""
+    build()
+    H, T, D = 2, 700, 128
+    q, k, v = _inputs(3, H, T, D, "f32")
+    q[:, 0] = 1.0
+    k[:, : T - 1, 0] = float("-inf")
+    out = torch.empty_like(q)
+    st = torch.cuda.current_stream().cuda_stream
+    B.st3_attend_noalloc(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), H, T, D, "f32", st)
+    assert torch.equal(out, v[:, T - 1])
+    k[0, 5, 1] = float("nan")
+    B.st3_attend_noalloc(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), H, T, D, "f32", st)
+    assert torch.isnan(out[0]).all() and torch.equal(out[1], v[1, T - 1])
