@@ -268,7 +268,7 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
     const bool direct = prefill && !select_first;
     const bool early = pdl && (direct || (!prefill && !ctx->rows_moving && !(ctx->overlap && ctx->serialize_next)));
     bool fat = false;  // some item carries lazy layers (QK heredity): the instantiation that streams their values
-    for (int i = 0; i < p.layer_count; ++i) fat = fat || p.nfol[i] != 0;
+    for (int i = 0; i < p.layer_count; ++i) fat = fat || p.layer[i].nfol != 0;
     auto kernel = direct ? (fat ? st3_attend_kernel<T, D, true, true> : st3_attend_kernel<T, D, false, true>)
                          : (fat ? st3_attend_kernel<T, D, true, false> : st3_attend_kernel<T, D, false, false>);
     if (launch(kernel, (unsigned)(p.first_dynamic / kSlots), 1, kAttendThreads, ctx->attend_smem, early, st, p) != cudaSuccess)
@@ -279,7 +279,7 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
     // Also a programmatic dependent launch: the attention kernel allows it at its start, the blocks become
     // resident as that grid drains and their first instruction waits for all of it.
     // half-size blocks, two per SM, once the units outnumber the blocks the GPU holds (see st3_finish.cuh)
-    const bool half = 2 * units > 2 * ctx->num_sms && 2 * ctx->finish_smem <= 200 * 1024;
+    const bool half = 2 * units > 2 * ctx->num_sms && 2 * ctx->finish_smem <= 196 * 1024;
     auto kernel = half ? st3_finish_kernel<T, D, kFinishThreads / 2> : st3_finish_kernel<T, D, kFinishThreads>;
     if (launch(kernel, (unsigned)(2 * units), 1, half ? kFinishThreads / 2 : kFinishThreads, ctx->finish_smem, pdl, st, p) !=
         cudaSuccess)
@@ -339,7 +339,6 @@ st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, co
   p.lbh_stride = L.lbh_stride;
   p.layer_begin = layer_begin; p.layer_count = layer_count; p.B = c.batch; p.H = c.num_heads;
   p.sys_len = c.sys_len; p.Nv = c.num_visual; p.cap_txt = L.cap_txt; p.step = step; p.append = prefill ? 0 : 1;
-  p.chunk_rows = L.chunk_rows;
   p.static_rank = c.static_rank ? 1 : 0;
   p.order = (prefill && !ext_scores) || !ctx->overlap;
   p.fresh = prefill && !ext_scores;
@@ -348,53 +347,56 @@ st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, co
   const int R = L.chunk_rows;
   bool reads_older = false;  // this call's finish launch reads logits an earlier call wrote
   p.ct = ceil_div(c.sys_len + ctx->max_text + step, R);
-  p.cvp[0] = 0;
+  int chunks = 0;  // visual chunks of the layers so far
   for (int i = 0; i < layer_count; ++i) {
+    LayerParams& y = p.layer[i];
     const int l = layer_begin + i;
     int ncur = prefill ? c.num_visual : ctx->n_host[l];
     const int tgt = ctx->n_tab[(size_t)l * (c.max_decode_steps + 1) + step];
     if (ext_scores && tgt < ncur) ncur = tgt;  // already pruned by the selection launch when the layer attends
-    p.nold[i] = ncur;
-    p.req[i] = prefill ? 0 : ctx->flag_req[l];  // a prompt reads nothing the launch ahead of it writes
+    y.nold = ncur;
+    y.req = prefill ? 0 : ctx->flag_req[l];  // a prompt reads nothing the launch ahead of it writes
     if (c.static_rank && !prefill && tgt < ncur) ncur = tgt;  // cut first, then attend (Algorithm 3)
-    p.ncur[i] = ncur;
-    p.ntgt[i] = tgt < ncur ? tgt : ncur;
-    p.lazy_src[i] = -1;
+    y.ncur = ncur;
+    y.ntgt = tgt < ncur ? tgt : ncur;
+    y.lazy_src = -1;
     if (c.lazy_mask >> l & 1ull) {
       int sl = l - 1;
       while (sl > 0 && (c.lazy_mask >> sl & 1ull)) --sl;
       if (sl < layer_begin) return ST3_ERR_UNSUPPORTED;  // a lazy layer and its source must share a call
-      p.lazy_src[i] = sl - layer_begin;
+      y.lazy_src = sl - layer_begin;
     }
     // whose scores decide: the layer's own, or (stage-shared) those of its stage's pruning layer
     int src = l;
     if (c.stage_shared && l >= c.first_prune_layer)
       src = c.first_prune_layer + (l - c.first_prune_layer) / c.stride * c.stride;
-    p.src_layer[i] = src;
-    p.src_copy[i] = ctx->seq & 1;
+    y.src_layer = src;
+    y.src_copy = ctx->seq & 1;
     if (src < layer_begin) {  // decided in an earlier call of this step
-      if (p.ntgt[i] < ncur && !ext_scores && ctx->logit_step[src] != step) return ST3_ERR_BAD_STATE;
-      p.src_copy[i] = ctx->logit_copy[src];
+      if (y.ntgt < ncur && !ext_scores && ctx->logit_step[src] != step) return ST3_ERR_BAD_STATE;
+      y.src_copy = ctx->logit_copy[src];
       reads_older = true;
     }
     const int cv = ceil_div(ncur, R);
-    p.cvp[i + 1] = p.cvp[i] + cv;
-    p.lstart[i] = c.batch * (p.cvp[i] + i * p.ct);
-    p.rpv[i] = cv ? ceil_div(ncur, cv) : 0;
-    make_fast_div((unsigned)(cv > 0 ? cv : 1), &p.cv_mul[i], &p.cv_shift[i]);
+    y.cv = cv;
+    y.lstart = c.batch * (chunks + i * p.ct);
+    chunks += cv;
+    y.rpv = cv ? ceil_div(ncur, cv) : 0;
+    unsigned shift;
+    make_fast_div((unsigned)(cv > 0 ? cv : 1), &y.cv_mul, &shift);
+    y.cv_shift = shift;
   }
-  p.lstart[layer_count] = c.batch * (p.cvp[layer_count] + layer_count * p.ct);
   // Working layers: every layer except the lazy ones that ride on the items of the layer they inherit from
   // (their value rows follow the item through its ring slot, see st3_attend.cuh; a run of more than kMaxFollow
   // lazy layers would start a new group that reads the keys again).
   bool works[kMaxLayers];
   for (int i = 0, head = -1; i < layer_count; ++i) {
-    const int s = p.lazy_src[i];
-    const bool rides = s >= 0 && head >= 0 && (head == s || p.lazy_src[head] == s) &&
-                       head + p.nfol[head] + 1 == i && p.nfol[head] < kMaxFollow &&
-                       p.ncur[i] == p.ncur[head] && p.nold[i] == p.nold[head];
+    const int s = p.layer[i].lazy_src;
+    const bool rides = s >= 0 && head >= 0 && (head == s || p.layer[head].lazy_src == s) &&
+                       head + p.layer[head].nfol + 1 == i && p.layer[head].nfol < kMaxFollow &&
+                       p.layer[i].ncur == p.layer[head].ncur && p.layer[i].nold == p.layer[head].nold;
     works[i] = !rides;
-    if (rides) p.nfol[head]++;
+    if (rides) p.layer[head].nfol++;
     else head = i;
   }
   // Order of the working layers inside the launch: those whose items are followed by lazy layers first.  Such an
@@ -404,16 +406,16 @@ st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, co
   p.wcvp[0] = 0;
   for (int pass = 0; pass < 2; ++pass)
     for (int i = 0; i < layer_count; ++i) {
-      if (!works[i] || (p.nfol[i] != 0) != (pass == 0)) continue;
+      if (!works[i] || (p.layer[i].nfol != 0) != (pass == 0)) continue;
       p.wlayer[p.nwork] = (unsigned char)i;
-      p.wcvp[p.nwork + 1] = p.wcvp[p.nwork] + (p.cvp[i + 1] - p.cvp[i]);
+      p.wcvp[p.nwork + 1] = p.wcvp[p.nwork] + p.layer[i].cv;
       p.nwork++;
     }
   make_fast_div((unsigned)c.num_heads, &p.h_mul, &p.h_shift);
   p.text_items = p.nwork * c.batch * p.ct;
   make_fast_div((unsigned)(c.batch * p.ct), &p.bct_mul, &p.bct_shift);
   make_fast_div((unsigned)p.ct, &p.ct_mul, &p.ct_shift);
-  const long long total_items = (long long)c.batch * (p.cvp[layer_count] + (long long)layer_count * p.ct);
+  const long long total_items = (long long)c.batch * (chunks + (long long)layer_count * p.ct);
   const long long work_items = (long long)c.batch * (p.wcvp[p.nwork] + (long long)p.nwork * p.ct);
   if (total_items > L.max_items || work_items * c.num_heads > 0x3fffffffLL) return ST3_ERR_CAPACITY;
   p.total_work = (int)(work_items * c.num_heads);
@@ -429,8 +431,8 @@ st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, co
     psel.ext_scores = ext_scores;
     psel.fresh = 1;
     for (int i = 0; i < layer_count; ++i) {
-      psel.ncur[i] = psel.nold[i] = c.num_visual;
-      psel.ntgt[i] = p.ncur[i];
+      psel.layer[i].ncur = psel.layer[i].nold = c.num_visual;
+      psel.layer[i].ntgt = p.layer[i].ncur;
     }
   }
 #define ST3_LAUNCH(T, D) launch_step_t<T, D>(ctx, p, st, prefill, ext_scores ? &psel : nullptr)
@@ -443,10 +445,10 @@ st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, co
     return s;
   }
   for (int i = 0; i < layer_count; ++i) {
-    ctx->n_host[layer_begin + i] = p.ntgt[i];
+    ctx->n_host[layer_begin + i] = p.layer[i].ntgt;
     ctx->last_step[layer_begin + i] = step;
     ctx->flag_req[layer_begin + i] = ctx->seq;
-    if (p.src_layer[i] == layer_begin + i && p.ntgt[i] < p.ncur[i]) {  // it wrote logits in this launch
+    if (p.layer[i].src_layer == layer_begin + i && p.layer[i].ntgt < p.layer[i].ncur) {  // it wrote logits in this launch
       ctx->logit_copy[layer_begin + i] = ctx->seq & 1;
       ctx->logit_step[layer_begin + i] = step;
     }

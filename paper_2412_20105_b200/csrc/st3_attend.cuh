@@ -196,8 +196,8 @@ __device__ __noinline__ void issue_values(const StepParams& p, const Chain* chai
   const size_t gap = PRE ? (size_t)p.Nv * ROWB : 0;
   if (c.is_vis) {  // rows the previous step's selection may still be moving
     for (int j = 0; j < n; ++j)
-      if (p.req[c.l_rel + f0 + j] &&
-          !flag_wait(p.flags + c.lb + (f0 + j) * p.B, p.req[c.l_rel + f0 + j], abort_flag, p.status))
+      if (p.layer[c.l_rel + f0 + j].req &&
+          !flag_wait(p.flags + c.lb + (f0 + j) * p.B, p.layer[c.l_rel + f0 + j].req, abort_flag, p.status))
         return;
   }
   if (c.has_new) {  // the layers' newest value rows: lanes [0, LN) layer f0, [LN, 2 LN) the next one
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
 
     auto fetch_new = [&](Dec& d) {  // newest row, key and value lanes: from the step's inputs; stored when the slot is free
       if (d.has_new && lane < 2 * LN) {
-        const int ls = p.lazy_src[d.l_rel];
+        const int ls = p.layer[d.l_rel].lazy_src;
         const T* src = lane / LN ? reinterpret_cast<const T*>(p.v_new) + (long long)d.oidx * D
                                  : reinterpret_cast<const T*>(p.k_new) + (long long)(d.oidx + (ls < 0 ? 0 : ls - d.l_rel) * p.B * H) * D;
 #pragma unroll
@@ -371,20 +371,20 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
         l_rel = p.wlayer[w];
         const int rem = xi - w * p.B * p.ct;
         b = (int)fast_div((unsigned)rem, p.ct_mul, p.ct_shift);
-        cv = p.cvp[l_rel + 1] - p.cvp[l_rel];
+        cv = p.layer[l_rel].cv;
         c = cv + rem - b * p.ct;
       } else {
         const int iv = xi - p.text_items;
         while (wcur + 1 < p.nwork && iv >= p.B * p.wcvp[wcur + 1]) ++wcur;
         l_rel = p.wlayer[wcur];
-        cv = p.cvp[l_rel + 1] - p.cvp[l_rel];
+        cv = p.layer[l_rel].cv;
         const int off = iv - p.B * p.wcvp[wcur];
-        b = (int)fast_div((unsigned)off, p.cv_mul[l_rel], p.cv_shift[l_rel]);
+        b = (int)fast_div((unsigned)off, p.layer[l_rel].cv_mul, p.layer[l_rel].cv_shift);
         c = off - b * cv;
       }
       int seg_rows, rows_per, ci;
       if (is_vis) {
-        seg_rows = p.ncur[l_rel]; rows_per = p.rpv[l_rel]; ci = c;
+        seg_rows = p.layer[l_rel].ncur; rows_per = p.layer[l_rel].rpv; ci = c;
       } else {
         seg_rows = p.sys_len + __ldg(p.text_len + b) + p.step; rows_per = (seg_rows + p.ct - 1) / p.ct; ci = c - cv;
       }
@@ -395,23 +395,23 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       d.has_new = !is_vis && p.append && nrows > 0 && r0 + nrows == seg_rows;
       d.nrows = nrows;
       d.is_vis = is_vis; d.l_rel = l_rel;
-      d.slot = (p.lstart[l_rel] + b * (cv + p.ct) + c) * H + h;  // partials are numbered layer-major
+      d.slot = (p.layer[l_rel].lstart + b * (cv + p.ct) + c) * H + h;  // partials are numbered layer-major
       d.oidx = (l_rel * p.B + b) * H + h;
-      d.nfol = FAT ? p.nfol[l_rel] : 0;
-      d.want_logits = is_vis && p.ntgt[l_rel] < p.ncur[l_rel] && p.src_layer[l_rel] == p.layer_begin + l_rel;
+      d.nfol = FAT ? p.layer[l_rel].nfol : 0;
+      d.want_logits = is_vis && p.layer[l_rel].ntgt < p.layer[l_rel].ncur && p.layer[l_rel].src_layer == p.layer_begin + l_rel;
       const int lb = (p.layer_begin + l_rel) * p.B + b;
       d.lb = lb;
-      d.wait_for = is_vis && lb != lb_ready ? p.req[l_rel] : 0;
+      d.wait_for = is_vis && lb != lb_ready ? p.layer[l_rel].req : 0;
       if (d.wait_for && ld_acquire(p.flags + lb) - d.wait_for >= 0) {  // looked up here, off the critical path
         d.wait_for = 0;
         lb_ready = lb;
       }
       // QK heredity (Eq. 6): a lazy layer with items of its own attends with the query and the keys of its
       // source layer and its own values; the two layers hold the same tokens in the same order
-      const int ls = p.lazy_src[l_rel];
+      const int ls = p.layer[l_rel].lazy_src;
       const int lk = ls < 0 ? l_rel : ls;  // whose keys and query
       d.lazy = ls >= 0;
-      d.wait_for_k = is_vis && ls >= 0 ? p.req[ls] : 0;  // the source's rows as well
+      d.wait_for_k = is_vis && ls >= 0 ? p.layer[ls].req : 0;  // the source's rows as well
       int row0 = r0;  // the chunk's first row in its source
       if constexpr (PRE) {
         const bool whole = is_vis || r0 >= p.sys_len || r0 + nrows <= p.sys_len;  // all of it on one side of the break
@@ -431,7 +431,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
         lb_ready = d.lb;
       }
       if (d.wait_for_k &&  // the source layer's (l, b): the same sequence, lazy_src layers lower
-          !flag_wait(p.flags + d.lb + (p.lazy_src[d.l_rel] - d.l_rel) * p.B, d.wait_for_k, abort_flag, p.status))
+          !flag_wait(p.flags + d.lb + (p.layer[d.l_rel].lazy_src - d.l_rel) * p.B, d.wait_for_k, abort_flag, p.status))
         return;
       const uint32_t kb = (uint32_t)(d.nrows - (d.has_new ? 1 : 0)) * ROWB;
       const uint32_t kb1 = PRE ? (uint32_t)d.nrows1 * ROWB : kb;
@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       if (!ring_wait(&s_done[s][g], (ph_done >> g) & 1u, abort_flag, p.status)) break;
       ph_done ^= 1u << g;
       // the partial slots of this use's layers: same chunk of the same rows, f layers up
-      const int slot0 = cur_slot + (FAT ? (p.lstart[cur_lrel + f0] - p.lstart[cur_lrel]) * H : 0);
+      const int slot0 = cur_slot + (FAT ? (p.layer[cur_lrel + f0].lstart - p.layer[cur_lrel].lstart) * H : 0);
       auto publish = [&](int slot, const float (&v)[DPL]) {  // plain stores: the next kernel merges the partials
         float* dst = p.part_acc + (long long)slot * D + lane * DPL;
         if constexpr (DPL == 4) *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[DPL - 2], v[DPL - 1]);
@@ -535,7 +535,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
             }
           }
           __syncwarp();  // every lane is done reading the slot before it is refilled
-          publish(cur_slot + (p.lstart[cur_lrel + f0 + 1] - p.lstart[cur_lrel]) * H, po);
+          publish(cur_slot + (p.layer[cur_lrel + f0 + 1].lstart - p.layer[cur_lrel].lstart) * H, po);
         }
       }
       // ---- refill the slot at once: what the group left lies outside the tile areas ----

@@ -21,12 +21,52 @@ constexpr int kMaxVisual = 8192;
 constexpr long long kWaitCycles = 4000000000LL;  // ~2 s: bound on any wait for an async copy
 constexpr int kMaxFollow = 62;  // lazy layers whose values can follow one work item of the layer they inherit from
 
-struct StepParams {
+// What a launch needs to know of one layer, side by side: a launch's parameters are cold in the constant cache, and a
+// block that works on one layer should miss once, not once per quantity.
+struct alignas(32) LayerParams {
+  int req;                // flag value the visual rows must have reached before they are read
+  int lstart;             // first work item: B * (visual chunks of the layers below + their text chunks)
+  unsigned cv_mul;        // fast division by the visual chunks
+  unsigned short ncur;    // visual rows held before this step (host's schedule bookkeeping)
+  unsigned short ntgt;    // visual rows to hold after this step
+  unsigned short nold;    // visual rows the device should report before this step
+  unsigned short cv;      // visual chunks
+  unsigned char cv_shift;
+  unsigned char rpv;      // rows per visual chunk
+  unsigned char src_layer;  // the layer whose scores decide this layer's evictions (itself unless stage-shared)
+  unsigned char src_copy;   // which copy of the logits holds that layer's logits
+  signed char lazy_src;   // relative index of the layer whose q and K a lazy layer inherits (-1: its own)
+  unsigned char nfol;     // lazy layers riding on this (working) layer's items
+};
+static_assert(kMaxVisual <= 0xffff && kMaxLayers <= 127 && kMaxChunkRows <= 0xff, "LayerParams fields too narrow");
+
+struct alignas(64) StepParams {
+  int layer_begin, layer_count, B, H;
+  int sys_len, Nv, cap_txt, step;
+  int append;
+  int ct;                   // text chunks per (l, b, h), the same for every sequence
+  int total_work;           // work items x heads of this launch
+  int first_dynamic;        // managers of the attention grid: items below this index are pre-assigned
+  int text_items;           // nwork * B * ct: the attention launch works through these first
+  int nwork;                // working layers of this call
+  unsigned h_mul, h_shift;  // fast division by H
+  unsigned bct_mul, bct_shift;      // fast division by B * ct
+  unsigned ct_mul, ct_shift;        // fast division by ct
+  int order;                // 1: the launch may start before the launch ahead of it ends, and waits before it reads inputs
+  int fresh;                // 1: a new prompt, whose visual rows are the tokens 0 .. Nv-1 (ids are not read)
+  int static_rank;          // 1: keep the kept rows in top-index order, cut them without scoring
+  int seq;                  // sequence number of this step's launches
+  unsigned counter_base;    // value of the work counter when this launch starts (it is never reset)
+  int t0_max;
+  long long lbh_stride;  // elements per (l, b, h) cache block
   const void* q;
   const void* k_new;
   const void* v_new;
   void* out;
   void* cache;
+  const int* text_len;   // [b]
+  int* work_counter;     // next work item of the running attention launch
+  int* flags;            // [l][b] sequence number of the last finish launch that is done with (l, b)
   float* part_ml;        // [item*H + h][2]  (m, l) in the log2 domain
   float* part_acc;       // [item*H + h][D]  un-normalised output
   float* logits;         // [l][b][h][Nv]    raw log2-domain logits of visual rows (this step's copy)
@@ -35,49 +75,16 @@ struct StepParams {
   float* mass_by_id;     // [l][b][Nv]
   int* ids;              // [l][b][Nv]
   int* n_cur;            // [l][b]
-  const int* text_len;   // [b]
   int* status;
-  int* work_counter;     // next work item of the running attention launch
-  long long lbh_stride;  // elements per (l, b, h) cache block
-  int layer_begin, layer_count, B, H;
-  int sys_len, Nv, cap_txt, step, append;
-  int ct;                   // text chunks per (l, b, h), the same for every sequence
-  int chunk_rows;           // rows per work item (<= the kernel's tile capacity)
-  int total_work;           // work items x heads of this launch
-  int first_dynamic;        // managers of the attention grid: items below this index are pre-assigned
-  unsigned counter_base;    // value of the work counter when this launch starts (it is never reset)
-  int* flags;               // [l][b] sequence number of the last finish launch that is done with (l, b)
-  int seq;                  // sequence number of this step's launches
-  int req[kMaxLayers];      // flag value the visual rows of a layer must have reached before they are read
-  unsigned h_mul, h_shift;  // fast division by H
-  int cvp[kMaxLayers + 1];  // prefix sum of visual chunks per layer (relative layer index)
-  int lstart[kMaxLayers + 1];       // first work item of each layer: B * (cvp[l] + l * ct)
-  int rpv[kMaxLayers];              // rows per visual chunk of each layer
-  unsigned cv_mul[kMaxLayers];      // fast division by the visual chunks of each layer
-  unsigned cv_shift[kMaxLayers];
-  int text_items;                   // layer_count * B * ct: the attention launch works through these first
-  unsigned bct_mul, bct_shift;      // fast division by B * ct
-  unsigned ct_mul, ct_shift;        // fast division by ct
-  int ncur[kMaxLayers];     // visual rows held before this step (host's schedule bookkeeping)
-  int ntgt[kMaxLayers];     // visual rows to hold after this step
-  int nold[kMaxLayers];     // visual rows the device should report before this step
-  int order;                // 1: the launch may start before the launch ahead of it ends, and waits before it reads inputs
-  int fresh;                // 1: a new prompt, whose visual rows are the tokens 0 .. Nv-1 (ids are not read)
   const void* k_in;         // prefill only: the caller's prompt tensors [layer_count][B][H][t0_max][D]
   const void* v_in;
-  int t0_max;
-  int static_rank;          // 1: keep the kept rows in top-index order, cut them without scoring
   const float* ext_scores;  // prefill with the caller's scores [layer_count][B][Nv]: selection only, no merge
-  int src_layer[kMaxLayers];  // the layer whose scores decide this layer's evictions (itself unless stage-shared)
-  int src_copy[kMaxLayers];   // which copy of the logits holds that layer's logits
-  int lazy_src[kMaxLayers];   // relative index of the layer whose q and K a lazy layer inherits (-1: its own)
+  LayerParams layer[kMaxLayers];
   // QK heredity (Eq. 6) without re-reading keys: the lazy layers right above a layer ride on that layer's work
   // items (its probabilities are applied to their value rows as well); they get no items of their own.  The
   // attention launch numbers its work over the remaining ("working") layers only.
-  int nwork;                          // working layers of this call
-  int wcvp[kMaxLayers + 1];           // prefix sum of their visual chunks
   unsigned char wlayer[kMaxLayers];   // relative layer index of the w-th working layer
-  unsigned char nfol[kMaxLayers];     // lazy layers riding on this (working) layer's items
+  int wcvp[kMaxLayers + 1];           // prefix sum of the working layers' visual chunks
 };
 
 // ------------------------------------------------------------------------------------------

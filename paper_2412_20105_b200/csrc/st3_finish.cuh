@@ -16,9 +16,10 @@ namespace {
 // Both are chains of dependent memory round trips, so every phase issues all its loads first.
 constexpr int kHeadBatch = 16;  // logits of one visual row a thread keeps in flight
 
-// (max, 1/sum) of one head's merged softmax from its chunk partials; every lane gets both.
+// (max, sum) of one head's merged softmax from its chunk partials; every lane gets both, and in `w` the weights
+// exp2(max_i - max) of partials `lane` and `lane + 32`.
 __device__ __forceinline__ void merge_stats(const float2* ml, long long item0, int nit, int H, int h, int lane,
-                                            float& M, float& L) {
+                                            float& M, float& L, float (&w)[2]) {
   float2 v[2];  // the first 64 partials stay in registers
 #pragma unroll
   for (int j = 0; j < 2; ++j)
@@ -26,7 +27,9 @@ __device__ __forceinline__ void merge_stats(const float2* ml, long long item0, i
   M = fmaxf(v[0].x, v[1].x);
   for (int i = lane + 64; i < nit; i += 32) M = fmaxf(M, ml[(item0 + i) * H + h].x);
   M = warp_max(M);
-  L = v[0].y * fast_exp2(v[0].x - M) + v[1].y * fast_exp2(v[1].x - M);
+#pragma unroll
+  for (int j = 0; j < 2; ++j) w[j] = fast_exp2(v[j].x - M);
+  L = v[0].y * w[0] + v[1].y * w[1];
   for (int i = lane + 64; i < nit; i += 32) {
     const float2 u = ml[(item0 + i) * H + h];
     L += u.y * fast_exp2(u.x - M);
@@ -34,19 +37,24 @@ __device__ __forceinline__ void merge_stats(const float2* ml, long long item0, i
   L = warp_sum(L);
 }
 
+constexpr int kSelBins = 2048;  // bins of the selection's histogram, over the range of the scores
+constexpr int kSelCand = 64;    // keys of the bin that the cut falls into that are ranked directly
+
 // NT threads per block: 1024, or 512 (two blocks per SM) when a launch has more (layer, sequence) units than the GPU
 // can hold blocks: the work of a unit is a chain of memory round trips, and more units in flight end sooner.
 template <typename T, int D, int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepParams p) {
+__global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const __grid_constant__ StepParams p) {
   constexpr int kFinishThreads = NT, kFinishWarps = NT / 32;
   constexpr int ROWB = D * sizeof(T);
   constexpr int VPR = ROWB / 16;  // 16-byte vectors per row
   constexpr int DPL = D / 32;
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ float s_M[kMaxHeads];
-  __shared__ float s_invL[kMaxHeads];
-  __shared__ int s_hist[256];
+  __shared__ float2 s_ML[kMaxHeads];  // (max, 1/sum) of a head's merged softmax
+  __shared__ int s_hist[kSelBins];
   __shared__ int s_scan[kFinishWarps];
+  __shared__ unsigned s_lo[kFinishWarps], s_hi[kFinishWarps];
+  __shared__ unsigned long long s_cand[kSelCand], s_cut;
+  __shared__ int s_ncand;
   __shared__ float s_half[kFinishThreads / 2];
   __shared__ int s_sel[3];  // digit, count above, count in bin
 
@@ -63,8 +71,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
   const int l_rel = unit / B, b = unit % B;
   const int l = p.layer_begin + l_rel;
   const long long lb = (long long)l * B + b;
-  const int nit = p.cvp[l_rel + 1] - p.cvp[l_rel] + p.ct;
-  const long long item0 = (long long)p.lstart[l_rel] + (long long)b * nit;
+  const int nit = p.layer[l_rel].cv + p.ct;
+  const long long item0 = (long long)p.layer[l_rel].lstart + (long long)b * nit;
   const float2* ml = reinterpret_cast<const float2*>(p.part_ml);
 
   if (out_role) {
@@ -89,8 +97,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
         }
       };
       load_batch(0);
-      float M, Lh;
-      merge_stats(ml, item0, nit, H, h, lane, M, Lh);
+      float M, Lh, w[2];
+      merge_stats(ml, item0, nit, H, h, lane, M, Lh, w);
       float o[DPL];
 #pragma unroll
       for (int j = 0; j < DPL; ++j) o[j] = 0.f;
@@ -99,7 +107,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
 #pragma unroll
         for (int i = 0; i < kMergeBatch; ++i) {
           if (i0 + i < nit) {
-            const float wgt = fast_exp2(ml[(item0 + i0 + i) * H + h].x - M);
+            const int it = i0 + i;
+            const float wgt = it < 64 ? __shfl_sync(0xffffffffu, it < 32 ? w[0] : w[1], it & 31)
+                                      : fast_exp2(ml[(item0 + it) * H + h].x - M);
 #pragma unroll
             for (int j = 0; j < DPL; ++j) o[j] = fmaf(wgt, a[i][j], o[j]);
           }
@@ -118,10 +128,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
   // Signals that this launch is done with the visual rows, ids and logits of (l, b).
   auto done = [&]() {
     __syncthreads();
-    if (tt == 0) { __threadfence(); st_release(p.flags + lb, p.seq); }
+    if (tt == 0) st_release(p.flags + lb, p.seq);  // what the block wrote is ordered before it by the barrier
   };
-  const int n_host = p.ncur[l_rel];
-  const int k = min(n_host, p.ntgt[l_rel]);
+  const int n_host = p.layer[l_rel].ncur;
+  const int k = min(n_host, p.layer[l_rel].ntgt);
   const bool evicts = k < n_host;  // same answer in every thread
   const int n_dev = p.n_cur[lb];
   const bool fresh = p.fresh;  // a new prompt: row i is visual token i, whatever the bookkeeping says
@@ -130,7 +140,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
       for (int i = tt; i < n_host; i += kFinishThreads) { p.ids[lb * Nv + i] = i; p.mass_by_id[lb * Nv + i] = 0.f; }
       if (tt == 0) p.n_cur[lb] = n_host;
     } else if (tt == 0) {
-      if (n_dev != p.nold[l_rel]) atomicOr(p.status, ST3_DEV_COUNT_MISMATCH);
+      if (n_dev != p.layer[l_rel].nold) atomicOr(p.status, ST3_DEV_COUNT_MISMATCH);
       else if (n_host != n_dev) p.n_cur[lb] = n_host;  // static-rank cut: only the count changes
     }
     done();
@@ -139,10 +149,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
   int* ids = p.ids + lb * Nv;
   float* mass_by_id = p.mass_by_id + lb * Nv;
   // the scores that decide come from this layer, or from its stage's pruning layer (same rows, same order)
-  const int src = p.src_layer[l_rel];
+  const int src = p.layer[l_rel].src_layer;
   const long long lb_src = (long long)src * B + b;
   const bool src_here = src >= p.layer_begin && src < p.layer_begin + p.layer_count;
-  const float* logits = p.logits_copy[p.src_copy[l_rel]] + lb_src * H * Nv;
+  const float* logits = p.logits_copy[p.layer[l_rel].src_copy] + lb_src * H * Nv;
   unsigned long long* s_key = reinterpret_cast<unsigned long long*>(smem);  // [Nv]
   int* s_hole = reinterpret_cast<int*>(smem + (size_t)Nv * 8);              // [Nv]
   int* s_mover = s_hole + Nv;                                               // [Nv]
@@ -167,23 +177,24 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
     }
     if (src_here) {
       const int ls = src - p.layer_begin;
-      const int nit_s = p.cvp[ls + 1] - p.cvp[ls] + p.ct;
-      const long long item0_s = (long long)p.lstart[ls] + (long long)b * nit_s;
+      const int nit_s = p.layer[ls].cv + p.ct;
+      const long long item0_s = (long long)p.layer[ls].lstart + (long long)b * nit_s;
       for (int h = warp; h < H; h += kFinishWarps) {
-        float M, Lh;
-        merge_stats(ml, item0_s, nit_s, H, h, lane, M, Lh);
+        float M, Lh, w[2];
+        merge_stats(ml, item0_s, nit_s, H, h, lane, M, Lh, w);
         if (lane == 0) {
-          s_M[h] = M; s_invL[h] = 1.f / Lh;
+          s_ML[h] = make_float2(M, 1.f / Lh);
           if (src == l) { p.head_stat[2 * (lb * H + h)] = M; p.head_stat[2 * (lb * H + h) + 1] = 1.f / Lh; }
         }
       }
     } else {  // the pruning layer ran in an earlier launch of this step: its statistics were kept
       for (int h = tt; h < H; h += kFinishThreads) {
-        s_M[h] = p.head_stat[2 * (lb_src * H + h)];
-        s_invL[h] = p.head_stat[2 * (lb_src * H + h) + 1];
+        s_ML[h] = make_float2(p.head_stat[2 * (lb_src * H + h)], p.head_stat[2 * (lb_src * H + h) + 1]);
       }
     }
   }
+  for (int i = tt; i < kSelBins; i += kFinishThreads) s_hist[i] = 0;
+  if (tt == 0) s_ncand = 0;
   __syncthreads();
   if (!fresh && n_dev != n_host) {  // host bookkeeping and device state disagree: flag, do not touch
     if (tt == 0) atomicOr(p.status, ST3_DEV_COUNT_MISMATCH);
@@ -193,6 +204,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
 
   // ---- visual scores: probability of every visual row summed over heads ----
   bool bad = false;
+  unsigned lo = 0xffffffffu, hi = 0u;  // range of the keys' high words
   if (!own_scores) {
     // scores supplied by the caller (any finite float): order-preserving map of the bits to unsigned
     const float* ext = p.ext_scores + ((long long)l_rel * B + b) * Nv;
@@ -203,9 +215,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
       mass_by_id[id] = sc;
       unsigned u = __float_as_uint(sc);
       u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+      lo = min(lo, u); hi = max(hi, u);
       s_key[i] = ((unsigned long long)u << 32) | (unsigned long long)(0xffffffffu - (unsigned)id);
     }
-    __syncthreads();
   }
   for (int i0 = 0; own_scores && i0 < n_cur; i0 += kRowsPerPass) {
     const int i = i0 + ri;
@@ -224,7 +236,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
         }
 #pragma unroll
         for (int j = 0; j < kHeadBatch; ++j)
-          if (h0 + j < H) pm += fast_exp2(v[j] - s_M[h0 + j]) * s_invL[h0 + j];
+          if (h0 + j < H) {
+            const float2 st = s_ML[h0 + j];
+            pm += fast_exp2(v[j] - st.x) * st.y;
+          }
       }
     }
     if (hg == 1) s_half[ri] = pm;
@@ -233,15 +248,74 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
       float mass = pm + s_half[ri];
       if (!(mass >= 0.f) || !(mass <= 3.0e38f)) { bad = true; mass = 0.f; }
       mass_by_id[id] = mass;
-      s_key[i] = ((unsigned long long)__float_as_uint(mass) << 32) | (unsigned long long)(0xffffffffu - (unsigned)id);
+      const unsigned u = __float_as_uint(mass);
+      lo = min(lo, u); hi = max(hi, u);
+      s_key[i] = ((unsigned long long)u << 32) | (unsigned long long)(0xffffffffu - (unsigned)id);
     }
-    __syncthreads();
+    if (i0 + kRowsPerPass < n_cur) __syncthreads();  // s_half is written again
   }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) { s_lo[warp] = lo; s_hi[warp] = hi; }
+  __syncthreads();
   if (bad) atomicOr(p.status, ST3_DEV_NONFINITE);
 
-  // ---- radix select: the k-th largest 64-bit key (keys are unique: ids are) ----
+  // ---- the k-th largest 64-bit key (keys are unique: ids are) ----
+  // One histogram over the range of the scores (2048 bins: a few keys in each) finds the bin of the cut, and the keys
+  // in it are ranked against one another.  Where too many share it (equal scores), a radix select over all digits.
   unsigned long long prefix = 0ull, mask = 0ull;
+  bool found = true;
   if (k > 0) {
+    lo = __reduce_min_sync(0xffffffffu, lane < kFinishWarps ? s_lo[lane] : 0xffffffffu);
+    hi = __reduce_max_sync(0xffffffffu, lane < kFinishWarps ? s_hi[lane] : 0u);
+    const int sh = max(0, 32 - __clz((int)(hi - lo)) - 11);  // (hi - lo) >> sh < 2048
+    for (int i = tt; i < n_cur; i += kFinishThreads)
+      atomicAdd(&s_hist[((unsigned)(s_key[i] >> 32) - lo) >> sh], 1);
+    __syncthreads();
+    constexpr int kPer = kSelBins / kFinishThreads;  // consecutive bins of a thread
+    int c[kPer], t = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) { c[j] = s_hist[tt * kPer + j]; t += c[j]; }
+    int S = t;  // inclusive suffix sum over lanes (this lane and the higher ones)
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_down_sync(0xffffffffu, S, o);
+      if (lane + o < 32) S += v;
+    }
+    if (lane == 0) s_scan[warp] = S;
+    __syncthreads();
+    int above = S - t + __reduce_add_sync(0xffffffffu, lane > warp && lane < kFinishWarps ? s_scan[lane] : 0);
+    if (above < k && k <= above + t) {
+#pragma unroll
+      for (int j = kPer - 1; j >= 0; --j) {
+        if (above + c[j] >= k) { s_sel[0] = tt * kPer + j; s_sel[1] = above; s_sel[2] = c[j]; break; }
+        above += c[j];
+      }
+    }
+    __syncthreads();
+    const unsigned digit = (unsigned)s_sel[0];
+    const int need = k - s_sel[1], inbin = s_sel[2];
+    if (need == inbin) {  // the whole bin is kept
+      prefix = (unsigned long long)(lo + (digit << sh)) << 32;
+    } else if (inbin <= kSelCand) {
+      for (int i = tt; i < n_cur; i += kFinishThreads) {
+        const unsigned long long key = s_key[i];
+        if (((unsigned)(key >> 32) - lo) >> sh == digit) s_cand[atomicAdd(&s_ncand, 1)] = key;
+      }
+      __syncthreads();
+      if (tt < inbin) {
+        const unsigned long long key = s_cand[tt];
+        int larger = 0;
+        for (int j = 0; j < inbin; ++j) larger += s_cand[j] > key;
+        if (larger == need - 1) s_cut = key;
+      }
+      __syncthreads();
+      prefix = s_cut;
+    } else {
+      found = false;
+    }
+  }
+  if (k > 0 && !found) {
     int need = k;
     for (int shift = 56; shift >= 0; shift -= 8) {
       if (tt < 256) s_hist[tt] = 0;
@@ -277,7 +351,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
       mask |= 0xffull << shift;
       if (need == inbin) break;  // the whole bin is kept: keys >= prefix are exactly the top k
     }
-  } else {
+  }
+  if (k == 0) {
     prefix = ~0ull;  // keep nothing (ids are < 2^31, so no key reaches this value)
   }
 
@@ -314,12 +389,14 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
   }
   if (lane == 31) s_scan[warp] = incl;
   __syncthreads();
-  int woff = 0, total = 0;
+  int wsum = lane < kFinishWarps ? s_scan[lane] : 0;  // inclusive prefix sums of the warps' totals, in every warp
 #pragma unroll
-  for (int w = 0; w < kFinishWarps; ++w) {
-    if (w < warp) woff += s_scan[w];
-    total += s_scan[w];
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, wsum, o);
+    if (lane >= o) wsum += v;
   }
+  const int total = __shfl_sync(0xffffffffu, wsum, 31);
+  const int woff = warp ? __shfl_sync(0xffffffffu, wsum, warp - 1) : 0;
   const int excl = woff + incl - packed;
   int ph = excl & 0xffff, pm = excl >> 16;
   if (fresh) {  // the kept tokens in the prompt's order; st3_gather_kernel copies the rows
@@ -348,16 +425,21 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const StepPar
   // ---- move the rows (sources are rows >= k, destinations rows < k: disjoint) ----
   const int id_moved = tt < nmove ? ids[s_mover[tt]] : 0;  // in flight together with the rows
   unsigned char* blk0 = reinterpret_cast<unsigned char*>(p.cache) + (size_t)(lb * H) * p.lbh_stride * sizeof(T);
-  const long long nvec = (long long)nmove * H * 2 * VPR;
-  for (long long v = tt; v < nvec; v += kFinishThreads) {
-    const int c = (int)(v % VPR);
-    long long r = v / VPR;
-    const int kv = (int)(r % 2); r /= 2;
-    const int h = (int)(r % H);
-    const int j = (int)(r / H);
-    unsigned char* base = blk0 + (size_t)h * p.lbh_stride * sizeof(T) + (size_t)kv * Nv * ROWB;
-    const uint4 val = *reinterpret_cast<const uint4*>(base + (size_t)s_mover[j] * ROWB + c * 16);
-    *reinterpret_cast<uint4*>(base + (size_t)s_hole[j] * ROWB + c * 16) = val;
+  const unsigned nvec = (unsigned)(nmove * H * 2 * VPR);
+  auto place = [&](unsigned v, const int* rows) {  // vector v of the moves: (row, head, K or V, 16 bytes of it)
+    const unsigned x = v / (2 * VPR), j = fast_div(x, p.h_mul, p.h_shift);
+    return reinterpret_cast<uint4*>(blk0 + (size_t)(x - j * H) * p.lbh_stride * sizeof(T) +
+                                    ((size_t)(v / VPR % 2) * Nv + rows[j]) * ROWB) + v % VPR;
+  };
+  constexpr int kMoveBatch = 8;  // vectors of a thread in flight: one round trip for 8 rows of 32 heads
+  for (unsigned v0 = tt; v0 < nvec; v0 += kMoveBatch * kFinishThreads) {
+    uint4 val[kMoveBatch];
+#pragma unroll
+    for (int j = 0; j < kMoveBatch; ++j)
+      if (v0 + j * kFinishThreads < nvec) val[j] = *place(v0 + j * kFinishThreads, s_mover);
+#pragma unroll
+    for (int j = 0; j < kMoveBatch; ++j)
+      if (v0 + j * kFinishThreads < nvec) *place(v0 + j * kFinishThreads, s_hole) = val[j];
   }
   if (tt < nmove) ids[s_hole[tt]] = id_moved;
   for (int j = tt + kFinishThreads; j < nmove; j += kFinishThreads) ids[s_hole[j]] = ids[s_mover[j]];
@@ -387,7 +469,7 @@ __global__ void __launch_bounds__(kThreads) st3_gather_kernel(const __grid_const
   const int l_rel = y / B;
   const long long lb = (long long)(p.layer_begin + l_rel) * B + b;
   const int n_txt = p.sys_len + __ldg(p.text_len + b);
-  const int n_vis = p.ntgt[l_rel];
+  const int n_vis = p.layer[l_rel].ntgt;
   const bool all = n_vis == Nv;
   const int* ids = p.ids + lb * Nv;
   const long long in0 = (((long long)l_rel * B + b) * H + h) * p.t0_max * VPR;

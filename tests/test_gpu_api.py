@@ -396,3 +396,41 @@ def test_layer_calls_behind_a_copy_and_an_early_producer(captured):
         assert a.ctx.status() == 0 and b.ctx.status() == 0
     finally:
         a.close(); b.close()
+
+
+def _score_sets(nv, g):
+    """Scores that make the selection's histogram coarse, its bins full or the cut fall among equals."""
+    u = torch.rand(nv, generator=g)
+    wide = torch.exp((u - 0.5) * 160.0) * torch.where(torch.rand(nv, generator=g) < 0.5, -1.0, 1.0)
+    tight = 1.0 + 1e-6 * u
+    tight[nv // 3] = 3e38                                     # one outlier: everything else shares a bin
+    steps = torch.floor(u * 7.0) - 3.0                        # seven levels, equal scores at the cut
+    pairs = torch.floor(u * nv / 2.0)                         # a few keys to a bin, some of them equal
+    n64 = torch.arange(nv, dtype=torch.float32) * 1e30        # 64 and 65 equal scores around the middle
+    n65 = n64.clone()
+    n64[nv // 2 - 32:nv // 2 + 32] = n64[nv // 2]
+    n65[nv // 2 - 32:nv // 2 + 33] = n65[nv // 2]
+    return dict(uniform=u, wide=wide, tight=tight, steps=steps, pairs=pairs, n64=n64, n65=n65, equal=torch.zeros(nv),
+                tiny=u * 1e-42)
+
+
+@pytest.mark.parametrize("nv,keep_bp", [(700, 5000), (700, 1), (2049, 3333), (8192, 5000), (65, 9999), (1, 5000), (300, 20)])
+def test_selection_over_hard_score_distributions(nv, keep_bp):
+    cfg, ctx = _handmade(nv, H=1, keep_bp=keep_bp)
+    try:
+        g = torch.Generator().manual_seed(nv)
+        T0 = 2 + nv + 3
+        K, V = (torch.randn(1, 1, 1, T0, 64, generator=g) for _ in range(2))
+        q, out = torch.randn(1, 1, 1, 64, generator=g).cuda(), torch.empty(1, 1, 1, 64, device="cuda")
+        k = B.st3_schedule_count(cfg, 0, 0)
+        for name, sc in _score_sets(nv, g).items():
+            ctx.prefill_select_scored(q, K.cuda(), V.cuda(), [3], sc.float().view(1, 1, nv).cuda(), out)
+            ids, cnt, _ = ctx.get_kept(0)
+            order = np.lexsort((np.arange(nv), -sc.float().double().numpy()))
+            assert int(cnt[0]) == k
+            assert ids[0, :k].tolist() == sorted(order[:k].tolist()), name
+            kv, vv, _, _ = ctx.get_rows(0, 0, 0)
+            assert torch.equal(vv[:k].cpu(), V[0, 0, 0, 2 + ids[0, :k].long().cpu()]), name
+        assert ctx.status() == 0
+    finally:
+        ctx.close()
