@@ -33,6 +33,7 @@ constexpr int kBoxBytes = 128 * 128;  // one TMA box of Q: 128 rows x 64 bf16
 constexpr int kTileBytes2 = 2 * kBoxBytes;
 constexpr int kKBoxBytes = kKeys * 128;  // one TMA box of K or V: 64 rows x 64 bf16
 constexpr int kKTileBytes = 2 * kKBoxBytes;
+constexpr unsigned kPfWave = 2 * 148;  // blocks the GPU holds, two to an SM
 constexpr uint32_t kTmemCols = 256;   // S in columns [0,64), O in [128,256)
 
 // One box of [rows][64 bf16] of instance z, starting at row y (may be negative or reach past the instance's
@@ -171,7 +172,10 @@ struct PrefillParams {
   __nv_bfloat16* out;   // [num_inst][T][128]
   float* head_probs;    // [num_inst][num_visual] last-row probabilities per head
   int* status;          // error word (may be null)
+  float* fill;          // scores by original index, set to -1 ahead of the sum over heads (null: not wanted)
+  int fill_per_seq, num_heads;
   int T, sys_len, num_visual;
+  int tile_major;       // grid (instance, tile) instead of (tile, instance)
 };
 
 __global__ void __launch_bounds__(kPfThreads, 2)
@@ -199,13 +203,15 @@ st3_prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
   }
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int qt = (int)gridDim.x - 1 - (int)blockIdx.x, inst = blockIdx.y;   // an instance's longest causal prefixes start first
+  const int ntile = (int)(p.tile_major ? gridDim.y : gridDim.x);
+  const int inst = p.tile_major ? blockIdx.x : blockIdx.y;
+  const int qt = ntile - 1 - (int)(p.tile_major ? blockIdx.y : blockIdx.x);   // the longest causal prefixes start first
   const int T = p.T;
   const int row_base = inst * T;  // first row of this instance in the [num_inst * T][128] tensors
   // Query tiles are aligned to the END of the prompt: the ragged tile is the first one, where the causal prefix
   // is shortest, instead of the last one, where a mostly empty tile would walk every key.  Its rows before the
   // prompt (q0 < 0) are dead: their loads read the fill value (zeros), nothing is stored.
-  const int q0 = T - ((int)gridDim.x - qt) * kTile;                // first query row of this tile
+  const int q0 = T - (ntile - qt) * kTile;                // first query row of this tile
   const int nkt = (q0 + kTile + kKeys - 1) / kKeys;                // causal: key tiles up to the diagonal
 
   if (tid == 4 * 32) {   // the control warp's first lane: barriers, then the first loads at once (they are in
@@ -215,6 +221,10 @@ st3_prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
     mbar_init(&bar_p[0], 128); mbar_init(&bar_p[1], 128); mbar_init(&bar_done, 1);
     s_fail = 0;
     mbar_fence_init();
+    // This block may have been set up while the launch ahead was still running; whatever starts early behind this
+    // launch in turn finds that launch complete.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     mbar_expect_tx(&bar_q, kTileBytes2);
     tma_load_3d(sQ, &map_q, 0, q0, inst, &bar_q);
     tma_load_3d(sQ + kBoxBytes, &map_q, 64, q0, inst, &bar_q);
@@ -326,6 +336,11 @@ st3_prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
     bool ok = true;
     float* probs = p.head_probs ? p.head_probs + (size_t)inst * p.num_visual : nullptr;
     const bool last_row = live && qi == T - 1;
+    if (p.fill && inst % p.num_heads == 0) {   // one head of each sequence, its tiles in turn
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      float* fill = p.fill + (size_t)(inst / p.num_heads) * p.fill_per_seq;
+      for (int i = qt * kTile + r; i < p.fill_per_seq; i += ntile * kTile) fill[i] = -1.f;
+    }
     for (int kt = 0; kt < nkt && ok; ++kt) {
       ok = pf_wait_warp(&bar_s[kt & 1], (kt >> 1) & 1);   // a failed control warp stops issuing: this wait then runs out
       if (!ok) break;
@@ -345,7 +360,7 @@ st3_prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
 #pragma unroll
         for (int e = 0; e < 4; ++e) m4[e] = fmax3(m4[e], __uint_as_float(v[c + e]), __uint_as_float(v[c + 4 + e]));
       const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * sc;   // the scale is positive: max and scaling commute
-      if (probs && qt == (int)gridDim.x - 1 && warp == 3) {
+      if (probs && qt == ntile - 1 && warp == 3) {
         // the last query row lives in one lane of this warp: hand its logits on the visual positions to the
         // whole warp, which stores them coalesced; they are normalised once the row is complete
         const int src = 31;   // the last query row is the last row of the last tile
@@ -415,7 +430,7 @@ st3_prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
     }
     if (ok) { ok = pf_wait_warp(&bar_done, 0) && !*fail; }   // the last P V: O is complete
     const float inv_l = l > 0.f ? 1.f / l : 0.f;
-    if (probs && qt == (int)gridDim.x - 1) {   // this block holds the last query row (same answer in every thread)
+    if (probs && qt == ntile - 1) {   // this block holds the last query row (same answer in every thread)
       // alpha of this head: exp2(logit - ref) / sum over the visual positions, with the last row's final
       // reference and sum; the 128 softmax threads share the work
       if (last_row) { s_last[0] = ref; s_last[1] = ok ? inv_l : 0.f; }
@@ -455,36 +470,36 @@ st3_prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
   }
 }
 
-// scores[b][i] = sum over the heads of sequence b of the last row's probability on visual token i
-__global__ void st3_prefill_scores_kernel(const float* __restrict__ head_probs, float* __restrict__ scores, int num_heads,
-                                          int num_visual) {
-  const int b = blockIdx.y;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= num_visual) return;
+// scores[b][i] = sum over the heads of sequence b of the last row's probability on visual token i.  With `ids` the
+// layer ran on the visual tokens an earlier layer kept: position i of its visual span is original token ids[b][i], and
+// the scores go out indexed by original token (tokens not held: -1, written by the attention launch ahead).
+// Eight groups of heads side by side: one or two round trips instead of one per four heads (the sum of 32 heads and its launch: 4.5 -> 2.5 us).
+constexpr int kScoreGroups = 8;
+__global__ void __launch_bounds__(32 * kScoreGroups)
+st3_prefill_scores_kernel(const float* __restrict__ head_probs, const int* __restrict__ ids, float* __restrict__ scores,
+                          int* status, int num_heads, int num_visual, int num_visual_total) {
+  __shared__ float s_part[kScoreGroups][32];
+  const int b = blockIdx.y, lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  int id = i;
   float s = 0.f;
-  for (int h = 0; h < num_heads; ++h) s += head_probs[((size_t)b * num_heads + h) * num_visual + i];
-  scores[(size_t)b * num_visual + i] = s;
-}
-
-// The same sum for a layer that ran on the visual tokens an earlier layer kept: position i of the layer's visual
-// span is original token ids[b][i], and the scores go out indexed by original token (tokens not held: -1).
-__global__ void st3_prefill_fill_kernel(float* __restrict__ scores, long long n, float value) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) scores[i] = value;
-}
-__global__ void st3_prefill_scores_by_id_kernel(const float* __restrict__ head_probs, const int* __restrict__ ids,
-                                                float* __restrict__ scores, int* status, int num_heads, int num_visual,
-                                                int num_visual_total) {
-  const int b = blockIdx.y;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= num_visual) return;
-  const int id = ids[(size_t)b * num_visual + i];
+  if (i < num_visual) {
+    if (ids && g == 0) id = ids[(size_t)b * num_visual + i];
+    const float* src = head_probs + (size_t)b * num_heads * num_visual + i;
+#pragma unroll 4
+    for (int h = g; h < num_heads; h += kScoreGroups) s += src[(size_t)h * num_visual];
+  }
+  s_part[g][lane] = s;
+  __syncthreads();
+  if (g || i >= num_visual) return;
+#pragma unroll
+  for (int j = 1; j < kScoreGroups; ++j) s += s_part[j][lane];
   if ((unsigned)id >= (unsigned)num_visual_total) {  // reported, not used
     if (status) atomicOr(status, ST3_DEV_RANGE);
     return;
   }
-  float s = 0.f;
-  for (int h = 0; h < num_heads; ++h) s += head_probs[((size_t)b * num_heads + h) * num_visual + i];
   scores[(size_t)b * num_visual_total + id] = s;
 }
 
@@ -542,20 +557,30 @@ static st3_status prefill_attend_impl(const void* q, const void* k, const void* 
   p.head_probs = num_visual > 0 ? head_probs : nullptr;
   p.status = dev_status;
   p.T = seq_len; p.sys_len = sys_len; p.num_visual = num_visual;
-  const dim3 grid((unsigned)((seq_len + kTile - 1) / kTile), (unsigned)num_inst);
-  st3_prefill_attend_kernel<<<grid, kPfThreads, smem, st>>>(mq, mk, mv, p);
-  const int num_seq = num_inst / num_heads;
-  if (ids) {
-    const long long n = (long long)num_seq * num_visual_total;
-    st3_prefill_fill_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(scores, n, -1.f);
-    if (num_visual > 0) {
-      const dim3 g2((unsigned)((num_visual + 255) / 256), (unsigned)num_seq);
-      st3_prefill_scores_by_id_kernel<<<g2, 256, 0, st>>>(head_probs, ids, scores, dev_status, num_heads, num_visual,
-                                                          num_visual_total);
-    }
-  } else if (num_visual > 0) {
-    const dim3 g2((unsigned)((num_visual + 255) / 256), (unsigned)num_seq);
-    st3_prefill_scores_kernel<<<g2, 256, 0, st>>>(head_probs, scores, num_heads, num_visual);
+  p.fill = ids ? scores : nullptr;
+  p.fill_per_seq = num_visual_total; p.num_heads = num_heads;
+  const unsigned tiles = (unsigned)((seq_len + kTile - 1) / kTile);
+  // A grid of one wave: the longest tiles of all instances first, so that two of them share an SM only with short ones.
+  // Beyond that the tiles of an instance stay together, for its K and V to be read from L2.
+  p.tile_major = tiles * (unsigned)num_inst <= kPfWave;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = p.tile_major ? dim3((unsigned)num_inst, tiles) : dim3(tiles, (unsigned)num_inst);
+  cfg.blockDim = dim3(kPfThreads);
+  cfg.dynamicSmemBytes = kPfSmem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, st3_prefill_attend_kernel, mq, mk, mv, p) != cudaSuccess) return ST3_ERR_CUDA;
+  if (num_visual > 0) {
+    cfg.gridDim = dim3((unsigned)((num_visual + 31) / 32), (unsigned)(num_inst / num_heads));
+    cfg.blockDim = dim3(32 * kScoreGroups);
+    cfg.dynamicSmemBytes = 0;
+    if (cudaLaunchKernelEx(&cfg, st3_prefill_scores_kernel, (const float*)head_probs, ids, scores, dev_status, num_heads,
+                           num_visual, ids ? num_visual_total : num_visual) != cudaSuccess)
+      return ST3_ERR_CUDA;
   }
   return cudaGetLastError() == cudaSuccess ? ST3_OK : ST3_ERR_CUDA;
 }

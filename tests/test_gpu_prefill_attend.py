@@ -197,3 +197,40 @@ def test_unsupported_shapes_are_refused():
         B.st3_prefill_attend(x.data_ptr(), x.data_ptr(), x.data_ptr(), x.data_ptr(), None, None, None, 1, 1, 8, 64,
                              "bf16", 0, 0, 0)
     assert e.value.code == 7
+
+
+@pytest.mark.parametrize("T,one_wave", [(130, 148), (37, 296), (260, 98)])
+def test_one_wave_and_several_waves_give_the_same(T, one_wave):
+    """The largest grid of one wave runs its tiles longest first over all instances, the next larger one instance by
+    instance; what an instance computes does not depend on it."""
+    g = torch.Generator().manual_seed(T)
+    q, k, v = (torch.randn(one_wave + 1, T, 128, generator=g).to(torch.bfloat16).cuda() for _ in range(3))
+    res = []
+    for n in (one_wave, one_wave + 1):
+        out = torch.full((n, T, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+        probs, scores = torch.zeros(n, 20, device="cuda"), torch.zeros(n, 20, device="cuda")
+        B.st3_prefill_attend(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), probs.data_ptr(), scores.data_ptr(), None,
+                             n, 1, T, 128, "bf16", 3, 20, torch.cuda.current_stream().cuda_stream)
+        assert torch.equal(scores, probs)
+        res.append((out[:one_wave], scores[:one_wave]))
+    assert torch.equal(res[0][0], res[1][0]) and torch.equal(res[0][1], res[1][1])
+    p = torch.softmax((torch.einsum("nd,ntd->nt", q[:, -1].double(), k.double()) / 128 ** 0.5), dim=1)
+    assert torch.allclose(res[0][1].double(), p[:one_wave, 3:23], rtol=2e-3, atol=1e-7)
+
+
+@pytest.mark.parametrize("H,nv,total", [(9, 33, 70), (17, 32, 32), (3, 1, 4000), (2, 0, 129)])
+def test_scores_by_original_index(H, nv, total):
+    """Head counts and spans that do not fill the score kernel's groups; tokens not held read -1."""
+    T, nb, g = nv + 5, 2, torch.Generator().manual_seed(H)
+    q, k, v = (torch.randn(nb * H, T, 128, generator=g).to(torch.bfloat16).cuda() for _ in range(3))
+    ids = torch.stack([torch.randperm(total, generator=g)[:max(nv, 1)] for _ in range(nb)]).to(torch.int32).cuda()
+    out, probs = torch.empty_like(q), torch.zeros(nb * H, max(nv, 1), device="cuda")
+    scores = torch.full((nb, total), 7.0, device="cuda")
+    B.st3_prefill_attend_kept(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), probs.data_ptr(), scores.data_ptr(),
+                              None, nb * H, H, T, 128, "bf16", 2, nv, ids.data_ptr(), total,
+                              torch.cuda.current_stream().cuda_stream)
+    want = torch.full((nb, total), -1.0, dtype=torch.double, device="cuda")
+    if nv:
+        p = torch.softmax(torch.einsum("nd,ntd->nt", q[:, -1].double(), k.double()) / 128 ** 0.5, dim=1)[:, 2:2 + nv]
+        want.scatter_(1, ids.long(), p.view(nb, H, nv).sum(1))
+    assert torch.allclose(scores.double(), want, rtol=2e-3, atol=1e-7)
