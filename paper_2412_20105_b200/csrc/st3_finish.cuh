@@ -464,10 +464,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const __grid_
 constexpr int kGatherBlocks = 16;  // per (layer, sequence, head); 4, 8, 16 and 32 blocks and 1, 2 or 4 vectors in flight
                                    // per thread are within 3 % of one another on a batch, 16 or more best for one layer
 
+// It starts under the selection launch: the text rows, and the visual rows of layers that keep them all, are copied
+// without waiting for it.  What they need was complete before a block of that launch let this one start.
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads) st3_gather_kernel(const __grid_constant__ StepParams p) {
   constexpr int VPR = D * sizeof(T) / 16;
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int H = p.H, B = p.B, Nv = p.Nv;
   int y = blockIdx.y;
   const int h = y % H; y /= H;
@@ -482,27 +483,31 @@ __global__ void __launch_bounds__(kThreads) st3_gather_kernel(const __grid_const
   const uint4* srcK = reinterpret_cast<const uint4*>(p.k_in) + in0;
   const uint4* srcV = reinterpret_cast<const uint4*>(p.v_in) + in0;
   uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<T*>(p.cache) + (lb * H + h) * p.lbh_stride);
-  const int total = (n_vis + n_txt) * VPR;
+  const int total = (n_txt + n_vis) * VPR;
+  bool selected = all;  // the kept rows are known
   for (int i = blockIdx.x * kThreads + threadIdx.x; i < total; i += kGatherBlocks * kThreads) {
     const int row = i / VPR, c = i % VPR;
-    const bool vis = row < n_vis;
+    const bool vis = row >= n_txt;
     int src;  // row of the prompt
     if (vis) {
-      const int id = all ? row : ids[row];
+      if (!selected) asm volatile("griddepcontrol.wait;" ::: "memory");
+      selected = true;
+      const int id = all ? row - n_txt : ids[row - n_txt];
       if ((unsigned)id >= (unsigned)Nv) {  // a selection that failed: reported, not used
         atomicOr(p.status, ST3_DEV_RANGE);
         continue;
       }
       src = p.sys_len + id;
     } else {
-      src = row - n_vis < p.sys_len ? row - n_vis : row - n_vis + Nv;
+      src = row < p.sys_len ? row : row + Nv;
     }
     const uint4 kk = __ldg(srcK + src * VPR + c), vv = __ldg(srcV + src * VPR + c);
     // K_vis | V_vis | K_txt | V_txt
-    const long long d = vis ? i : 2LL * Nv * VPR + (i - n_vis * VPR);
+    const long long d = vis ? i - n_txt * VPR : 2LL * Nv * VPR + i;
     dst[d] = kk;
     dst[d + (long long)(vis ? Nv : p.cap_txt) * VPR] = vv;
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // this grid ends after the one ahead of it
 }
 
 }  // namespace
