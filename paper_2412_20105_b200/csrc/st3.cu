@@ -227,9 +227,11 @@ cudaError_t launch(void (*kernel)(A...), unsigned grid_x, unsigned grid_y, int t
   return cudaLaunchKernelEx(&cfg, kernel, p);
 }
 
-// prefill: the layers' prompt rows stand in p.k_in / p.v_in; select_first: prune by the caller's scores, then attend.
+// prefill: the layers' prompt rows stand in p.k_in / p.v_in; gathers: a launch copies (some of) them to the cache;
+// select_first: prune by the caller's scores, then attend.
 template <typename T, int D>
-st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, bool prefill, const StepParams* select_first) {
+st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, bool prefill, bool gathers,
+                         const StepParams* select_first) {
   const st3_config& c = ctx->cfg;
   const int units = p.layer_count * c.batch;
   const bool pdl = !ctx->profiling;  // the events between the launches want each one to end before the next begins
@@ -287,7 +289,7 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
   }
   if (e2) cudaEventRecord(e2, st);
   ctx->launches += 2;
-  if (prefill && !select_first && !gather()) return ST3_ERR_CUDA;
+  if (gathers && !select_first && !gather()) return ST3_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? ST3_OK : ST3_ERR_CUDA;
 }
 
@@ -425,6 +427,15 @@ st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, co
     p.first_dynamic = (need < full ? (need > 0 ? need : 1) : full) * kSlots;
   }
 
+  bool lazy = false, evicts = false;
+  for (int i = 0; i < layer_count; ++i) {
+    lazy = lazy || p.layer[i].lazy_src >= 0;
+    evicts = evicts || p.layer[i].ntgt < p.layer[i].ncur;
+  }
+  // The attention launch caches what it can, unless it is over after one item a ring slot: then the end of these writes
+  // would be waited for (one small fp32 layer 21.5 -> 23.5 us), and the launch that copies the kept rows is needed anyway.
+  p.store_rows = prefill && !ext_scores && !lazy && p.total_work > p.first_dynamic;
+  const bool gathers = prefill && (evicts || !p.store_rows);
   StepParams psel;
   if (ext_scores) {  // parameters of the selection-only launch: all Nv rows held, cut to the schedule
     psel = p;
@@ -435,7 +446,7 @@ st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, co
       psel.layer[i].ntgt = p.layer[i].ncur;
     }
   }
-#define ST3_LAUNCH(T, D) launch_step_t<T, D>(ctx, p, st, prefill, ext_scores ? &psel : nullptr)
+#define ST3_LAUNCH(T, D) launch_step_t<T, D>(ctx, p, st, prefill, gathers, ext_scores ? &psel : nullptr)
   const st3_status s = ST3_DISPATCH(ctx, ST3_LAUNCH);
 #undef ST3_LAUNCH
   if (s != ST3_OK) {
@@ -456,7 +467,7 @@ st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, co
   // Those logits are protected by no flag, so an attention launch that may overwrite them must not overlap this
   // call's selection: with st3_set_overlap it is launched without the programmatic attribute.
   ctx->serialize_next = reads_older;
-  ctx->rows_moving = prefill;
+  ctx->rows_moving = gathers;
   ctx->seq++;
   ctx->counter_base += (unsigned)p.total_work;  // one fetch per work item (the first of each manager is fixed)
   ctx->last_stream = st;

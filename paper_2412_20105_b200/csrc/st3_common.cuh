@@ -54,6 +54,7 @@ struct alignas(64) StepParams {
   unsigned ct_mul, ct_shift;        // fast division by ct
   int order;                // 1: the launch may start before the launch ahead of it ends, and waits before it reads inputs
   int fresh;                // 1: a new prompt, whose visual rows are the tokens 0 .. Nv-1 (ids are not read)
+  int store_rows;           // 1: a prompt's attention launch caches the rows that no selection decides
   int static_rank;          // 1: keep the kept rows in top-index order, cut them without scoring
   int seq;                  // sequence number of this step's launches
   unsigned counter_base;    // value of the work counter when this launch starts (it is never reset)

@@ -464,8 +464,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const __grid_
 constexpr int kGatherBlocks = 16;  // per (layer, sequence, head); 4, 8, 16 and 32 blocks and 1, 2 or 4 vectors in flight
                                    // per thread are within 3 % of one another on a batch, 16 or more best for one layer
 
-// It starts under the selection launch: the text rows, and the visual rows of layers that keep them all, are copied
-// without waiting for it.  What they need was complete before a block of that launch let this one start.
+// Where the attention launch has not cached them (p.store_rows), the text rows and the visual rows of layers that keep
+// them all are copied as well, under the selection launch: what they need was complete before a block of it let this
+// launch start.
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads) st3_gather_kernel(const __grid_constant__ StepParams p) {
   constexpr int VPR = D * sizeof(T) / 16;
@@ -475,9 +476,9 @@ __global__ void __launch_bounds__(kThreads) st3_gather_kernel(const __grid_const
   const int b = y % B;
   const int l_rel = y / B;
   const long long lb = (long long)(p.layer_begin + l_rel) * B + b;
-  const int n_txt = p.sys_len + __ldg(p.text_len + b);
-  const int n_vis = p.layer[l_rel].ntgt;
-  const bool all = n_vis == Nv;
+  const int n_txt = p.store_rows ? 0 : p.sys_len + __ldg(p.text_len + b);
+  const bool all = p.layer[l_rel].ntgt == Nv;
+  const int n_vis = all && p.store_rows ? 0 : p.layer[l_rel].ntgt;
   const int* ids = p.ids + lb * Nv;
   const long long in0 = (((long long)l_rel * B + b) * H + h) * p.t0_max * VPR;
   const uint4* srcK = reinterpret_cast<const uint4*>(p.k_in) + in0;

@@ -252,17 +252,22 @@ def test_free_running_against_the_oracle(name):
     assert rep["max_output_error_while_in_agreement"] <= (OUT_ABS_F32 if wl.dtype == "f32" else OUT_REL_BF16)
 
 
-@pytest.mark.parametrize("dtype,D,sys_len,text,rows,first_bp,lazy", [
-    ("bf16", 128, 0, 1, 0, 5000, 0),       # no system rows: the text chunk lies behind the visual rows
-    ("bf16", 128, 63, 2, 64, 10000, 0),    # one row past a chunk; the pruning layers keep nothing
-    ("f32", 128, 64, 64, 64, 2500, 0),     # chunks end at the break between system and text rows
-    ("bf16", 64, 33, 70, 16, 0, 0),        # chunks of several sizes across the break; everything is kept
-    ("f32", 64, 7, 20, 16, 6000, 0b1010),  # the break inside a chunk of a layer that lazy layers follow
-    ("bf16", 128, 35, 41, 0, 5000, 0b11010),
+@pytest.mark.parametrize("dtype,D,sys_len,text,rows,first_bp,lazy,heads", [
+    ("bf16", 128, 0, 1, 0, 5000, 0, 3),       # no system rows: the text chunk lies behind the visual rows
+    ("bf16", 128, 63, 2, 64, 10000, 0, 3),    # one row past a chunk; the pruning layers keep nothing
+    ("f32", 128, 64, 64, 64, 2500, 0, 3),     # chunks end at the break between system and text rows
+    ("bf16", 64, 33, 70, 16, 0, 0, 3),        # chunks of several sizes across the break; everything is kept
+    ("f32", 64, 7, 20, 16, 6000, 0b1010, 3),  # the break inside a chunk of a layer that lazy layers follow
+    ("bf16", 128, 35, 41, 0, 5000, 0b11010, 3),
+    # more items than ring slots: the attention launch caches text rows and unpruned layers itself
+    ("bf16", 128, 35, 41, 8, 5000, 0, 9),
+    ("f32", 128, 9, 70, 7, 0, 0, 7),
+    ("bf16", 64, 0, 3, 5, 10000, 0, 11),
+    ("f32", 64, 40, 33, 9, 3000, 0b1010, 13),
 ])
-def test_prompt_is_attended_in_place_and_kept_rows_are_copied(dtype, D, sys_len, text, rows, first_bp, lazy):
+def test_prompt_is_attended_in_place_and_kept_rows_are_copied(dtype, D, sys_len, text, rows, first_bp, lazy, heads):
     """The prompt's system and text rows stand on both sides of its visual rows; the cache holds them side by side."""
-    wl = get_workload("tiny").scaled(dtype=dtype, head_dim=D, num_heads=3, num_layers=5, batch=2, sys_len=sys_len,
+    wl = get_workload("tiny").scaled(dtype=dtype, head_dim=D, num_heads=heads, num_layers=5, batch=2, sys_len=sys_len,
                                      num_visual=77, text_len_min=max(1, text // 3), text_len_max=text, decode_steps=4,
                                      first_prune_layer=2, stride=5, first_ratio_bp=first_bp, tau=4.0, num_planted=7)
     stats = run_and_check(wl, 2, rows_checks=10, rows_per_chunk=rows, lazy_mask=lazy, stage_shared=int(lazy != 0))
