@@ -179,8 +179,8 @@ def path_bytes(wl, cfg, B_mod, text_len):
     written (2r), the query read and the output written (2*H*D*e), and, where the layer evicts at this step,
     one fp32 score term per head per visual row written and read back plus ids and scores ((8H+8)*n_cur) and
     the rows that close the holes read and written (2*r*d for d evicted rows, an upper bound on what hole
-    filling moves).  Prefill: the prompt rows read and written into the cache (2*r*T0), read again by the last
-    query's attention (r*T0), the same selection terms.  Partials of the split attention are scratch of this
+    filling moves).  Prefill: the prompt rows read by the last query's attention (r*T0), the rows that are kept
+    written into the cache, the same score terms.  Partials of the split attention are scratch of this
     implementation and are not counted."""
     e = 2 if wl.dtype == "bf16" else 4
     H, D = wl.num_heads, wl.head_dim
@@ -195,9 +195,9 @@ def path_bytes(wl, cfg, B_mod, text_len):
             rl, io = (r // 2, H * D * e) if l in lazy else (r, 2 * H * D * e)
             for b in range(wl.batch):
                 t_cur = wl.sys_len + n_cur + int(text_len[b]) + step
-                total += rl * t_cur + io + (2 * rl if step > 0 else 2 * rl * t_cur)
+                total += rl * t_cur + io + (2 * rl if step > 0 else rl * (t_cur - n_cur + n_tgt))
                 if n_tgt < n_cur:
-                    total += (8 * H + 8) * n_cur + 2 * rl * (n_cur - n_tgt)
+                    total += (8 * H + 8) * n_cur + (2 * rl * (n_cur - n_tgt) if step > 0 else 0)
     return total
 
 
@@ -375,7 +375,7 @@ class Job:
 
     def host_pipeline(self, n):
         """n generations through the host-buffer calls on TWO library contexts and two streams, alternating: the
-        prompt of generation g+1 crosses the bus (and is ingested and trimmed) while generation g decodes.  The
+        prompt of generation g+1 crosses the bus (and is attended and trimmed) while generation g decodes.  The
         inputs are the same pinned buffers for both; each context has its own output buffers.  Forks from and
         joins the current stream, so events around the call time all of it."""
         B, L = self.B, self.wl.num_layers
@@ -836,7 +836,7 @@ def main():
                        "api": "st3_prefill_select_host + st3_decode_step_host + st3_host_sync: pinned host buffers, "
                               "the library's two copy streams run ahead of and behind the kernels; consecutive batches "
                               "alternate between two library contexts on two streams, so that a batch's prompt is "
-                              "copied, ingested and trimmed while the batch before it decodes",
+                              "copied, attended and trimmed while the batch before it decodes",
                        "generations_timed": n_pipe,
                        "one_context": {"value": job_value(tokens_per_gen, args.steps, world, ms_one),
                                        "ms_per_step": ms_one / args.steps,

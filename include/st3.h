@@ -112,8 +112,8 @@ typedef struct {
  * ignored and its key rows are never read.  Source and lazy layer must hold the same tokens in the
  * same order: both below first_prune_layer, or both in one pruning stage with stage_shared = 1 (else
  * st3_create returns ST3_ERR_INVALID_ARG), and they must be processed in the same call (else
- * ST3_ERR_UNSUPPORTED).  In this version a lazy layer re-reads its source's keys (same bytes as a
- * normal layer); what it saves is the key cache and the key/query projections of the caller. */
+ * ST3_ERR_UNSUPPORTED).  A lazy layer's value rows are read with its source's items: it saves the
+ * key rows, and the caller its key/query projections. */
 
 /* Scheduled visual-row count n(l, t) of layer `layer` after decode step `step` (0 = after
  * prefill).  Pure host function.  PVTP: layers below first_prune_layer keep everything; layer l
@@ -131,9 +131,9 @@ st3_status st3_workspace_size(const st3_config* cfg, size_t* bytes);
  * default stream, which is synchronised before returning.  *out is NULL on failure. */
 st3_status st3_create(const st3_config* cfg, void* dev_workspace, size_t bytes, st3_ctx** out);
 
-/* Prefill half of Algorithm 3 for layers [layer_begin, layer_begin+layer_count): ingests the
- * prompt's K/V rows into the cache, attends with the last prompt token's query over the whole
- * prompt, scores the visual tokens and keeps the n(l,0) best (Eq. 3).
+/* Prefill half of Algorithm 3 for layers [layer_begin, layer_begin+layer_count): attends with the
+ * last prompt token's query over the whole prompt, where it stands, scores the visual tokens, keeps the
+ * n(l,0) best (Eq. 3) and caches their K/V rows and the text's.
  *   q_last   dev  [layer_count][B][H][D]
  *   k, v     dev  [layer_count][B][H][t0_max][D], t0_max = sys_len + num_visual + max_text_len,
  *                 rows in the order [S | V | I]; rows past a sequence's text length are ignored
@@ -194,7 +194,7 @@ st3_status st3_decode_step_host(st3_ctx* ctx, int32_t step, int32_t layer_begin,
                                 void* out_host, void* cuda_stream);
 
 /* st3_prefill_select with HOST buffers (pinned), same shapes: the prompt's K/V rows travel layer by layer
- * through two staging areas (st3_config.host_prefill = 1, else ST3_ERR_BAD_STATE), so that layer l is ingested,
+ * through two staging areas (st3_config.host_prefill = 1, else ST3_ERR_BAD_STATE), so that layer l is
  * attended and trimmed while layer l+1 is on the bus.  Same rules for the buffers as st3_decode_step_host.
  * Not available with lazy layers (a lazy layer and its source must share a call): ST3_ERR_UNSUPPORTED. */
 st3_status st3_prefill_select_host(st3_ctx* ctx, int32_t layer_begin, int32_t layer_count, const void* q_last_host,
