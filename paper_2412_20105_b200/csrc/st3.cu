@@ -279,7 +279,7 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
   if (e1) cudaEventRecord(e1, st);
   {
     // Also a programmatic dependent launch: the attention kernel allows it at its start, the blocks become
-    // resident as that grid drains and their first instruction waits for all of it.
+    // resident as that grid drains, read their parameters and wait for all of it.
     // half-size blocks, two per SM, once the units outnumber the blocks the GPU holds (see st3_finish.cuh)
     const bool half = 2 * units > 2 * ctx->num_sms && 2 * ctx->finish_smem <= 196 * 1024;
     auto kernel = half ? st3_finish_kernel<T, D, kFinishThreads / 2> : st3_finish_kernel<T, D, kFinishThreads>;
