@@ -447,6 +447,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const __grid_
     for (int j = 0; j < kMoveBatch; ++j)
       if (v0 + j * kFinishThreads < nvec) *place(v0 + j * kFinishThreads, s_hole) = val[j];
   }
+  proxy_fence();  // the next attention launch reads the moved rows with bulk copies once it sees the flag
   if (tt < nmove) ids[s_hole[tt]] = id_moved;
   for (int j = tt + kFinishThreads; j < nmove; j += kFinishThreads) ids[s_hole[j]] = ids[s_mover[j]];
   if (tt == 0) p.n_cur[lb] = k;

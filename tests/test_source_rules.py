@@ -1,0 +1,35 @@
+"""Rules of memory order that no run can show to hold, checked on the sources."""
+import os
+import re
+
+from native import HERE
+
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2412_20105_b200", "csrc")
+
+
+def _code(name):
+    """The source without comments."""
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*|/\*.*?\*/", "", f.read(), flags=re.S)
+
+
+def _body(src, head):
+    """The braces' contents of the definition that starts with `head`."""
+    i = src.index("{", src.index(head))
+    depth, j = 1, i + 1
+    while depth:
+        depth += {"{": 1, "}": -1}.get(src[j], 0)
+        j += 1
+    return src[i:j]
+
+
+def test_rows_behind_a_flag_are_fenced_between_the_proxies():
+    """The selection moves rows with ordinary stores, the attention reads them with bulk copies: a proxy fence on both
+    sides of the flag, and no look-up of a flag around it."""
+    attend, finish = _code("st3_attend.cuh"), _code("st3_finish.cuh")
+    seen = _body(attend, "bool flag_seen(")
+    assert seen.index("ld_acquire(") < seen.index("proxy_fence()")
+    assert attend.count("ld_acquire(") == 2                       # its definition and flag_seen
+    moves = finish[finish.index("kMoveBatch = 8"):]
+    assert moves.index("proxy_fence()") < moves.index("done()")
+    assert "fence.proxy.async" in _body(_code("st3_common.cuh"), "void proxy_fence(")
