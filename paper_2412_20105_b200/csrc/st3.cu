@@ -996,10 +996,10 @@ __global__ void st3_na_merge_kernel(T* __restrict__ out, int nchunk, const float
 // kNaBatch groups in flight at once, softmax relative to the warp's running maximum), the warps' results meet in
 // shared memory and the blocks' results in that of the cluster's first block.
 // One latency for the loads and one cluster barrier bound it at 7B size (32 x 675 rows).
+// Ordinary loads and no __restrict__: the launch ahead may still have been writing q, K and V when this one started.
 constexpr int kNaBatch = 8;
 template <typename T, int D>
-__global__ void __launch_bounds__(kThreads, 2) st3_na_cluster_kernel(const T* __restrict__ q, const T* __restrict__ K,
-                                                                     const T* __restrict__ V, T* __restrict__ out,
+__global__ void __launch_bounds__(kThreads, 2) st3_na_cluster_kernel(const T* q, const T* K, const T* V, T* out,
                                                                      int num_rows) {
   constexpr int EPL = 16 / sizeof(T), LPR = D / EPL, RPW = 32 / LPR;
   __shared__ float s_m[kWarps], s_l[kWarps];
@@ -1018,7 +1018,7 @@ __global__ void __launch_bounds__(kThreads, 2) st3_na_cluster_kernel(const T* __
   const uint4* gK = reinterpret_cast<const uint4*>(K + (long long)h * num_rows * D) + lir;
   const uint4* gV = reinterpret_cast<const uint4*>(V + (long long)h * num_rows * D) + lir;
   float qf[EPL];
-  unpack16(__ldg(reinterpret_cast<const uint4*>(q + (long long)h * D) + lir), qf);
+  unpack16(reinterpret_cast<const uint4*>(q + (long long)h * D)[lir], qf);
   const float sc = 1.4426950408889634f * rsqrtf((float)D);
 #pragma unroll
   for (int e = 0; e < EPL; ++e) qf[e] *= sc;
@@ -1030,7 +1030,7 @@ __global__ void __launch_bounds__(kThreads, 2) st3_na_cluster_kernel(const T* __
 #pragma unroll
     for (int u = 0; u < kNaBatch; ++u) {
       const int r = rb + u * kWarps * RPW + sub;
-      if (r < r1) { kk[u] = __ldg(gK + (long long)r * LPR); vv[u] = __ldg(gV + (long long)r * LPR); }
+      if (r < r1) { kk[u] = gK[(long long)r * LPR]; vv[u] = gV[(long long)r * LPR]; }
     }
     float s[kNaBatch], mx = m;
 #pragma unroll

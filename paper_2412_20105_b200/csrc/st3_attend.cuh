@@ -226,7 +226,7 @@ __device__ __noinline__ void issue_values(const StepParams& p, const Chain* chai
 #pragma unroll
       for (int i = 0; i < NV; ++i) {
         const int cc = (lane % LN) + i * LN;
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(src) + cc);
+        const uint4 v = reinterpret_cast<const uint4*>(src)[cc];
         reinterpret_cast<uint4*>(dstg)[cc] = v;
         *reinterpret_cast<uint4*>((j ? areaB : areaA) + (size_t)(c.nrows - 1) * ROWB + cc * 16) = v;
       }
@@ -363,13 +363,15 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       return blk + 2LL * p.Nv * D + (long long)kv * p.cap_txt * D;
     };
 
-    auto fetch_new = [&](Dec& d) {  // newest row, key and value lanes: from the step's inputs; stored when the slot is free
+    // Newest row, key and value lanes: from the step's inputs; stored when the slot is free.  Ordinary loads: the launch
+    // ahead may have been writing these when this one started, which a read-only load (__ldg) rules out.
+    auto fetch_new = [&](Dec& d) {
       if (d.has_new && lane < 2 * LN) {
         const int ls = p.layer[d.l_rel].lazy_src;
         const T* src = lane / LN ? reinterpret_cast<const T*>(p.v_new) + (long long)d.oidx * D
                                  : reinterpret_cast<const T*>(p.k_new) + (long long)(d.oidx + (ls < 0 ? 0 : ls - d.l_rel) * p.B * H) * D;
 #pragma unroll
-        for (int i = 0; i < NV; ++i) d.nv[i] = __ldg(reinterpret_cast<const uint4*>(src) + (lane % LN) + i * LN);
+        for (int i = 0; i < NV; ++i) d.nv[i] = reinterpret_cast<const uint4*>(src)[(lane % LN) + i * LN];
       }
     };
     auto decode = [&](Dec& d) {

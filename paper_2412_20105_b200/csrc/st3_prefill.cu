@@ -478,10 +478,11 @@ st3_prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
 // layer ran on the visual tokens an earlier layer kept: position i of its visual span is original token ids[b][i], and
 // the scores go out indexed by original token (tokens not held: -1, written by the attention launch ahead).
 // Eight groups of heads side by side: one or two round trips instead of one per four heads (the sum of 32 heads and its launch: 4.5 -> 2.5 us).
+// No __restrict__: the attention launch may still be writing head_probs when these blocks are set up.
 constexpr int kScoreGroups = 8;
 __global__ void __launch_bounds__(32 * kScoreGroups)
-st3_prefill_scores_kernel(const float* __restrict__ head_probs, const int* __restrict__ ids, float* __restrict__ scores,
-                          int* status, int num_heads, int num_visual, int num_visual_total) {
+st3_prefill_scores_kernel(const float* head_probs, const int* ids, float* scores, int* status, int num_heads,
+                          int num_visual, int num_visual_total) {
   __shared__ float s_part[kScoreGroups][32];
   const int b = blockIdx.y, lane = threadIdx.x & 31, g = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane;

@@ -1,0 +1,174 @@
+"""Plain stream order: every entry point whose launches start early, behind a producer that signals its completion
+before it writes, with one set of input buffers rewritten in place from call to call and nothing synchronised between."""
+import pytest
+import torch
+
+from paper_2412_20105_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+ROUNDS = 4
+
+
+def _packed(tensors):
+    """The tensors side by side in one buffer, and views of a second buffer of the same layout (stale: zeros)."""
+    offs, n = [], 0
+    for t in tensors:
+        offs.append(n)
+        n += (t.numel() * t.element_size() + 255) // 256 * 256
+    src = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    dst = torch.zeros_like(src)
+    view = lambda buf, o, t: buf[o:o + t.numel() * t.element_size()].view(t.dtype).view(t.shape)
+    for o, t in zip(offs, tensors):
+        view(src, o, t).copy_(t)
+    return src, dst, [view(dst, o, t) for o, t in zip(offs, tensors)]
+
+
+def _rows(g, *shape, dtype=torch.bfloat16):
+    return torch.randn(*shape, generator=g).to(dtype).cuda()
+
+
+def _context(dtype, heads=4, visual=300):
+    cfg = B.make_config(num_layers=2, num_heads=heads, head_dim=128, dtype=dtype, batch=2, sys_len=7, num_visual=visual,
+                        max_text_len=40, max_decode_steps=4, first_prune_layer=0, stride=1, step_ratio_bp=1000, tau=8.0)
+    return cfg, B.Context(cfg)
+
+
+def _held(ctx):
+    """What the context holds, enqueued behind the call."""
+    ids, cnt, mass = zip(*[ctx.get_kept(l) for l in range(2)])
+    rows = ctx.get_rows(1, 1, 3)
+    n = [B.st3_schedule_count(ctx.cfg, l, 0) for l in range(2)]
+    return [i[:, :k] for i, k in zip(ids, n)] + list(cnt) + list(mass) + [rows[0][:n[1]], rows[1][:n[1]],
+                                                                          rows[2][:40], rows[3][:40]]
+
+
+def _prefill(dtype, scored):
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    cfg, ctx = _context(dtype)
+    T = 7 + 300 + 40
+
+    def inputs(g):
+        kv = [_rows(g, *ctx.io_shape(), dtype=tdt)] + [_rows(g, 2, 2, 4, T, 128, dtype=tdt) for _ in range(2)]
+        return kv + ([torch.rand(2, 2, 300, generator=g).cuda()] if scored else [])
+
+    def call(t):
+        out = torch.empty_like(t[0])
+        if scored:
+            ctx.prefill_select_scored(t[0], t[1], t[2], [33, 40], t[3], out)
+        else:
+            ctx.prefill_select(t[0], t[1], t[2], [33, 40], out)
+        return [out] + _held(ctx)
+
+    return inputs, call, ctx
+
+
+def _decode(dtype, layers_per_call):
+    """Steps 1 .. ROUNDS of one generation after a prompt of fixed contents; a second run of it starts over."""
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    cfg, ctx = _context(dtype)
+    g0 = torch.Generator().manual_seed(99)
+    q, k, v = _rows(g0, *ctx.io_shape(), dtype=tdt), *(_rows(g0, 2, 2, 4, 347, 128, dtype=tdt) for _ in range(2))
+    step = [0]
+
+    def inputs(g):
+        return [_rows(g, *ctx.io_shape(), dtype=tdt) for _ in range(3)]
+
+    def call(t):
+        if step[0] == 0:
+            ctx.prefill_select(q, k, v, [33, 40], torch.empty_like(q))
+        step[0] += 1
+        out = torch.empty_like(t[0])
+        for l in range(0, 2, layers_per_call):
+            s = slice(l, l + layers_per_call)
+            ctx.decode_step(step[0], t[0][s], t[1][s], t[2][s], out[s], layer_begin=l)
+        kept = [x for l in range(2) for x in (ctx.get_kept(l)[1], ctx.get_kept(l)[2])]
+        if step[0] == ROUNDS:
+            step[0] = 0
+        return [out] + kept
+
+    return inputs, call, ctx
+
+
+def _prompt(kept):
+    H, nb, T, sys, nv, total = 6, 2, 331, 7, 290, 400
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    probs = torch.zeros(nb * H, nv, device="cuda")
+
+    def inputs(g):
+        t = [_rows(g, nb * H, T, 128) for _ in range(3)]
+        if kept:
+            t.append(torch.stack([torch.randperm(total, generator=g)[:nv] for _ in range(nb)]).to(torch.int32).cuda())
+        return t
+
+    def call(t):
+        out = torch.empty_like(t[0])
+        scores = torch.empty(nb, total if kept else nv, device="cuda")
+        st = torch.cuda.current_stream().cuda_stream
+        ptrs = [x.data_ptr() for x in (t[0], t[1], t[2], out, probs, scores, status)]
+        if kept:
+            B.st3_prefill_attend_kept(*ptrs, nb * H, H, T, 128, "bf16", sys, nv, t[3].data_ptr(), total, st)
+        else:
+            B.st3_prefill_attend(*ptrs, nb * H, H, T, 128, "bf16", sys, nv, st)
+        return [out, scores, status.clone()]
+
+    return inputs, call, None
+
+
+def _noalloc(dtype, H, T, D):
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+
+    def inputs(g):
+        return [_rows(g, H, D, dtype=tdt), _rows(g, H, T, D, dtype=tdt), _rows(g, H, T, D, dtype=tdt)]
+
+    def call(t):
+        out = torch.empty_like(t[0])
+        B.st3_attend_noalloc(t[0].data_ptr(), t[1].data_ptr(), t[2].data_ptr(), out.data_ptr(), H, T, D, dtype,
+                             torch.cuda.current_stream().cuda_stream)
+        return [out]
+
+    return inputs, call, None
+
+
+CALLS = {
+    "prefill_bf16": lambda: _prefill("bf16", False), "prefill_f32": lambda: _prefill("f32", False),
+    "scored_bf16": lambda: _prefill("bf16", True), "scored_f32": lambda: _prefill("f32", True),
+    "decode_bf16": lambda: _decode("bf16", 2), "decode_f32_layers": lambda: _decode("f32", 1),
+    "decode_bf16_layers": lambda: _decode("bf16", 1),
+    "prompt": lambda: _prompt(False), "prompt_kept": lambda: _prompt(True),
+    "noalloc_bf16": lambda: _noalloc("bf16", 32, 675, 128), "noalloc_f32": lambda: _noalloc("f32", 3, 65, 64),
+    "noalloc_long": lambda: _noalloc("bf16", 2, 8300, 128),
+}
+
+
+@pytest.mark.parametrize("name", list(CALLS))
+def test_inputs_rewritten_in_place_by_an_early_producer(name):
+    import native
+    lib = native.load()
+    inputs, call, ctx = CALLS[name]()
+    try:
+        g = torch.Generator().manual_seed(len(name))
+        sets = [_packed(inputs(g)) for _ in range(ROUNDS)]
+        want = []
+        for src, dst, views in sets:                                   # inputs in place long before the call
+            dst.copy_(src)
+            torch.cuda.synchronize()
+            want.append([x.clone() for x in call(views)])
+            torch.cuda.synchronize()
+        _, dst, views = sets[0]                                        # one set of buffers for every call
+        dst.zero_()
+        if name.startswith("noalloc"):
+            call(views)                                                # (the two-launch form looks its array up once)
+        torch.cuda.synchronize()
+        got, st = [], torch.cuda.current_stream().cuda_stream
+        for src, _, _ in sets:
+            assert lib.st3_test_early_trigger_copy(dst.data_ptr(), src.data_ptr(), src.numel() // 16, 30, st) == 0
+            got.append(call(views))
+        torch.cuda.synchronize()
+        for i, (a, b) in enumerate(zip(want, got)):
+            for j, (x, y) in enumerate(zip(a, b)):
+                assert torch.equal(x, y), (name, i, j)
+        if ctx is not None:
+            assert ctx.status() == 0
+    finally:
+        if ctx is not None:
+            ctx.close()

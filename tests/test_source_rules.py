@@ -33,3 +33,17 @@ def test_rows_behind_a_flag_are_fenced_between_the_proxies():
     moves = finish[finish.index("kMoveBatch = 8"):]
     assert moves.index("proxy_fence()") < moves.index("done()")
     assert "fence.proxy.async" in _body(_code("st3_common.cuh"), "void proxy_fence(")
+
+
+def test_launches_that_start_early_read_inputs_with_ordinary_loads():
+    """A read-only load may be moved above griddepcontrol.wait and promises that nobody writes while the kernel runs;
+    the launch ahead of one that starts early may.  What was complete before the grid can start is exempt: the text
+    lengths, and the prompt where the kept rows are copied."""
+    attend, st3, prefill = _code("st3_attend.cuh"), _code("st3.cu"), _code("st3_prefill.cu")
+    assert re.findall(r"__ldg\(([^)]*)\)", attend) == ["p.text_len + b"]
+    assert "__restrict__" not in attend + _code("st3_finish.cuh") + prefill and "__ldg" not in prefill
+    cluster = st3[st3.index("st3_na_cluster_kernel("):]
+    assert "__restrict__" not in cluster[:cluster.index("{")]
+    assert "__ldg" not in _body(st3, "st3_na_cluster_kernel(")
+    gather = _body(_code("st3_finish.cuh"), "st3_gather_kernel(")
+    assert set(re.findall(r"__ldg\((\w+)", gather)) == {"p", "srcK", "srcV"}
