@@ -641,6 +641,9 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
     }
   } else {
     // ===================== consumers =====================
+    // The limit on the waits below is for this launch's own copies, not for the work ahead of it, which may take any time
+    // after it has let this launch start.  Nothing is lost: the first query comes after that work anyway.
+    if (p.order) asm volatile("griddepcontrol.wait;" ::: "memory");
     const int grp = (warp - kSlots) / kGroupWarps;
     const int w = (warp - kSlots) % kGroupWarps;
     const int r8 = lane >> 2, c4 = lane & 3;

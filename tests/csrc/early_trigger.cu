@@ -21,9 +21,9 @@ __global__ void early_trigger_copy_kernel(uint4* __restrict__ dst, const uint4* 
 }  // namespace
 
 // Copies n16 16-byte vectors from src to dst on `stream`, delay_us microseconds after the kernel has
-// allowed its dependents to launch (delay_us <= 1000).  Returns 0 on success.
+// allowed its dependents to launch (at most four seconds).  Returns 0 on success.
 extern "C" int st3_test_early_trigger_copy(void* dst, const void* src, size_t n16, int delay_us, void* stream) {
-  if (!dst || !src || delay_us < 0 || delay_us > 1000) return 1;
+  if (!dst || !src || delay_us < 0 || delay_us > 4000000) return 1;
   early_trigger_copy_kernel<<<8, 256, 0, static_cast<cudaStream_t>(stream)>>>(
       static_cast<uint4*>(dst), static_cast<const uint4*>(src), n16, (unsigned)delay_us * 1000u);
   return cudaGetLastError() == cudaSuccess ? 0 : 2;

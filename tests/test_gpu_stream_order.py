@@ -172,3 +172,35 @@ def test_inputs_rewritten_in_place_by_an_early_producer(name):
     finally:
         if ctx is not None:
             ctx.close()
+
+
+@pytest.mark.parametrize("name", ["decode_bf16", "decode_f32_layers", "prefill_bf16", "scored_bf16", "prompt"])
+def test_a_producer_that_takes_longer_than_a_wait_may(name):
+    """The limit on a wait for a copy (4e9 cycles, about two seconds) is not spent on the caller's earlier work: a kernel
+    that lets its dependents start and writes the inputs 2.6 s later."""
+    import native
+    lib = native.load()
+    inputs, call, ctx = CALLS[name]()
+    try:
+        src, dst, views = _packed(inputs(torch.Generator().manual_seed(1)))
+        got = []
+        for delay in (0, 2600000):
+            if delay and ctx is not None:      # a context of its own for the second run
+                ctx.close()
+                inputs, call, ctx = CALLS[name]()
+            dst.zero_()
+            torch.cuda.synchronize()
+            if name.startswith("decode"):      # the prompt, and the first step
+                dst.copy_(src)
+                call(views)
+                dst.zero_()
+            st = torch.cuda.current_stream().cuda_stream
+            assert lib.st3_test_early_trigger_copy(dst.data_ptr(), src.data_ptr(), src.numel() // 16, delay, st) == 0
+            got.append([x.clone() for x in call(views)])
+            torch.cuda.synchronize()
+            if ctx is not None:
+                assert ctx.status() == 0
+        assert all(torch.equal(x, y) for x, y in zip(*got))
+    finally:
+        if ctx is not None:
+            ctx.close()

@@ -47,3 +47,13 @@ def test_launches_that_start_early_read_inputs_with_ordinary_loads():
     assert "__ldg" not in _body(st3, "st3_na_cluster_kernel(")
     gather = _body(_code("st3_finish.cuh"), "st3_gather_kernel(")
     assert set(re.findall(r"__ldg\((\w+)", gather)) == {"p", "srcK", "srcV"}
+
+
+def test_limits_on_waits_do_not_count_the_work_ahead():
+    """Whoever waits with a limit in a launch that starts early has waited for the launch ahead before."""
+    attend = _code("st3_attend.cuh")
+    roles = attend[attend.index("unsigned live = "):]
+    consumers = attend[attend.index("const int grp = (warp - kSlots)") - 400:attend.index("unsigned live = ")]
+    assert "ring_wait(" in roles and 'if (p.order) asm volatile("griddepcontrol.wait;"' in consumers
+    prompt = _body(_code("st3_prefill.cu"), "st3_prefill_attend_kernel(")
+    assert prompt.index("griddepcontrol.wait") < prompt.index("__syncthreads()") < prompt.index("pf_wait")
