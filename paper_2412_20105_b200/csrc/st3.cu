@@ -212,10 +212,10 @@ namespace {
 
 // Launches `kernel`; `programmatic`: it may be set up (and start) while the launch ahead of it is still running.
 template <typename... A>
-cudaError_t launch(void (*kernel)(A...), unsigned grid_x, unsigned grid_y, int threads, int smem, bool programmatic,
-                   cudaStream_t st, const StepParams& p) {
+cudaError_t launch(void (*kernel)(A...), dim3 grid, int threads, int smem, bool programmatic, cudaStream_t st,
+                   const StepParams& p) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid_x, grid_y);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = (size_t)smem;
   cfg.stream = st;
@@ -238,13 +238,13 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
   // the kept rows and the text go to the cache once the selection is known
   auto gather = [&]() {
     ctx->launches++;
-    return launch(st3_gather_kernel<T, D>, kGatherBlocks, (unsigned)(c.num_heads * units), kThreads, 0, pdl, st,
-                  select_first ? *select_first : p) == cudaSuccess;
+    const dim3 grid(kGatherBlocks, (unsigned)(c.num_heads * p.layer_count), (unsigned)c.batch);
+    return launch(st3_gather_kernel<T, D>, grid, kThreads, 0, pdl, st, select_first ? *select_first : p) == cudaSuccess;
   };
   if (select_first) {  // prune by the caller's scores before the layer attends
     ctx->launches++;
-    if (launch(st3_finish_kernel<T, D, kFinishThreads>, (unsigned)(2 * units), 1, kFinishThreads, ctx->finish_smem, pdl,
-               st, *select_first) != cudaSuccess || !gather())
+    if (launch(st3_finish_kernel<T, D, kFinishThreads>, (unsigned)(2 * units), kFinishThreads, ctx->finish_smem, pdl, st,
+               *select_first) != cudaSuccess || !gather())
       return ST3_ERR_CUDA;
   }
   cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr;
@@ -273,7 +273,7 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
     for (int i = 0; i < p.layer_count; ++i) fat = fat || p.layer[i].nfol != 0;
     auto kernel = direct ? (fat ? st3_attend_kernel<T, D, true, true> : st3_attend_kernel<T, D, false, true>)
                          : (fat ? st3_attend_kernel<T, D, true, false> : st3_attend_kernel<T, D, false, false>);
-    if (launch(kernel, (unsigned)(p.first_dynamic / kSlots), 1, kAttendThreads, ctx->attend_smem, early, st, p) != cudaSuccess)
+    if (launch(kernel, (unsigned)(p.first_dynamic / kSlots), kAttendThreads, ctx->attend_smem, early, st, p) != cudaSuccess)
       return ST3_ERR_CUDA;
   }
   if (e1) cudaEventRecord(e1, st);
@@ -283,7 +283,7 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
     // half-size blocks, two per SM, once the units outnumber the blocks the GPU holds (see st3_finish.cuh)
     const bool half = 2 * units > 2 * ctx->num_sms && 2 * ctx->finish_smem <= 196 * 1024;
     auto kernel = half ? st3_finish_kernel<T, D, kFinishThreads / 2> : st3_finish_kernel<T, D, kFinishThreads>;
-    if (launch(kernel, (unsigned)(2 * units), 1, half ? kFinishThreads / 2 : kFinishThreads, ctx->finish_smem, pdl, st, p) !=
+    if (launch(kernel, (unsigned)(2 * units), half ? kFinishThreads / 2 : kFinishThreads, ctx->finish_smem, pdl, st, p) !=
         cudaSuccess)
       return ST3_ERR_CUDA;
   }

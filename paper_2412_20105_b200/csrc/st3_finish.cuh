@@ -472,10 +472,8 @@ template <typename T, int D>
 __global__ void __launch_bounds__(kThreads) st3_gather_kernel(const __grid_constant__ StepParams p) {
   constexpr int VPR = D * sizeof(T) / 16;
   const int H = p.H, B = p.B, Nv = p.Nv;
-  int y = blockIdx.y;
-  const int h = y % H; y /= H;
-  const int b = y % B;
-  const int l_rel = y / B;
+  // grid (kGatherBlocks, heads x layers, sequences): all of it in y would exceed the 65535 a dimension holds
+  const int h = blockIdx.y % H, l_rel = blockIdx.y / H, b = blockIdx.z;
   const long long lb = (long long)(p.layer_begin + l_rel) * B + b;
   const int n_txt = p.store_rows ? 0 : p.sys_len + __ldg(p.text_len + b);
   const bool all = p.layer[l_rel].ntgt == Nv;

@@ -185,7 +185,7 @@ def test_rows_held_and_launch_counters_follow_the_schedule():
         assert run.ctx.rows_held() == (0, 0)
         n0 = run.ctx.launch_count()
         run.prefill()
-        assert run.ctx.launch_count() - n0 == 3                   # ingest, attend, finish
+        assert run.ctx.launch_count() - n0 == 3                   # attend, finish, gather
         sched = make_schedule(wl)
         text = run.g.text_len
         for t in range(0, 4):
@@ -434,3 +434,33 @@ def test_selection_over_hard_score_distributions(nv, keep_bp):
         assert ctx.status() == 0
     finally:
         ctx.close()
+
+
+def test_more_heads_sequences_and_layers_than_a_grid_dimension_holds():
+    """65 536 (layer, sequence, head) units in one call: 64 sequences of the same contents against one of them."""
+    L, H, D, nv, text, nb = 32, 32, 64, 8, 3, 64
+    T0 = 1 + nv + text
+    g = torch.Generator().manual_seed(12)
+    rows = lambda *s: torch.randn(*s, generator=g).to(torch.bfloat16).cuda()
+    q, K, V = rows(L, 1, H, D), rows(L, 1, H, T0, D), rows(L, 1, H, T0, D)
+    q1, k1, v1 = rows(L, 1, H, D), rows(L, 1, H, D), rows(L, 1, H, D)
+    res = []
+    for n in (1, nb):
+        cfg = B.make_config(num_layers=L, num_heads=H, head_dim=D, dtype="bf16", batch=n, sys_len=1, num_visual=nv,
+                            max_text_len=text, max_decode_steps=1, stride=7, step_ratio_bp=1000, tau=4.0)
+        ctx = B.Context(cfg)
+        try:
+            many = lambda t: t.expand(t.shape[0], n, *t.shape[2:]).contiguous()
+            out0, out1 = torch.empty_like(many(q)), torch.empty_like(many(q))
+            ctx.prefill_select(many(q), many(K), many(V), [text] * n, out0)
+            kept = [ctx.get_kept(l)[:2] for l in range(L)]
+            ctx.decode_step(1, many(q1), many(k1), many(v1), out1)
+            assert ctx.status() == 0
+            res.append((out0, out1, kept))
+        finally:
+            ctx.close()
+    (a0, a1, ka), (b0, b1, kb) = res
+    assert torch.equal(a0.expand_as(b0), b0) and torch.equal(a1.expand_as(b1), b1)
+    for (ia, ca), (ib, cb) in zip(ka, kb):
+        c = int(ca[0])
+        assert (cb == c).all() and torch.equal(ia[:, :c].expand(nb, c), ib[:, :c])
