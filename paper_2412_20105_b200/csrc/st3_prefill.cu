@@ -221,10 +221,8 @@ st3_prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
     mbar_init(&bar_p[0], 128); mbar_init(&bar_p[1], 128); mbar_init(&bar_done, 1);
     s_fail = 0;
     mbar_fence_init();
-    // This block may have been set up while the launch ahead was still running; whatever starts early behind this
-    // launch in turn finds that launch complete.
+    // This block may have been set up while the launch ahead was still running.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     mbar_expect_tx(&bar_q, kTileBytes2);
     tma_load_3d(sQ, &map_q, 0, q0, inst, &bar_q);
     tma_load_3d(sQ + kBoxBytes, &map_q, 64, q0, inst, &bar_q);
@@ -250,6 +248,9 @@ st3_prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // Only now may a launch behind this one start: it finds the launch ahead complete, and a kernel that takes tensor memory
+  // before it waits for this grid cannot take what a block of this grid still needs.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const uint32_t tmem = s_tmem;
   const uint32_t tmem_O = tmem + 128;   // S(t) lives at column 64 * (t & 1)
   volatile int* fail = &s_fail;

@@ -57,3 +57,11 @@ def test_limits_on_waits_do_not_count_the_work_ahead():
     assert "ring_wait(" in roles and 'if (p.order) asm volatile("griddepcontrol.wait;"' in consumers
     prompt = _body(_code("st3_prefill.cu"), "st3_prefill_attend_kernel(")
     assert prompt.index("griddepcontrol.wait") < prompt.index("__syncthreads()") < prompt.index("pf_wait")
+
+
+def test_tensor_memory_is_taken_before_a_successor_may_start():
+    """A successor that takes all tensor memory of an SM ahead of its own wait would otherwise keep a block of the prompt
+    attention from its share, and wait for that block."""
+    prompt = _body(_code("st3_prefill.cu"), "st3_prefill_attend_kernel(")
+    alloc = prompt.index("tcgen05.alloc")
+    assert alloc < prompt.index("__syncthreads()", alloc) < prompt.index("griddepcontrol.launch_dependents")
