@@ -64,14 +64,19 @@ __device__ __forceinline__ unsigned fast_div(unsigned n, unsigned mul, unsigned 
   return (__umulhi(n, mul) + n) >> shift;  // exact for n < 2^31 (host: make_fast_div)
 }
 // Bounded wait of a whole warp that also gives up when another role has already aborted; the
-// answer is the same in every lane.
+// answer is the same in every lane.  The limit is for this launch's own copies: it does not run while the launch ahead,
+// which may take any time after it has let this one start, holds back the inputs (abort_flag[1]).  The consumers do not
+// wait for that launch themselves: they would meet their first instructions cold after it (a 7B prompt, one call per
+// layer, 1 242 -> 1 255 us a pass).
 __device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status) {
   bool ok = mbar_try_wait(bar, parity);
   if (!ok) {
-    const long long t0 = clock64();
+    long long t0 = clock64();
     while (!(ok = mbar_try_wait(bar, parity))) {
       if (*abort_flag) break;
-      if (clock64() - t0 > kWaitCycles) {
+      if (abort_flag[1]) {
+        t0 = clock64();
+      } else if (clock64() - t0 > kWaitCycles) {
         *abort_flag = 1;
         atomicOr(status, ST3_DEV_COPY_TIMEOUT);
         break;
@@ -212,7 +217,7 @@ __device__ __noinline__ void issue_values(const StepParams& p, const Chain* chai
   // one layer of cache blocks, or of the prompt's tensor
   const size_t layer_bytes = (size_t)p.B * H * (PRE ? (size_t)p.t0_max * D : (size_t)p.lbh_stride) * sizeof(T);
   const size_t gap = PRE ? (size_t)p.Nv * ROWB : 0;
-  if (c.is_vis) {  // rows the previous step's selection may still be moving
+  if (!PRE && c.is_vis) {  // rows the previous step's selection may still be moving
     for (int j = 0; j < n; ++j)
       if (p.layer[c.l_rel + f0 + j].req &&
           !flag_wait(p.flags + c.lb + (f0 + j) * p.B, p.layer[c.l_rel + f0 + j].req, abort_flag, p.status))
@@ -293,7 +298,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
   // group's next use of the slot comes two uses later, after the manager has dealt with this one).
   __shared__ float s_stat[kSlots][kGroups][kGroupWarps][2];
   __shared__ __align__(16) float s_res[kSlots][kGroups][kGroupWarps][D];
-  __shared__ int s_abort;
+  __shared__ int s_abort[2];  // a wait ran out; the launch ahead holds back this one's inputs
 
   // The finish launch that follows may be set up while this kernel runs (its blocks take the SMs this grid's
   // blocks leave and wait there for the whole grid: no launch latency between the two kernels).
@@ -304,11 +309,12 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       for (int g = 0; g < kGroups; ++g) {
         mbar_init(&s_fullK[s][g], 1); mbar_init(&s_fullV[s][g], 1); mbar_init(&s_done[s][g], kGroupWarps);
       }
-    s_abort = 0;
+    s_abort[0] = 0;
+    s_abort[1] = p.order;
     mbar_fence_init();
   }
   __syncthreads();
-  volatile int* abort_flag = &s_abort;
+  volatile int* abort_flag = s_abort;
   const int H = p.H;
 
   if (warp < kSlots) {
@@ -343,6 +349,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
     if constexpr (PRE) {  // the prompt's rows are inputs too
       if (!inputs_ready) asm volatile("griddepcontrol.wait;" ::: "memory");
       inputs_ready = true;
+      if (lane == 0) abort_flag[1] = 0;
     }
     int wcur = 0;  // working layer of the previous visual item: this warp's items arrive in increasing order
     int lb_ready = -1;  // the (l, b) whose visual rows were last seen released by the previous finish launch
@@ -425,7 +432,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       d.want_logits = is_vis && p.layer[l_rel].ntgt < p.layer[l_rel].ncur && p.layer[l_rel].src_layer == p.layer_begin + l_rel;
       const int lb = (p.layer_begin + l_rel) * p.B + b;
       d.lb = lb;
-      d.wait_for = is_vis && lb != lb_ready ? p.layer[l_rel].req : 0;
+      d.wait_for = !PRE && is_vis && lb != lb_ready ? p.layer[l_rel].req : 0;  // no launch moves a prompt's rows
       if (d.wait_for && flag_seen(p.flags + lb, d.wait_for)) {  // looked up here, off the critical path
         d.wait_for = 0;
         lb_ready = lb;
@@ -435,7 +442,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       const int ls = p.layer[l_rel].lazy_src;
       const int lk = ls < 0 ? l_rel : ls;  // whose keys and query
       d.lazy = ls >= 0;
-      d.wait_for_k = is_vis && ls >= 0 ? p.layer[ls].req : 0;  // the source's rows as well
+      d.wait_for_k = !PRE && is_vis && ls >= 0 ? p.layer[ls].req : 0;  // the source's rows as well
       int row0 = r0;  // the chunk's first row in its source
       if constexpr (PRE) {
         const bool whole = is_vis || r0 >= p.sys_len || r0 + nrows <= p.sys_len;  // all of it on one side of the break
@@ -479,6 +486,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
         asm volatile("griddepcontrol.wait;" ::: "memory");
         inputs_ready = true;
         fetch_new(d);
+        if (lane == 0) abort_flag[1] = 0;
       }
       if (d.has_new) {
         if (lane < 2 * LN) {
@@ -641,9 +649,6 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
     }
   } else {
     // ===================== consumers =====================
-    // The limit on the waits below is for this launch's own copies, not for the work ahead of it, which may take any time
-    // after it has let this launch start.  Nothing is lost: the first query comes after that work anyway.
-    if (p.order) asm volatile("griddepcontrol.wait;" ::: "memory");
     const int grp = (warp - kSlots) / kGroupWarps;
     const int w = (warp - kSlots) % kGroupWarps;
     const int r8 = lane >> 2, c4 = lane & 3;

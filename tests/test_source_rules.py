@@ -50,11 +50,14 @@ def test_launches_that_start_early_read_inputs_with_ordinary_loads():
 
 
 def test_limits_on_waits_do_not_count_the_work_ahead():
-    """Whoever waits with a limit in a launch that starts early has waited for the launch ahead before."""
+    """In a launch that starts early a limit runs only once the launch ahead has ended: the attention kernel restarts its
+    clock until a manager has waited for that launch, the prompt attention waits for it first."""
     attend = _code("st3_attend.cuh")
-    roles = attend[attend.index("unsigned live = "):]
-    consumers = attend[attend.index("const int grp = (warp - kSlots)") - 400:attend.index("unsigned live = ")]
-    assert "ring_wait(" in roles and 'if (p.order) asm volatile("griddepcontrol.wait;"' in consumers
+    wait = _body(attend, "bool ring_wait(")
+    assert wait.index("if (abort_flag[1])") < wait.index("else if (clock64() - t0 > kWaitCycles)")
+    assert "s_abort[1] = p.order;" in attend
+    waits = [m.end() for m in re.finditer("griddepcontrol.wait", attend)]
+    assert len(waits) == 3 and all("abort_flag[1] = 0;" in attend[i:i + 200] for i in waits[:2])    # and one at the end
     prompt = _body(_code("st3_prefill.cu"), "st3_prefill_attend_kernel(")
     assert prompt.index("griddepcontrol.wait") < prompt.index("__syncthreads()") < prompt.index("pf_wait")
 
