@@ -280,8 +280,10 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
   {
     // Also a programmatic dependent launch: the attention kernel allows it at its start, the blocks become
     // resident as that grid drains, read their parameters and wait for all of it.
-    // half-size blocks, two per SM, once the units outnumber the blocks the GPU holds (see st3_finish.cuh)
-    const bool half = 2 * units > 2 * ctx->num_sms && 2 * ctx->finish_smem <= 196 * 1024;
+    // half-size blocks, two per SM, once the units outnumber the blocks the GPU holds (see st3_finish.cuh); two of them
+    // and their 11 KB of static shared memory each fit the 228 KB of an SM up to 6399 visual tokens (296 units of that many:
+    // 44.2 -> 31.6 us)
+    const bool half = 2 * units > 2 * ctx->num_sms && 2 * ctx->finish_smem <= 200 * 1024;
     auto kernel = half ? st3_finish_kernel<T, D, kFinishThreads / 2> : st3_finish_kernel<T, D, kFinishThreads>;
     if (launch(kernel, (unsigned)(2 * units), half ? kFinishThreads / 2 : kFinishThreads, ctx->finish_smem, pdl, st, p) !=
         cudaSuccess)

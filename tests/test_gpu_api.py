@@ -464,3 +464,32 @@ def test_more_heads_sequences_and_layers_than_a_grid_dimension_holds():
     for (ia, ca), (ib, cb) in zip(ka, kb):
         c = int(ca[0])
         assert (cb == c).all() and torch.equal(ia[:, :c].expand(nb, c), ib[:, :c])
+
+
+@pytest.mark.parametrize("nv,threads", [(6399, 512), (6400, 1024)])
+def test_half_size_selection_blocks_up_to_what_two_of_them_leave_of_an_sm(nv, threads):
+    """Many units: two selection blocks of 512 threads to an SM, as long as their shared memory fits twice."""
+    nb, D = 150, 64
+    cfg = B.make_config(num_layers=1, num_heads=1, head_dim=D, dtype="bf16", batch=nb, sys_len=1, num_visual=nv,
+                        max_text_len=2, max_decode_steps=1, stride=1, step_ratio_bp=0, first_prune_layer=0, tau=4.0)
+    ctx = B.Context(cfg)
+    try:
+        g = torch.Generator(device="cuda").manual_seed(nv)
+        rows = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+        q, K, V = rows(1, nb, 1, D), rows(1, nb, 1, nv + 3, D), rows(1, nb, 1, nv + 3, D)
+        out = torch.empty_like(q)
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA], acc_events=True) as prof:
+            ctx.prefill_select(q, K, V, [2] * nb, out)
+            torch.cuda.synchronize()
+        names = [e.key for e in prof.key_averages() if "st3_finish_kernel" in e.key]
+        assert len(names) == 1 and f", {threads}>" in names[0], names
+        p = torch.softmax(torch.einsum("bd,btd->bt", q[0, :, 0].double(), K[0, :, 0].double()) / D ** 0.5, dim=1)
+        ref = torch.einsum("bt,btd->bd", p, V[0, :, 0].double())
+        assert (out[0, :, 0].double() - ref).abs().max() <= 2e-2 * ref.abs().max()
+        ids, cnt, mass = ctx.get_kept(0)
+        n = nv // 2
+        assert (cnt == n).all() and ctx.status() == 0
+        cut = mass.sort(dim=1, descending=True).values[:, n - 1:n]                 # the kept are the n best
+        assert (mass.gather(1, ids[:, :n].long()) >= cut).all()
+    finally:
+        ctx.close()
