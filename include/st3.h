@@ -227,7 +227,8 @@ st3_status st3_get_status(st3_ctx* ctx, int32_t* word);
 st3_status st3_rows_held(st3_ctx* ctx, int64_t* visual_rows, int64_t* other_rows);
 
 /* Kernel timing for roofline reports.  While enabled, every prefill/decode call records CUDA
- * events around its attention kernel and around its select/compact kernel on the call's stream.
+ * events around its attention kernel and around its select/compact kernel on the call's stream; of a prompt the
+ * copy of the kept rows to the cache counts as part of the latter, as it is what compacts them.
  * st3_profile_read synchronises, returns the accumulated milliseconds and launch counts since
  * enabling (any pointer may be NULL) and clears them. */
 st3_status st3_profile_enable(st3_ctx* ctx, int32_t on);

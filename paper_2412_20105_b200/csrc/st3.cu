@@ -188,7 +188,7 @@ struct st3_ctx {
   cudaStream_t last_stream;
   int64_t launches;
   bool profiling;
-  std::vector<cudaEvent_t> ev_pool;  // triples: before attend, after attend, after finish
+  std::vector<cudaEvent_t> ev_pool;  // triples: before attend, after attend, after finish (and a prompt's gather)
   size_t ev_used;
   int attend_smem, finish_smem, num_sms, attend_ctas_per_sm;
   int seq;                     // sequence number of the next step's launches (starts at 1)
@@ -289,9 +289,9 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
         cudaSuccess)
       return ST3_ERR_CUDA;
   }
-  if (e2) cudaEventRecord(e2, st);
   ctx->launches += 2;
   if (gathers && !select_first && !gather()) return ST3_ERR_CUDA;
+  if (e2) cudaEventRecord(e2, st);  // behind the copy of a prompt's kept rows: it is part of the compaction
   return cudaGetLastError() == cudaSuccess ? ST3_OK : ST3_ERR_CUDA;
 }
 

@@ -493,3 +493,25 @@ def test_half_size_selection_blocks_up_to_what_two_of_them_leave_of_an_sm(nv, th
         assert (mass.gather(1, ids[:, :n].long()) >= cut).all()
     finally:
         ctx.close()
+
+
+def test_profile_counts_the_copy_of_a_prompts_kept_rows():
+    """The select/compact time of a prompt holds the copy of the kept rows: it is no shorter than their bytes take at
+    8 TB/s, less what the L2 cache (126 MB) may still hold of either side.  The selection alone is far shorter."""
+    L, H, nb, D, nv = 3, 32, 8, 128, 2880
+    cfg = B.make_config(num_layers=L, num_heads=H, head_dim=D, dtype="bf16", batch=nb, sys_len=4, num_visual=nv,
+                        max_text_len=4, max_decode_steps=1, stride=3, step_ratio_bp=0, first_prune_layer=0, tau=4.0)
+    ctx = B.Context(cfg)
+    try:
+        q = torch.randn(L, nb, H, D, device="cuda").to(torch.bfloat16)
+        K, V = (torch.randn(L, nb, H, nv + 8, D, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+        out = torch.empty_like(q)
+        B.st3_profile_enable(ctx.handle, True)
+        for _ in range(3):
+            ctx.prefill_select(q, K, V, [4] * nb, out)
+        _, f_ms, _, nf = B.st3_profile_read(ctx.handle)
+        moved = 2 * 2 * L * nb * H * (nv // 2) * D * 2            # K and V, read and written
+        assert nf == 3 and f_ms / nf * 1e-3 >= (moved - 2 * 126e6) / 8e12, f_ms / nf
+        assert ctx.status() == 0
+    finally:
+        ctx.close()
