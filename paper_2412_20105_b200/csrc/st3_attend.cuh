@@ -86,6 +86,15 @@ __device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity, volati
   return __all_sync(0xffffffffu, ok);
 }
 
+// After a wait ran out: a copy that is still on its way must not land in shared memory this block has given up.  Waits
+// for it, again with a limit.
+__device__ __noinline__ bool copy_settled(uint64_t* bar, uint32_t parity) {
+  const long long t0 = clock64();
+  bool ok;
+  while (!(ok = mbar_try_wait(bar, parity)) && clock64() - t0 <= kWaitCycles) {}
+  return ok;
+}
+
 // The finish launch of the previous step may still be running when this kernel starts (programmatic
 // dependent launch): visual rows of (l, b) are read only after that launch has signalled them.
 __device__ __forceinline__ int ld_acquire(const int* p) {
@@ -249,6 +258,8 @@ __device__ __noinline__ void issue_values(const StepParams& p, const Chain* chai
       } else {
         mbar_arrive(barB);
       }
+    } else {
+      mbar_arrive(barB);  // nothing for area B: its phase moves on with the use all the same
     }
     if (kb) {
       mbar_expect_tx(barA, kb);
@@ -541,7 +552,8 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
     int f0 = 0, fn = 1;    // the layers of the item this use works on: f0 .. f0+fn-1 layers above the item's own
     float M = -INFINITY, Lsum = 0.f, wgt = 0.f;  // of the item: maximum, sum, this lane's warp's weight
     int nw = 0;
-    for (int use = 0; cur_valid; ++use) {
+    int use = 0;
+    for (; cur_valid; ++use) {
       if (!have_nxt) { decode(nxt); have_nxt = true; }  // in the shadow of this item's copies and the consumers' work
       const int g = (use + s) % kGroups;
       // what follows this use: more lazy layers of the same item, or the next item
@@ -639,6 +651,11 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       }
       publish(slot0, po);
     }
+    if (cur_valid) {  // left by a wait that ran out: the copies of this use are the only ones that may not have landed
+      const int g = (use + s) % kGroups;
+      const uint32_t par = (uint32_t)use >> 1 & 1u;  // every use of a group is a phase of both its barriers
+      if (copy_settled(&s_fullK[s][g], par)) copy_settled(&s_fullV[s][g], par);
+    }
     if constexpr (PRE && !FAT) {
       if (lane == 0) bulk_written();
     }
@@ -693,7 +710,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
                                                     (phf & bitB) ? 1u : 0u, vonly, base, nrows, lane, abort_flag,
                                                     p.status);
           if (!okv) break;
-          if (vonly == 2) phf ^= bitB;
+          phf ^= bitB;
           __syncwarp();
           if (lane == 0) mbar_arrive(&s_done[s][grp]);
           continue;

@@ -515,3 +515,35 @@ def test_profile_counts_the_copy_of_a_prompts_kept_rows():
         assert ctx.status() == 0
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("lazy", [False, True])
+def test_a_wait_that_runs_out_is_reported(lazy):
+    """A flag that nothing sets: the attention launch gives up after its limit, waits for its copies in flight and ends;
+    the host reads the status, and a context of its own works as before."""
+    kw = dict(stage_shared=1, lazy_mask=0b101010) if lazy else {}
+    wl = _small(first_prune_layer=2, stride=4)
+    run, after = GpuRun(wl, **kw), GpuRun(wl, **kw)
+    try:
+        run.prefill()
+        run.decode(1)
+        words = run.ctx.workspace[run.ctx._ws_ptr - run.ctx.workspace.data_ptr():][:run.ctx.workspace_bytes // 256 * 256]
+        words = words.view(torch.int32).view(-1, 64)
+        n = wl.num_layers * wl.batch                            # one flag per (layer, sequence), 256-byte aligned
+        before = (words[:, :n] == 2).all(1)                     # the second call of the context
+        run.decode(2)
+        where = (before & (words[:, :n] == 3).all(1)).nonzero().flatten()
+        assert where.numel() == 1
+        words[where[0], :n] = -1000
+        torch.cuda.synchronize()
+        run.decode(3)
+        assert run.ctx.status(raise_on_error=False) & B.DEV_COPY_TIMEOUT
+        after.prefill()
+        for t in range(1, 4):
+            before_step = after.snapshot(range(wl.num_layers))
+            after.decode(t)
+        for l in range(wl.num_layers):
+            after.check_decode_unit(0, l, 3, before_step[l])
+        assert after.ctx.status() == 0
+    finally:
+        run.close(); after.close()

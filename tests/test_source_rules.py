@@ -68,3 +68,11 @@ def test_tensor_memory_is_taken_before_a_successor_may_start():
     prompt = _body(_code("st3_prefill.cu"), "st3_prefill_attend_kernel(")
     alloc = prompt.index("tcgen05.alloc")
     assert alloc < prompt.index("__syncthreads()", alloc) < prompt.index("griddepcontrol.launch_dependents")
+
+
+def test_a_block_that_gives_up_waits_for_its_copies():
+    attend = _code("st3_attend.cuh")
+    left = attend[attend.index("publish(slot0, po);"):attend.index("s_desc[s].info = -1;")]
+    assert "if (cur_valid) {" in left and left.count("copy_settled(") == 2 and "bulk_written()" in left
+    settled = _body(attend, "bool copy_settled(")
+    assert "kWaitCycles" in settled and "abort" not in settled
