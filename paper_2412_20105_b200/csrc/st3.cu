@@ -13,7 +13,7 @@
 //                       rows for layers that evict at this step; the newest token's row is appended
 //                       on the way.
 //   st3_finish_kernel   per (layer, sequence) one block merges the partials of every head into the
-//                       attention output and one block scores the visual rows, radix-selects the rows
+//                       attention output and one block scores the visual rows, selects the rows
 //                       to keep (ties toward the lower original index) and fills the holes among the
 //                       first n_new rows with the kept rows of the tail.
 // A prompt (prefill) is attended in the caller's tensors; a third launch, st3_gather_kernel, then copies the text and
@@ -1146,13 +1146,33 @@ st3_status na_scratch(float** ml, float** acc) {
   return ST3_OK;
 }
 
+// Blocks that share a head.  While all heads fit the GPU at once: eight, fewer for rows under 512 (32 to 128 rows a block:
+// no difference).  More heads come in waves of blocks; a wave costs the rows of a block (its keys' bytes) and about as much
+// as 48 KB of them for its start and its merge, and the cheapest power of two is taken (3, 5, 6 and 7 blocks a head pack
+// badly).  GPU us a call, always eight blocks / this rule (two launches): 128 heads of 675 rows, bf16, D = 128 21.2 / 12.6
+// (20.5); 256 of 2048 62.3 / 46.6 (60.7); 64 of 4000, fp32 44.4 / 42.1 (55.4); 1024 of 512, D = 64 124 / 37 (37).  Left
+// slower than two launches: more than 512 heads of up to 128 rows (1024 of 64, D = 64 16.9 against 12.4).
+int na_blocks(int H, int rows, int row_bytes) {
+  constexpr int kSlots = 2 * 148;  // blocks the GPU holds
+  constexpr long long kWave = 48 * 1024;
+  const int most = rows >= kNaMaxCluster * 64 ? kNaMaxCluster : ceil_div(rows, 64);
+  if ((long long)H * most <= kSlots) return most;
+  int best = 1;
+  long long cost = 0;
+  for (int n = 1; n <= most; n *= 2) {
+    const long long c = ceil_div(H * n, kSlots) * (kWave + (long long)ceil_div(rows, n) * row_bytes);
+    if (n == 1 || c < cost) { cost = c; best = n; }
+  }
+  return best;
+}
+
 template <typename T, int D>
 st3_status na_launch(const void* q, const void* k, const void* v, void* out, int H, int rows, cudaStream_t st) {
   // The one-launch form, unless a few heads of very many rows would leave most of the GPU idle: eight blocks a head keep
   // 16 heads on 128 SMs.  GPU time a call, two launches against one: 32 x 675 rows (bf16, D = 128) 17.2 / 5.6 us,
   // 40 x 1500 18.5 / 14.9, 4 x 8000 21.3 / 16.8, 64 x 8000 67.8 / 46.8; 1 x 100000 74.6 / 161.6.
   if (rows <= kNaLongRows || H >= 16) {
-    const int nblk = rows >= kNaMaxCluster * 64 ? kNaMaxCluster : ceil_div(rows, 64);  // 32 to 128 rows: no difference
+    const int nblk = na_blocks(H, rows, D * (int)sizeof(T));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)nblk, (unsigned)H);
     cfg.blockDim = dim3(kThreads);

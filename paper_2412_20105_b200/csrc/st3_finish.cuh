@@ -11,7 +11,7 @@ namespace {
 // Two blocks per (layer, sequence), on different SMs, that never wait for each other:
 //   OUT block   merges the chunk partials of every head into the attention output (a warp per head);
 //   TRIM block  merges only the (max, sum) pairs, turns the raw logits into head-summed
-//               probabilities, radix-selects the rows to keep, pairs holes with kept tail rows and
+//               probabilities, selects the rows to keep, pairs holes with kept tail rows and
 //               moves the rows.
 // Both are chains of dependent memory round trips, so every phase issues all its loads first.
 constexpr int kHeadBatch = 16;  // logits of one visual row a thread keeps in flight

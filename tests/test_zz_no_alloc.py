@@ -109,3 +109,20 @@ def test_rows_without_weight_and_a_nan():
     k[0, 5, 1] = float("nan")
     B.st3_attend_noalloc(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), H, T, D, "f32", st)
     assert torch.isnan(out[0]).all() and torch.equal(out[1], v[1, T - 1])
+
+
+# eight blocks a head and the next larger head count; four, two and one block; several waves; every type and head size
+@pytest.mark.parametrize("H,T,D,dtype", [(1, 6144, 128, "f32"), (1, 6145, 128, "f32"), (12, 8192, 128, "f32"),
+                                         (13, 6200, 128, "f32"), (37, 675, 128, "bf16"), (38, 675, 128, "bf16"),
+                                         (74, 1031, 64, "bf16"), (75, 1031, 64, "f32"), (149, 700, 128, "bf16"),
+                                         (300, 513, 64, "bf16"), (512, 129, 128, "f32"), (700, 1, 128, "bf16"),
+                                         (1185, 65, 64, "f32"), (1500, 33, 64, "bf16"), (2400, 300, 128, "bf16"),
+                                         (8192, 31, 64, "bf16"), (4096, 200, 64, "f32")])
+def test_shapes_of_the_one_launch_form(H, T, D, dtype):
+    build()
+    q, k, v = _inputs(H + T, H, T, D, dtype)
+    out = torch.full_like(q, float("nan"))
+    B.st3_attend_noalloc(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), H, T, D, dtype,
+                         torch.cuda.current_stream().cuda_stream)
+    p = torch.softmax(torch.einsum("htd,hd->ht", k.double(), q.double()) / D ** 0.5, dim=1)
+    assert_out_close(f64(out), f64(torch.einsum("ht,htd->hd", p, v.double())), dtype, f"{H} x {T}")
