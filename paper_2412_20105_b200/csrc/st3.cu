@@ -435,7 +435,7 @@ st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, co
     evicts = evicts || p.layer[i].ntgt < p.layer[i].ncur;
   }
   // The attention launch caches what it can, unless it is over after one item a ring slot: then the end of these writes
-  // would be waited for (one small fp32 layer 21.5 -> 23.5 us), and the launch that copies the kept rows is needed anyway.
+  // would be waited for (a small fp32 layer that prunes 14.7 -> 15.0 us; one that keeps all 9.0 -> 8.6), and the launch that copies the kept rows is needed anyway.
   p.store_rows = prefill && !ext_scores && !lazy && p.total_work > p.first_dynamic;
   const bool gathers = prefill && (evicts || !p.store_rows);
   StepParams psel;

@@ -278,7 +278,7 @@ __device__ __noinline__ void issue_values(const StepParams& p, const Chain* chai
 // prompt row that is not kept now crosses the memory bus once instead of three times.  Text rows, and all rows of a layer
 // that keeps them, go to the cache straight from the tile (p.store_rows; not with lazy layers, whose items are not
 // their own): read once and written once instead of read twice.  st3_prefill_select of three NeXT layers of 8 sequences
-// that keep everything 566 -> 388 us, of 32 7B layers of 8 sequences 890 -> 816, of a 13B layer of 16 101 -> 97.
+// that keep everything 559 -> 381 us, of 32 7B layers of 8 sequences 897 -> 804, of a 13B layer of 16 that prunes 96 -> 91.
 template <typename T, int D, bool FAT, bool PRE>
 __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __grid_constant__ StepParams p) {
   constexpr int EPL = 16 / sizeof(T);      // elements per 16-byte chunk

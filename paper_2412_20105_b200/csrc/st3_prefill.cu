@@ -351,8 +351,8 @@ st3_prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
       tmem_ld64(tmem_S + lane_addr, v);
       const int j0 = kt * kKeys;
       // The tile reaches past the position of the warp's first row: mask (also covers keys >= T).  Decided per warp, not
-      // per block: half the warps see the next-to-last tile whole (256.0 -> 251.5 us at 1024 x 675, 710 -> 705 at
-      // 256 x 3043, 20.6 -> 19.8 at 32 x 675).  Leaving out a warp's softmax where it sees nothing of a tile gained another
+      // per block: half the warps see the next-to-last tile whole (255.7 -> 251.6 us at 1024 x 675, 711.9 -> 705.4 at
+      // 256 x 3043, 19.1 -> 18.4 at 32 x 675).  Leaving out a warp's softmax where it sees nothing of a tile gained another
       // 1 % at 1024 x 675 and lost 1-3 % on grids that do not fill the GPU.
       if (j0 + kKeys > q0 + warp * 32 + 1) {
 #pragma unroll
