@@ -31,6 +31,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <vector>
 
@@ -190,7 +191,7 @@ struct st3_ctx {
   bool profiling;
   std::vector<cudaEvent_t> ev_pool;  // triples: before attend, after attend, after finish (and a prompt's gather)
   size_t ev_used;
-  int attend_smem, finish_smem, num_sms, attend_ctas_per_sm;
+  int attend_smem, finish_smem, stage_rows, num_sms, attend_ctas_per_sm;
   int seq;                     // sequence number of the next step's launches (starts at 1)
   unsigned counter_base;       // what the device work counter will read when the next launch starts
   std::vector<int> flag_req;   // per layer: sequence number of the last finish launch over it (0: none)
@@ -243,7 +244,7 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
   };
   if (select_first) {  // prune by the caller's scores before the layer attends
     ctx->launches++;
-    if (launch(st3_finish_kernel<T, D, kFinishThreads>, (unsigned)(2 * units), kFinishThreads, ctx->finish_smem, pdl, st,
+    if (launch(st3_finish_kernel<T, D, 1, kFinishThreads>, (unsigned)(2 * units), kFinishThreads, ctx->finish_smem, pdl, st,
                *select_first) != cudaSuccess || !gather())
       return ST3_ERR_CUDA;
   }
@@ -280,13 +281,13 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
   {
     // Also a programmatic dependent launch: the attention kernel allows it at its start, the blocks become
     // resident as that grid drains, read their parameters and wait for all of it.
-    // half-size blocks, two per SM, once the units outnumber the blocks the GPU holds (see st3_finish.cuh); two of them
-    // and their 11 KB of static shared memory each fit the 228 KB of an SM up to 6399 visual tokens (296 units of that many:
-    // 44.2 -> 31.6 us)
-    const bool half = 2 * units > 2 * ctx->num_sms && 2 * ctx->finish_smem <= 200 * 1024;
-    auto kernel = half ? st3_finish_kernel<T, D, kFinishThreads / 2> : st3_finish_kernel<T, D, kFinishThreads>;
-    if (launch(kernel, (unsigned)(2 * units), half ? kFinishThreads / 2 : kFinishThreads, ctx->finish_smem, pdl, st, p) !=
-        cudaSuccess)
+    // Two blocks per SM (with half the registers each) once the units outnumber the SMs (see st3_finish.cuh), as long as
+    // they fit: up to 6399 visual tokens; beyond, one of twice the threads.
+    const bool many = units > ctx->num_sms, two = many && 2 * ctx->finish_smem <= 200 * 1024;
+    auto kernel = two ? st3_finish_kernel<T, D, 2, kFinishThreads>
+                  : many ? st3_finish_kernel<T, D, 1, 2 * kFinishThreads> : st3_finish_kernel<T, D, 1, kFinishThreads>;
+    if (launch(kernel, (unsigned)(2 * units), many && !two ? 2 * kFinishThreads : kFinishThreads, ctx->finish_smem, pdl, st,
+               p) != cudaSuccess)
       return ST3_ERR_CUDA;
   }
   ctx->launches += 2;
@@ -301,11 +302,10 @@ st3_status set_attrs_t(st3_ctx* ctx) {
                       st3_attend_kernel<T, D, false, true>, st3_attend_kernel<T, D, true, true>})
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->attend_smem) != cudaSuccess)
       return ST3_ERR_CUDA;
-  if (cudaFuncSetAttribute(st3_finish_kernel<T, D, kFinishThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           ctx->finish_smem) != cudaSuccess ||
-      cudaFuncSetAttribute(st3_finish_kernel<T, D, kFinishThreads / 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           ctx->finish_smem) != cudaSuccess)
-    return ST3_ERR_CUDA;
+  for (auto kernel : {st3_finish_kernel<T, D, 1, kFinishThreads>, st3_finish_kernel<T, D, 2, kFinishThreads>,
+                      st3_finish_kernel<T, D, 1, 2 * kFinishThreads>})
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->finish_smem) != cudaSuccess)
+      return ST3_ERR_CUDA;
   return ST3_OK;
 }
 
@@ -343,7 +343,7 @@ st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, co
   p.lbh_stride = L.lbh_stride;
   p.layer_begin = layer_begin; p.layer_count = layer_count; p.B = c.batch; p.H = c.num_heads;
   p.sys_len = c.sys_len; p.Nv = c.num_visual; p.cap_txt = L.cap_txt; p.step = step; p.append = prefill ? 0 : 1;
-  p.static_rank = c.static_rank ? 1 : 0;
+  p.static_rank = c.static_rank ? 1 : 0; p.stage_rows = ctx->stage_rows;
   p.order = (prefill && !ext_scores) || !ctx->overlap;
   p.fresh = prefill && !ext_scores;
   p.k_in = prefill ? k : nullptr; p.v_in = prefill ? v : nullptr;
@@ -544,7 +544,15 @@ st3_status st3_create(const st3_config* cfg, void* dev_workspace, size_t bytes, 
   }
   ctx->num_sms = sms;
   ctx->attend_ctas_per_sm = tile_bytes(cfg) > 16384 ? 1 : 2;
-  ctx->finish_smem = (int)((size_t)cfg->num_visual * 16 + 16);
+  // Selection: 16 bytes a row (key, two lists), and a stage for the logits that lies over the second list: all rows if
+  // 48 KB hold them, less where two blocks with their 16 bytes a row would no longer fit an SM, at least 48 rows a head.
+  {
+    const int rows = 16 * cfg->num_visual + 16, tail = 12 * cfg->num_visual;  // the stage starts at `tail`
+    const int room = std::max(std::min(100 * 1024, tail + 48 * 1024), rows) - tail;
+    const int fit = std::max(room / (4 * cfg->num_heads) - 16, 32) / 32, all = ceil_div(std::max(cfg->num_visual, 48) - 16, 32);
+    ctx->stage_rows = 32 * std::min(fit, all) + 16;
+    ctx->finish_smem = std::max(rows, tail + 4 * cfg->num_heads * ctx->stage_rows);
+  }
   if (ctx->attend_smem > 200 * 1024 || ctx->finish_smem > 200 * 1024) { delete ctx; return ST3_ERR_UNSUPPORTED; }
 #define ST3_ATTR(T, D) set_attrs_t<T, D>(ctx)
   st3_status s = ST3_DISPATCH(ctx, ST3_ATTR);

@@ -13,7 +13,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kFinishThreads = 1024;
+constexpr int kFinishThreads = 512;  // of a selection block
 constexpr int kMaxChunkRows = 128;  // upper bound on the rows of one work item
 constexpr int kMaxLayers = 64;
 constexpr int kMaxHeads = 128;
@@ -54,6 +54,7 @@ struct alignas(64) StepParams {
   unsigned ct_mul, ct_shift;        // fast division by ct
   int order;                // 1: the launch may start before the launch ahead of it ends, and waits before it reads inputs
   int fresh;                // 1: a new prompt, whose visual rows are the tokens 0 .. Nv-1 (ids are not read)
+  int stage_rows;           // rows of one head's logits that the selection holds in shared memory at a time
   int store_rows;           // 1: a prompt's attention launch caches the rows that no selection decides
   int static_rank;          // 1: keep the kept rows in top-index order, cut them without scoring
   int seq;                  // sequence number of this step's launches
@@ -129,6 +130,12 @@ __device__ __forceinline__ float fast_exp2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+
+// 4 bytes global -> shared without a register in between; copies4_landed waits for all of the calling thread's
+__device__ __forceinline__ void copy4_async(void* dst_smem, const void* src_gmem) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst_smem)), "l"(src_gmem) : "memory");
+}
+__device__ __forceinline__ void copies4_landed() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // 16 bytes -> EPL floats
 __device__ __forceinline__ void unpack16(const uint4& v, float (&f)[8]) {  // bf16 x 8

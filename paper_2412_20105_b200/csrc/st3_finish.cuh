@@ -14,8 +14,6 @@ namespace {
 //               probabilities, selects the rows to keep, pairs holes with kept tail rows and
 //               moves the rows.
 // Both are chains of dependent memory round trips, so every phase issues all its loads first.
-constexpr int kHeadBatch = 16;  // logits of one visual row a thread keeps in flight
-
 // (max, sum) of one head's merged softmax from its chunk partials; every lane gets both, and in `w` the weights
 // exp2(max_i - max) of partials `lane` and `lane + 32`.
 __device__ __forceinline__ void merge_stats(const float2* ml, long long item0, int nit, int H, int h, int lane,
@@ -37,26 +35,25 @@ __device__ __forceinline__ void merge_stats(const float2* ml, long long item0, i
   L = warp_sum(L);
 }
 
-constexpr int kSelBins = 2048;  // bins of the selection's histogram, over the range of the scores
+constexpr int kSelBins = 256;   // bins of the selection's histogram, over the range of the scores; eight to a lane
 constexpr int kSelCand = 64;    // keys of the bin that the cut falls into that are ranked directly
 
-// NT threads per block: 1024, or 512 (two blocks per SM) when a launch has more (layer, sequence) units than the GPU
-// can hold blocks: the work of a unit is a chain of memory round trips, and more units in flight end sooner.
-template <typename T, int D, int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const __grid_constant__ StepParams p) {
+// BPS blocks of NT threads to an SM: one of 512 with 128 registers each, two of them when a launch has more (layer,
+// sequence) units than the GPU holds blocks (the work of a unit is a chain of round trips, and more units in flight end
+// sooner), or one of 1024 where two do not fit.
+template <typename T, int D, int BPS, int NT>
+__global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_constant__ StepParams p) {
   constexpr int kFinishThreads = NT, kFinishWarps = NT / 32;
   constexpr int ROWB = D * sizeof(T);
   constexpr int VPR = ROWB / 16;  // 16-byte vectors per row
   constexpr int DPL = D / 32;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ float2 s_ML[kMaxHeads];  // (max, 1/sum) of a head's merged softmax
-  __shared__ int s_hist[kSelBins];
-  __shared__ int s_scan[kFinishWarps];
+  __shared__ __align__(16) int s_hist[kSelBins];
   __shared__ unsigned s_lo[kFinishWarps], s_hi[kFinishWarps];
-  __shared__ unsigned long long s_cand[kSelCand], s_cut;
-  __shared__ int s_ncand;
-  __shared__ float s_half[kFinishThreads / 2];
-  __shared__ int s_sel[3];  // digit, count above, count in bin
+  __shared__ unsigned long long s_cand[kSelCand];
+  __shared__ int s_ncand, s_again;
+  __shared__ unsigned s_word[kMaxVisual / 32];  // a bit per row: moves (or, of a prompt, is kept)
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int B = p.B, H = p.H, Nv = p.Nv;
@@ -92,7 +89,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const __grid_
   if (out_role) {
     if (p.ext_scores) return;  // selection-only launch: nothing to merge yet
     // ===================== OUT block: attention output of every head =====================
-    constexpr int kMergeBatch = 8;  // partials in flight per round trip
+    constexpr int kMergeBatch = 8 * 1024 / (BPS * NT);  // partials in flight per round trip, as the registers allow
     for (int h = tid >> 5; h < H; h += kFinishWarps) {
       float a[kMergeBatch][DPL];
       auto load_batch = [&](int i0) {
@@ -165,41 +162,59 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const __grid_
   const long long lb_src = (long long)src * B + b;
   const float* logits = p.logits_copy[y.src_copy] + lb_src * H * Nv;
   unsigned long long* s_key = reinterpret_cast<unsigned long long*>(smem);  // [Nv]
-  int* s_hole = reinterpret_cast<int*>(smem + (size_t)Nv * 8);              // [Nv]
+  int* s_hole = reinterpret_cast<int*>(smem + (size_t)Nv * 8);              // [Nv], the ids until the scores are known
   int* s_mover = s_hole + Nv;                                               // [Nv]
   const int n_cur = n_host;
 
-  // Thread (row r, half g) of a pass sums every second batch of 16 heads of its row; half 1 hands its
-  // sum to half 0 through shared memory, so the order of the additions is fixed.  The first batch of
-  // the first pass is requested now, together with the (max, sum) pairs: one round trip for both.
-  constexpr int kRowsPerPass = kFinishThreads / 2;
-  const int ri = tt % kRowsPerPass, hg = tt / kRowsPerPass;
-  float pre[kHeadBatch];
-  int id0 = 0;
+  // The logits of all heads (as many rows as the stage holds) and the ids are requested now, together with the (max, sum)
+  // pairs: one round trip for all of them, and no registers to hold them.
   const bool own_scores = p.ext_scores == nullptr;
+  const int pitch = p.stage_rows;  // 16 (mod 32): the two halves of a warp read two heads without bank conflicts
+  float* s_log = reinterpret_cast<float*>(s_mover);  // [H][pitch]; the list of movers comes later
+  auto stage = [&](int c0) {
+    const int rows = min(pitch, n_cur - c0);
+    for (int h = warp; h < H; h += kFinishWarps)
+      for (int i = lane; i < rows; i += 32) copy4_async(s_log + h * pitch + i, logits + (h * Nv + c0 + i));
+  };
   if (own_scores) {
-    if (ri < n_cur) {
-      if (hg == 0) id0 = fresh ? ri : ids[ri];
-#pragma unroll
-      for (int j = 0; j < kHeadBatch; ++j) {
-        const int h = hg * kHeadBatch + j;
-        pre[j] = h < H ? logits[(long long)h * Nv + ri] : -INFINITY;
-      }
-    }
+    stage(0);
+    if (!fresh)
+      for (int i = tt; i < n_cur; i += kFinishThreads) copy4_async(s_hole + i, ids + i);
     if (src_here) {
-      for (int h = warp; h < H; h += kFinishWarps) {
-        float M, Lh, w[2];
-        merge_stats(ml, item0_s, nit_s, H, h, lane, M, Lh, w);
-        if (lane == 0) {
-          s_ML[h] = make_float2(M, 1.f / Lh);
-          if (src == l) { p.head_stat[2 * (lb * H + h)] = M; p.head_stat[2 * (lb * H + h) + 1] = 1.f / Lh; }
+      // (max, sum) of the heads: a warp takes eight heads, four lanes to a head
+      for (int h0 = warp * 8; h0 < H; h0 += kFinishWarps * 8) {
+        const int h = h0 + (lane & 7), part = lane >> 3;
+        constexpr int kStatBatch = 4;  // pairs of a lane in flight
+        float M = -INFINITY, L = 0.f;
+        for (int c0 = part; c0 < nit_s; c0 += 4 * kStatBatch) {
+          float2 u[kStatBatch];
+#pragma unroll
+          for (int j = 0; j < kStatBatch; ++j)
+            u[j] = h < H && c0 + 4 * j < nit_s ? ml[(item0_s + c0 + 4 * j) * H + h] : make_float2(-INFINITY, 0.f);
+          float m = M;
+#pragma unroll
+          for (int j = 0; j < kStatBatch; ++j) m = fmaxf(m, u[j].x);
+          const float ref = m > -INFINITY ? m : 0.f;  // a lane without pairs keeps zeros
+          L *= fast_exp2(M - ref);
+#pragma unroll
+          for (int j = 0; j < kStatBatch; ++j) L = fmaf(u[j].y, fast_exp2(u[j].x - ref), L);
+          M = m;
+        }
+        float m = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 8));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+        L *= fast_exp2(M - m);
+        L += __shfl_xor_sync(0xffffffffu, L, 8);
+        L += __shfl_xor_sync(0xffffffffu, L, 16);
+        if (part == 0 && h < H) {
+          const float2 st = make_float2(m, 1.f / L);
+          s_ML[h] = st;
+          if (src == l) *reinterpret_cast<float2*>(p.head_stat + 2 * (lb * H + h)) = st;
         }
       }
     } else {  // the pruning layer ran in an earlier launch of this step: its statistics were kept
-      for (int h = tt; h < H; h += kFinishThreads) {
-        s_ML[h] = make_float2(p.head_stat[2 * (lb_src * H + h)], p.head_stat[2 * (lb_src * H + h) + 1]);
-      }
+      for (int h = tt; h < H; h += kFinishThreads) s_ML[h] = *reinterpret_cast<const float2*>(p.head_stat + 2 * (lb_src * H + h));
     }
+    copies4_landed();
   }
   __syncthreads();
   if (!fresh && n_dev != n_host) {  // host bookkeeping and device state disagree: flag, do not touch
@@ -225,141 +240,123 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const __grid_
       s_key[i] = ((unsigned long long)u << 32) | (unsigned long long)(0xffffffffu - (unsigned)id);
     }
   }
-  for (int i0 = 0; own_scores && i0 < n_cur; i0 += kRowsPerPass) {
-    const int i = i0 + ri;
-    float pm = 0.f;
-    int id = id0;
-    if (i < n_cur) {
-      if (i0 && hg == 0) id = fresh ? i : ids[i];
-      for (int h0 = hg * kHeadBatch; h0 < H; h0 += 2 * kHeadBatch) {
-        float v[kHeadBatch];
-        if (i0 == 0 && h0 == hg * kHeadBatch) {
-#pragma unroll
-          for (int j = 0; j < kHeadBatch; ++j) v[j] = pre[j];
-        } else {
-#pragma unroll
-          for (int j = 0; j < kHeadBatch; ++j) v[j] = h0 + j < H ? logits[(long long)(h0 + j) * Nv + i] : -INFINITY;
-        }
-#pragma unroll
-        for (int j = 0; j < kHeadBatch; ++j)
-          if (h0 + j < H) {
-            const float2 st = s_ML[h0 + j];
-            pm += fast_exp2(v[j] - st.x) * st.y;
-          }
+  // A warp scores 16 rows a pass: lane (row r, half g) sums every second head of its row, and one shuffle adds the halves,
+  // so the order of the additions is fixed.
+  for (int c0 = 0; own_scores && c0 < n_cur; c0 += pitch) {
+    if (c0) {
+      __syncthreads();
+      stage(c0);
+      copies4_landed();
+      __syncthreads();
+    }
+    const int rows = min(pitch, n_cur - c0), g = lane >> 4;
+    for (int r0 = warp * 16; r0 < rows; r0 += kFinishWarps * 16) {
+      const int r = r0 + (lane & 15), i = c0 + r;
+      const float* at = s_log + min(r, rows - 1);
+      float mass = 0.f;
+#pragma unroll 8
+      for (int h = g; h < H; h += 2) {
+        const float2 st = s_ML[h];
+        mass += fast_exp2(at[h * pitch] - st.x) * st.y;
+      }
+      mass += __shfl_xor_sync(0xffffffffu, mass, 16);
+      if (g == 0 && r < rows) {
+        if (!(mass >= 0.f) || !(mass <= 3.0e38f)) { bad = true; mass = 0.f; }
+        const int id = fresh ? i : s_hole[i];
+        mass_by_id[id] = mass;
+        const unsigned u = __float_as_uint(mass);
+        lo = min(lo, u); hi = max(hi, u);
+        s_key[i] = ((unsigned long long)u << 32) | (unsigned long long)(0xffffffffu - (unsigned)id);
       }
     }
-    if (hg == 1) s_half[ri] = pm;
-    __syncthreads();
-    if (hg == 0 && i < n_cur) {
-      float mass = pm + s_half[ri];
-      if (!(mass >= 0.f) || !(mass <= 3.0e38f)) { bad = true; mass = 0.f; }
-      mass_by_id[id] = mass;
-      const unsigned u = __float_as_uint(mass);
-      lo = min(lo, u); hi = max(hi, u);
-      s_key[i] = ((unsigned long long)u << 32) | (unsigned long long)(0xffffffffu - (unsigned)id);
-    }
-    if (i0 + kRowsPerPass < n_cur) __syncthreads();  // s_half is written again
   }
+  if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(p.status, ST3_DEV_NONFINITE);
   lo = __reduce_min_sync(0xffffffffu, lo);
   hi = __reduce_max_sync(0xffffffffu, hi);
   if (lane == 0) { s_lo[warp] = lo; s_hi[warp] = hi; }
   __syncthreads();
-  if (bad) atomicOr(p.status, ST3_DEV_NONFINITE);
+
+  // From here on row i belongs to thread i; the warps without rows go straight to the barriers and leave the issue slots to
+  // the others.
+  const bool works = warp * 32 < n_cur;
 
   // ---- the k-th largest 64-bit key (keys are unique: ids are) ----
-  // One histogram over the range of the scores (2048 bins: a few keys in each) finds the bin of the cut, and the keys
-  // in it are ranked against one another.  Where too many share it (equal scores), a radix select over all digits.
-  unsigned long long prefix = 0ull, mask = 0ull;
-  bool found = true;
+  // A histogram over the range of the keys finds the bin of the cut, and the keys in it are ranked against one another.
+  // Where too many share it (narrow or equal scores), the same once more over that bin's range.  Every working warp
+  // derives the bin and the cut by itself.
+  unsigned long long prefix = ~0ull;  // k = 0: no key reaches this value (ids are < 2^31)
   if (k > 0) {
     lo = __reduce_min_sync(0xffffffffu, lane < kFinishWarps ? s_lo[lane] : 0xffffffffu);
     hi = __reduce_max_sync(0xffffffffu, lane < kFinishWarps ? s_hi[lane] : 0u);
-    const int sh = max(0, 32 - __clz((int)(hi - lo)) - 11);  // (hi - lo) >> sh < 2048
-    for (int i = tt; i < n_cur; i += kFinishThreads)
-      atomicAdd(&s_hist[((unsigned)(s_key[i] >> 32) - lo) >> sh], 1);
-    __syncthreads();
-    constexpr int kPer = kSelBins / kFinishThreads;  // consecutive bins of a thread
-    int c[kPer], t = 0;
-#pragma unroll
-    for (int j = 0; j < kPer; ++j) { c[j] = s_hist[tt * kPer + j]; t += c[j]; }
-    int S = t;  // inclusive suffix sum over lanes (this lane and the higher ones)
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_down_sync(0xffffffffu, S, o);
-      if (lane + o < 32) S += v;
-    }
-    if (lane == 0) s_scan[warp] = S;
-    __syncthreads();
-    int above = S - t + __reduce_add_sync(0xffffffffu, lane > warp && lane < kFinishWarps ? s_scan[lane] : 0);
-    if (above < k && k <= above + t) {
-#pragma unroll
-      for (int j = kPer - 1; j >= 0; --j) {
-        if (above + c[j] >= k) { s_sel[0] = tt * kPer + j; s_sel[1] = above; s_sel[2] = c[j]; break; }
-        above += c[j];
-      }
-    }
-    __syncthreads();
-    const unsigned digit = (unsigned)s_sel[0];
-    const int need = k - s_sel[1], inbin = s_sel[2];
-    if (need == inbin) {  // the whole bin is kept
-      prefix = (unsigned long long)(lo + (digit << sh)) << 32;
-    } else if (inbin <= kSelCand) {
-      for (int i = tt; i < n_cur; i += kFinishThreads) {
-        const unsigned long long key = s_key[i];
-        if (((unsigned)(key >> 32) - lo) >> sh == digit) s_cand[atomicAdd(&s_ncand, 1)] = key;
-      }
-      __syncthreads();
-      if (tt < inbin) {
-        const unsigned long long key = s_cand[tt];
-        int larger = 0;
-        for (int j = 0; j < inbin; ++j) larger += s_cand[j] > key;
-        if (larger == need - 1) s_cut = key;
-      }
-      __syncthreads();
-      prefix = s_cut;
-    } else {
-      found = false;
-    }
-  }
-  if (k > 0 && !found) {
+    unsigned long long base = (unsigned long long)lo << 32;  // first key of bin 0
+    int sh = 64 - 8 - __clz((int)(hi - lo)), width = 64;     // log2 of a bin's keys, of all bins' keys
     int need = k;
-    for (int shift = 56; shift >= 0; shift -= 8) {
-      if (tt < 256) s_hist[tt] = 0;
-      __syncthreads();
-      for (int i = tt; i < n_cur; i += kFinishThreads) {
-        const unsigned long long key = s_key[i];
-        if ((key & mask) == prefix) atomicAdd(&s_hist[(int)((key >> shift) & 0xffull)], 1);
-      }
-      __syncthreads();
-      if (warp == 0) {
-        int c[8], t = 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) { c[j] = s_hist[lane * 8 + j]; t += c[j]; }
-        int S = t;  // inclusive suffix sum over lanes (this lane and the higher ones)
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int v = __shfl_down_sync(0xffffffffu, S, o);
-          if (lane + o < 32) S += v;
-        }
-        int above = S - t;
-        if (above < need && need <= S) {
-#pragma unroll
-          for (int j = 7; j >= 0; --j) {
-            if (above + c[j] >= need) { s_sel[0] = lane * 8 + j; s_sel[1] = above; s_sel[2] = c[j]; break; }
-            above += c[j];
+    for (;;) {
+      auto inside = [&](unsigned long long key) { return width == 64 || (key - base) >> width == 0; };
+      if (works) {
+        for (int i = tt; i < n_cur; i += kFinishThreads) {
+          const unsigned long long key = s_key[i];
+          if (inside(key)) {
+            const unsigned d = (unsigned)((key - base) >> sh);
+            atomicAdd(&s_hist[(d & 4) * 32 + (d >> 3) * 4 + (d & 3)], 1);  // a lane's eight bins as two vectors
           }
         }
       }
       __syncthreads();
-      const int digit = s_sel[0], above = s_sel[1], inbin = s_sel[2];
-      need -= above;
-      prefix |= (unsigned long long)digit << shift;
-      mask |= 0xffull << shift;
-      if (need == inbin) break;  // the whole bin is kept: keys >= prefix are exactly the top k
+      int inbin = 0;
+      if (works) {
+        const int4 a = reinterpret_cast<const int4*>(s_hist)[lane], c4 = reinterpret_cast<const int4*>(s_hist)[32 + lane];
+        const int c[8] = {a.x, a.y, a.z, a.w, c4.x, c4.y, c4.z, c4.w};
+        const int t = c[0] + c[1] + c[2] + c[3] + c[4] + c[5] + c[6] + c[7];
+        int S = t;  // inclusive suffix sum over lanes (this lane and the higher ones)
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int x = __shfl_down_sync(0xffffffffu, S, o);
+          if (lane + o < 32) S += x;
+        }
+        int above = S - t, digit = 0, in = 0;
+        const unsigned who = __ballot_sync(0xffffffffu, above < need && need <= S);
+#pragma unroll
+        for (int j = 7; j >= 0; --j) {
+          const bool here = above < need;  // still above the cut: bin j may hold it
+          digit = here ? j : digit;
+          in = here ? c[j] : in;
+          above += here ? c[j] : 0;
+        }
+        const int from = __ffs(who) - 1;
+        digit = __shfl_sync(0xffffffffu, digit + lane * 8, from);
+        inbin = __shfl_sync(0xffffffffu, in, from);
+        need -= __shfl_sync(0xffffffffu, above - in, from);
+        base += (unsigned long long)digit << sh;
+        width = sh;
+        sh = max(0, sh - 8);
+        if (need < inbin && inbin <= kSelCand) {
+          for (int i = tt; i < n_cur; i += kFinishThreads) {
+            const unsigned long long key = s_key[i];
+            if (inside(key)) s_cand[atomicAdd(&s_ncand, 1)] = key;
+          }
+        }
+        if (tt == 0) s_again = need < inbin && inbin > kSelCand;
+      }
+      __syncthreads();
+      if (!s_again) {
+        prefix = base;  // the whole bin is kept
+        if (works && need < inbin) {
+          const unsigned long long k0 = lane < inbin ? s_cand[lane] : 0ull, k1 = lane + 32 < inbin ? s_cand[lane + 32] : 0ull;
+          int l0 = 0, l1 = 0;  // larger keys
+          for (int j = 0; j < inbin; ++j) {
+            const unsigned long long x = s_cand[j];
+            l0 += x > k0; l1 += x > k1;
+          }
+          const unsigned b0 = __ballot_sync(0xffffffffu, lane < inbin && l0 == need - 1);
+          const unsigned b1 = __ballot_sync(0xffffffffu, lane + 32 < inbin && l1 == need - 1);
+          prefix = __shfl_sync(0xffffffffu, b0 ? k0 : k1, __ffs(b0 ? b0 : b1) - 1);
+        }
+        break;
+      }
+      for (int i = tt; i < kSelBins; i += kFinishThreads) s_hist[i] = 0;
+      __syncthreads();
     }
-  }
-  if (k == 0) {
-    prefix = ~0ull;  // keep nothing (ids are < 2^31, so no key reaches this value)
   }
 
   if (fresh && p.static_rank) {
@@ -377,48 +374,49 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const __grid_
     return;
   }
 
-  // ---- pair every hole among the first k rows with a kept row of the tail ----
-  const int per = (n_cur + kFinishThreads - 1) / kFinishThreads;
-  const int i0 = min(n_cur, tt * per), i1 = min(n_cur, i0 + per);
-  int nh = 0, nm = 0;
-  for (int i = i0; i < i1; ++i) {
-    const bool keep = s_key[i] >= prefix;
-    nh += fresh ? keep : (i < k && !keep);
-    nm += !fresh && i >= k && keep;
+  // ---- pair every hole among the first k rows with a kept row of the tail (of a prompt: number the kept rows) ----
+  if (works) {
+    for (int i0 = warp * 32; i0 < n_cur; i0 += kFinishThreads) {
+      const int i = i0 + lane;
+      const bool keep = i < n_cur && s_key[i] >= prefix;
+      const unsigned word = __ballot_sync(0xffffffffu, i < n_cur && (fresh ? keep : keep != (i < k)));
+      if (lane == 0) s_word[i0 >> 5] = word;
+    }
   }
-  const int packed = nh | (nm << 16);
-  int incl = packed;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += v;
-  }
-  if (lane == 31) s_scan[warp] = incl;
   __syncthreads();
-  int wsum = lane < kFinishWarps ? s_scan[lane] : 0;  // inclusive prefix sums of the warps' totals, in every warp
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, wsum, o);
-    if (lane >= o) wsum += v;
+  const int low_words = fresh ? kMaxVisual / 32 : k >> 5;  // words of the first k rows, and the bits of the word across
+  const unsigned low_bits = (1u << (k & 31)) - 1;          // the border
+  auto low_of = [&](int x) { return x < low_words ? 0xffffffffu : x == low_words ? low_bits : 0u; };
+  auto count_before = [&](int nw) {  // bits of the words below nw: holes | movers << 16, the same in every lane
+    int c = 0;
+    for (int x = lane; x < nw; x += 32) {
+      const unsigned word = s_word[x], m = low_of(x);
+      c += __popc(word & m) | __popc(word & ~m) << 16;
+    }
+    return __reduce_add_sync(0xffffffffu, c);
+  };
+  const int total = count_before((n_cur + 31) >> 5);
+  if (works) {
+    for (int i0 = warp * 32; i0 < n_cur; i0 += kFinishThreads) {
+      const unsigned word = s_word[i0 >> 5], m = low_of(i0 >> 5);
+      if (!word) continue;
+      const int before = count_before(i0 >> 5);
+      const unsigned lt = (1u << lane) - 1;
+      if (word >> lane & 1u) {
+        const int i = i0 + lane;
+        if (fresh) ids[before + __popc(word & lt)] = i;  // the prompt's order; st3_gather_kernel copies the rows
+        else if (m >> lane & 1u) s_hole[(before & 0xffff) + __popc(word & m & lt)] = i;
+        else s_mover[(before >> 16) + __popc(word & ~m & lt)] = i;
+      }
+    }
   }
-  const int total = __shfl_sync(0xffffffffu, wsum, 31);
-  const int woff = warp ? __shfl_sync(0xffffffffu, wsum, warp - 1) : 0;
-  const int excl = woff + incl - packed;
-  int ph = excl & 0xffff, pm = excl >> 16;
-  if (fresh) {  // the kept tokens in the prompt's order; st3_gather_kernel copies the rows
-    for (int i = i0; i < i1; ++i)
-      if (s_key[i] >= prefix) ids[ph++] = i;
+  if (fresh) {
     if (tt == 0) {
       p.n_cur[lb] = k;
-      if ((total & 0xffff) != k) atomicOr(p.status, ST3_DEV_RANGE);  // cannot happen: exactly k keys pass the threshold
+      if (total != k) atomicOr(p.status, ST3_DEV_RANGE);  // cannot happen: exactly k keys pass the threshold
     }
     done();
     return;
-  }
-  for (int i = i0; i < i1; ++i) {
-    const bool keep = s_key[i] >= prefix;
-    if (i < k && !keep) s_hole[ph++] = i;
-    if (i >= k && keep) s_mover[pm++] = i;
   }
   __syncthreads();
   const int nmove = total & 0xffff;
@@ -429,27 +427,28 @@ __global__ void __launch_bounds__(NT, 1024 / NT) st3_finish_kernel(const __grid_
   }
 
   // ---- move the rows (sources are rows >= k, destinations rows < k: disjoint) ----
-  const int id_moved = tt < nmove ? ids[s_mover[tt]] : 0;  // in flight together with the rows
-  unsigned char* blk0 = reinterpret_cast<unsigned char*>(p.cache) + (size_t)(lb * H) * p.lbh_stride * sizeof(T);
-  const unsigned nvec = (unsigned)(nmove * H * 2 * VPR);
-  auto place = [&](unsigned v, const int* rows) {  // vector v of the moves: (row, head, K or V, 16 bytes of it)
-    const unsigned x = v / (2 * VPR), j = fast_div(x, p.h_mul, p.h_shift);
-    return reinterpret_cast<uint4*>(blk0 + (size_t)(x - j * H) * p.lbh_stride * sizeof(T) +
-                                    ((size_t)(v / VPR % 2) * Nv + rows[j]) * ROWB) + v % VPR;
+  // A thread's vectors are the same 16 bytes of the key or value row of one (row, head) pair after another.
+  constexpr int VPP = 2 * VPR, kPairs = kFinishThreads / VPP;  // vectors of a pair, pairs side by side
+  unsigned char* blk0 = reinterpret_cast<unsigned char*>(p.cache) + (size_t)(lb * H) * p.lbh_stride * sizeof(T) +
+                        (size_t)(tt / VPR % 2) * Nv * ROWB + tt % VPR * 16;
+  const int npair = nmove * H;
+  const size_t head_bytes = (size_t)p.lbh_stride * sizeof(T);
+  auto place = [&](int x, const int* rows) {
+    const unsigned r = fast_div((unsigned)x, p.h_mul, p.h_shift);
+    return reinterpret_cast<uint4*>(blk0 + (x - r * H) * head_bytes + rows[r] * ROWB);
   };
-  constexpr int kMoveBatch = 8;  // vectors of a thread in flight: one round trip for 8 rows of 32 heads
-  for (unsigned v0 = tt; v0 < nvec; v0 += kMoveBatch * kFinishThreads) {
+  constexpr int kMoveBatch = 8 / (BPS * NT / 512);  // vectors of a thread in flight
+  for (int x0 = tt / VPP; x0 < npair; x0 += kMoveBatch * kPairs) {
     uint4 val[kMoveBatch];
 #pragma unroll
     for (int j = 0; j < kMoveBatch; ++j)
-      if (v0 + j * kFinishThreads < nvec) val[j] = *place(v0 + j * kFinishThreads, s_mover);
+      if (x0 + j * kPairs < npair) val[j] = *place(x0 + j * kPairs, s_mover);
 #pragma unroll
     for (int j = 0; j < kMoveBatch; ++j)
-      if (v0 + j * kFinishThreads < nvec) *place(v0 + j * kFinishThreads, s_hole) = val[j];
+      if (x0 + j * kPairs < npair) *place(x0 + j * kPairs, s_hole) = val[j];
   }
   proxy_fence();  // the next attention launch reads the moved rows with bulk copies once it sees the flag
-  if (tt < nmove) ids[s_hole[tt]] = id_moved;
-  for (int j = tt + kFinishThreads; j < nmove; j += kFinishThreads) ids[s_hole[j]] = ids[s_mover[j]];
+  for (int j = tt; j < nmove; j += kFinishThreads) ids[s_hole[j]] = (int)(0xffffffffu - (unsigned)s_key[s_mover[j]]);  // the key's low word
   if (tt == 0) p.n_cur[lb] = k;
   done();
 }
