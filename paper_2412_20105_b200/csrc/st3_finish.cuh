@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ float2 s_ML[kMaxHeads];  // (max, 1/sum) of a head's merged softmax
   __shared__ __align__(16) int s_hist[kSelBins];
-  __shared__ unsigned s_lo[kFinishWarps], s_hi[kFinishWarps];
+  __shared__ unsigned s_lo, s_hi;
   __shared__ unsigned long long s_cand[kSelCand];
   __shared__ int s_ncand, s_again;
   __shared__ unsigned s_word[kMaxVisual / 32];  // a bit per row: moves (or, of a prompt, is kept)
@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
   const long long item0_s = src_here ? (long long)p.layer[src - p.layer_begin].lstart + (long long)b * nit_s : 0;
   if (!out_role) {
     for (int i = tid; i < kSelBins; i += kFinishThreads) s_hist[i] = 0;
-    if (tid == 0) s_ncand = 0;
+    if (tid == 0) { s_ncand = 0; s_lo = 0xffffffffu; s_hi = 0u; }
   }
   // The parameters a block needs are read before it waits: they are cold in the constant cache (one 7B layer a call
   // 11.07 -> 10.88 us, a small fp32 layer 10.1 -> 9.7, a 13B layer of 16 sequences 44.6 -> 43.5).
@@ -166,55 +166,67 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
   int* s_mover = s_hole + Nv;                                               // [Nv]
   const int n_cur = n_host;
 
-  // The logits of all heads (as many rows as the stage holds) and the ids are requested now, together with the (max, sum)
-  // pairs: one round trip for all of them, and no registers to hold them.
+  // The (max, sum) pairs, the logits of all heads (as many rows as the stage holds) and the ids are requested now: one round
+  // trip for all of them, and no registers to hold the logits.
   const bool own_scores = p.ext_scores == nullptr;
-  const int pitch = p.stage_rows;  // 16 (mod 32): the two halves of a warp read two heads without bank conflicts
-  float* s_log = reinterpret_cast<float*>(s_mover);  // [H][pitch]; the list of movers comes later
+  const int pitch = p.stage_rows;  // 16 (mod 32): a quarter of a warp reads two heads without bank conflicts
+  float* s_log = reinterpret_cast<float*>(smem + ((size_t)Nv * 12 + 15) / 16 * 16);  // [H][pitch], over the list of movers
   auto stage = [&](int c0) {
     const int rows = min(pitch, n_cur - c0);
-    for (int h = warp; h < H; h += kFinishWarps)
-      for (int i = lane; i < rows; i += 32) copy4_async(s_log + h * pitch + i, logits + (h * Nv + c0 + i));
+    if (Nv % 4 == 0) {  // every head's logits start on 16 bytes
+      for (int h = warp; h < H; h += kFinishWarps)
+        for (int i = 4 * lane; i < rows; i += 128) copy_async<16>(s_log + h * pitch + i, logits + (h * Nv + c0 + i));
+    } else {
+      for (int h = warp; h < H; h += kFinishWarps)
+        for (int i = lane; i < rows; i += 32) copy_async<4>(s_log + h * pitch + i, logits + (h * Nv + c0 + i));
+    }
   };
   if (own_scores) {
+    // (max, sum) of the heads: a warp takes eight heads, four lanes to a head
+    constexpr int kStatBatch = 4;  // pairs of a lane in flight
+    static_assert(kFinishWarps * 8 >= kMaxHeads, "one pass over the heads");
+    const int h = warp * 8 + (lane & 7), part = lane >> 3;
+    const bool merges = src_here && warp * 8 < H;
+    float2 u[kStatBatch];
+    auto load_pairs = [&](int c0) {
+#pragma unroll
+      for (int j = 0; j < kStatBatch; ++j)
+        u[j] = h < H && c0 + 4 * j < nit_s ? ml[(item0_s + c0 + 4 * j) * H + h] : make_float2(-INFINITY, 0.f);
+    };
+    if (merges) load_pairs(part);
     stage(0);
     if (!fresh)
-      for (int i = tt; i < n_cur; i += kFinishThreads) copy4_async(s_hole + i, ids + i);
-    if (src_here) {
-      // (max, sum) of the heads: a warp takes eight heads, four lanes to a head
-      for (int h0 = warp * 8; h0 < H; h0 += kFinishWarps * 8) {
-        const int h = h0 + (lane & 7), part = lane >> 3;
-        constexpr int kStatBatch = 4;  // pairs of a lane in flight
-        float M = -INFINITY, L = 0.f;
-        for (int c0 = part; c0 < nit_s; c0 += 4 * kStatBatch) {
-          float2 u[kStatBatch];
+      for (int i = tt; i < n_cur; i += kFinishThreads) copy_async<4>(s_hole + i, ids + i);
+    if (merges) {
+      float M = -INFINITY, L = 0.f;
+      for (int c0 = part;;) {
+        float m = M;
 #pragma unroll
-          for (int j = 0; j < kStatBatch; ++j)
-            u[j] = h < H && c0 + 4 * j < nit_s ? ml[(item0_s + c0 + 4 * j) * H + h] : make_float2(-INFINITY, 0.f);
-          float m = M;
+        for (int j = 0; j < kStatBatch; ++j) m = fmaxf(m, u[j].x);
+        const float ref = m > -INFINITY ? m : 0.f;  // a lane without pairs keeps zeros
+        L *= fast_exp2(M - ref);
 #pragma unroll
-          for (int j = 0; j < kStatBatch; ++j) m = fmaxf(m, u[j].x);
-          const float ref = m > -INFINITY ? m : 0.f;  // a lane without pairs keeps zeros
-          L *= fast_exp2(M - ref);
-#pragma unroll
-          for (int j = 0; j < kStatBatch; ++j) L = fmaf(u[j].y, fast_exp2(u[j].x - ref), L);
-          M = m;
-        }
-        float m = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 8));
-        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
-        L *= fast_exp2(M - m);
-        L += __shfl_xor_sync(0xffffffffu, L, 8);
-        L += __shfl_xor_sync(0xffffffffu, L, 16);
-        if (part == 0 && h < H) {
-          const float2 st = make_float2(m, 1.f / L);
-          s_ML[h] = st;
-          if (src == l) *reinterpret_cast<float2*>(p.head_stat + 2 * (lb * H + h)) = st;
-        }
+        for (int j = 0; j < kStatBatch; ++j) L = fmaf(u[j].y, fast_exp2(u[j].x - ref), L);
+        M = m;
+        c0 += 4 * kStatBatch;
+        if (c0 >= nit_s) break;
+        load_pairs(c0);
       }
-    } else {  // the pruning layer ran in an earlier launch of this step: its statistics were kept
-      for (int h = tt; h < H; h += kFinishThreads) s_ML[h] = *reinterpret_cast<const float2*>(p.head_stat + 2 * (lb_src * H + h));
+      __syncwarp();
+      float m = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 8));
+      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+      L *= fast_exp2(M - m);
+      L += __shfl_xor_sync(0xffffffffu, L, 8);
+      L += __shfl_xor_sync(0xffffffffu, L, 16);
+      if (part == 0 && h < H) {
+        const float2 st = make_float2(m, 1.f / L);
+        s_ML[h] = st;
+        if (src == l) *reinterpret_cast<float2*>(p.head_stat + 2 * (lb * H + h)) = st;
+      }
+    } else if (!src_here) {  // the pruning layer ran in an earlier launch of this step: its statistics were kept
+      for (int i = tt; i < H; i += kFinishThreads) s_ML[i] = *reinterpret_cast<const float2*>(p.head_stat + 2 * (lb_src * H + i));
     }
-    copies4_landed();
+    copies_landed();
   }
   __syncthreads();
   if (!fresh && n_dev != n_host) {  // host bookkeeping and device state disagree: flag, do not touch
@@ -240,27 +252,37 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
       s_key[i] = ((unsigned long long)u << 32) | (unsigned long long)(0xffffffffu - (unsigned)id);
     }
   }
-  // A warp scores 16 rows a pass: lane (row r, half g) sums every second head of its row, and one shuffle adds the halves,
-  // so the order of the additions is fixed.
+  // A warp scores 16 rows a pass: lane (four rows, group g) sums every eighth head of its rows, and the groups' sums meet in
+  // four shuffles that leave a lane with one row: a fixed order of additions, and a third of the shared-memory reads that a
+  // row per lane takes (1 540 -> 700 cycles for 288 rows of 32 heads).
   for (int c0 = 0; own_scores && c0 < n_cur; c0 += pitch) {
     if (c0) {
       __syncthreads();
       stage(c0);
-      copies4_landed();
+      copies_landed();
       __syncthreads();
     }
-    const int rows = min(pitch, n_cur - c0), g = lane >> 4;
+    const int rows = min(pitch, n_cur - c0), g = lane >> 2;
     for (int r0 = warp * 16; r0 < rows; r0 += kFinishWarps * 16) {
-      const int r = r0 + (lane & 15), i = c0 + r;
-      const float* at = s_log + min(r, rows - 1);
-      float mass = 0.f;
-#pragma unroll 8
-      for (int h = g; h < H; h += 2) {
+      const float* at = s_log + min(r0 + (lane & 3) * 4, (rows - 1) & ~3);
+      float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll 4
+      for (int h = g; h < H; h += 8) {
         const float2 st = s_ML[h];
-        mass += fast_exp2(at[h * pitch] - st.x) * st.y;
+        const float4 x = *reinterpret_cast<const float4*>(at + h * pitch);
+        a0 += fast_exp2(x.x - st.x) * st.y;
+        a1 += fast_exp2(x.y - st.x) * st.y;
+        a2 += fast_exp2(x.z - st.x) * st.y;
+        a3 += fast_exp2(x.w - st.x) * st.y;
       }
-      mass += __shfl_xor_sync(0xffffffffu, mass, 16);
-      if (g == 0 && r < rows) {
+      __syncwarp();
+      const bool up = lane & 16, odd = lane & 8;
+      const float b0 = (up ? a2 : a0) + __shfl_xor_sync(0xffffffffu, up ? a0 : a2, 16);
+      const float b1 = (up ? a3 : a1) + __shfl_xor_sync(0xffffffffu, up ? a1 : a3, 16);
+      float mass = (odd ? b1 : b0) + __shfl_xor_sync(0xffffffffu, odd ? b0 : b1, 8);
+      mass += __shfl_xor_sync(0xffffffffu, mass, 4);
+      const int r = r0 + (lane & 3) * 4 + (up ? 2 : 0) + (odd ? 1 : 0), i = c0 + r;
+      if (!(lane & 4) && r < rows) {
         if (!(mass >= 0.f) || !(mass <= 3.0e38f)) { bad = true; mass = 0.f; }
         const int id = fresh ? i : s_hole[i];
         mass_by_id[id] = mass;
@@ -273,7 +295,7 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(p.status, ST3_DEV_NONFINITE);
   lo = __reduce_min_sync(0xffffffffu, lo);
   hi = __reduce_max_sync(0xffffffffu, hi);
-  if (lane == 0) { s_lo[warp] = lo; s_hi[warp] = hi; }
+  if (lane == 0) { atomicMin(&s_lo, lo); atomicMax(&s_hi, hi); }
   __syncthreads();
 
   // From here on row i belongs to thread i; the warps without rows go straight to the barriers and leave the issue slots to
@@ -286,47 +308,47 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
   // derives the bin and the cut by itself.
   unsigned long long prefix = ~0ull;  // k = 0: no key reaches this value (ids are < 2^31)
   if (k > 0) {
-    lo = __reduce_min_sync(0xffffffffu, lane < kFinishWarps ? s_lo[lane] : 0xffffffffu);
-    hi = __reduce_max_sync(0xffffffffu, lane < kFinishWarps ? s_hi[lane] : 0u);
+    lo = s_lo;
     unsigned long long base = (unsigned long long)lo << 32;  // first key of bin 0
-    int sh = 64 - 8 - __clz((int)(hi - lo)), width = 64;     // log2 of a bin's keys, of all bins' keys
-    int need = k;
+    int sh = 32 + max(0, 24 - __clz((int)(s_hi - lo)));      // log2 of a bin's keys: the high words make 256 bins
+    int width = 64, need = k;                                // log2 of all bins' keys; how many of them are kept
     for (;;) {
       auto inside = [&](unsigned long long key) { return width == 64 || (key - base) >> width == 0; };
       if (works) {
         for (int i = tt; i < n_cur; i += kFinishThreads) {
           const unsigned long long key = s_key[i];
-          if (inside(key)) {
-            const unsigned d = (unsigned)((key - base) >> sh);
-            atomicAdd(&s_hist[(d & 4) * 32 + (d >> 3) * 4 + (d & 3)], 1);  // a lane's eight bins as two vectors
-          }
+          const unsigned d = width == 64 ? ((unsigned)(key >> 32) - lo) >> (sh - 32) : (unsigned)((key - base) >> sh);
+          if (inside(key)) atomicAdd(&s_hist[(d & 4) * 32 + (d >> 3) * 4 + (d & 3)], 1);  // a lane's bins as two vectors
         }
       }
       __syncthreads();
       int inbin = 0;
       if (works) {
         const int4 a = reinterpret_cast<const int4*>(s_hist)[lane], c4 = reinterpret_cast<const int4*>(s_hist)[32 + lane];
-        const int c[8] = {a.x, a.y, a.z, a.w, c4.x, c4.y, c4.z, c4.w};
-        const int t = c[0] + c[1] + c[2] + c[3] + c[4] + c[5] + c[6] + c[7];
-        int S = t;  // inclusive suffix sum over lanes (this lane and the higher ones)
+        // keys of this lane's bins j and above (and none: f[8])
+        const int f7 = c4.w, f6 = f7 + c4.z, f5 = f6 + c4.y, f4 = f5 + c4.x, f3 = f4 + a.w, f2 = f3 + a.z, f1 = f2 + a.y, f0 = f1 + a.x;
+        int S = f0;  // inclusive suffix sum over lanes (this lane and the higher ones)
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
           const int x = __shfl_down_sync(0xffffffffu, S, o);
           if (lane + o < 32) S += x;
         }
-        int above = S - t, digit = 0, in = 0;
-        const unsigned who = __ballot_sync(0xffffffffu, above < need && need <= S);
+        const int want = need - (S - f0);  // of this lane's bins
+        const unsigned who = __ballot_sync(0xffffffffu, 0 < want && want <= f0);
+        // the highest bin j with want <= f[j]
+        const int f[9] = {f0, f1, f2, f3, f4, f5, f6, f7, 0};
+        int digit = -1, upto = f0, above = 0;
 #pragma unroll
-        for (int j = 7; j >= 0; --j) {
-          const bool here = above < need;  // still above the cut: bin j may hold it
-          digit = here ? j : digit;
-          in = here ? c[j] : in;
-          above += here ? c[j] : 0;
+        for (int j = 0; j < 8; ++j) {
+          digit += want <= f[j];
+          upto = want <= f[j] ? f[j] : upto;
         }
+#pragma unroll
+        for (int j = 8; j >= 1; --j) above = want > f[j] ? f[j] : above;
         const int from = __ffs(who) - 1;
         digit = __shfl_sync(0xffffffffu, digit + lane * 8, from);
-        inbin = __shfl_sync(0xffffffffu, in, from);
-        need -= __shfl_sync(0xffffffffu, above - in, from);
+        inbin = __shfl_sync(0xffffffffu, upto - above, from);
+        need = __shfl_sync(0xffffffffu, want - above, from);
         base += (unsigned long long)digit << sh;
         width = sh;
         sh = max(0, sh - 8);
@@ -387,27 +409,24 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
   const int low_words = fresh ? kMaxVisual / 32 : k >> 5;  // words of the first k rows, and the bits of the word across
   const unsigned low_bits = (1u << (k & 31)) - 1;          // the border
   auto low_of = [&](int x) { return x < low_words ? 0xffffffffu : x == low_words ? low_bits : 0u; };
-  auto count_before = [&](int nw) {  // bits of the words below nw: holes | movers << 16, the same in every lane
-    int c = 0;
-    for (int x = lane; x < nw; x += 32) {
+  const int nwords = (n_cur + 31) >> 5;
+  int total = 0;  // set bits: holes | movers << 16
+  for (int w0 = warp; w0 == warp || w0 < nwords; w0 += kFinishWarps) {
+    int all = 0, before = 0;  // of all words, and of the words below w0
+    for (int x = lane; x < nwords; x += 32) {
       const unsigned word = s_word[x], m = low_of(x);
-      c += __popc(word & m) | __popc(word & ~m) << 16;
+      const int c = __popc(word & m) | __popc(word & ~m) << 16;
+      all += c;
+      before += x < w0 ? c : 0;
     }
-    return __reduce_add_sync(0xffffffffu, c);
-  };
-  const int total = count_before((n_cur + 31) >> 5);
-  if (works) {
-    for (int i0 = warp * 32; i0 < n_cur; i0 += kFinishThreads) {
-      const unsigned word = s_word[i0 >> 5], m = low_of(i0 >> 5);
-      if (!word) continue;
-      const int before = count_before(i0 >> 5);
-      const unsigned lt = (1u << lane) - 1;
-      if (word >> lane & 1u) {
-        const int i = i0 + lane;
-        if (fresh) ids[before + __popc(word & lt)] = i;  // the prompt's order; st3_gather_kernel copies the rows
-        else if (m >> lane & 1u) s_hole[(before & 0xffff) + __popc(word & m & lt)] = i;
-        else s_mover[(before >> 16) + __popc(word & ~m & lt)] = i;
-      }
+    total = __reduce_add_sync(0xffffffffu, all);
+    before = __reduce_add_sync(0xffffffffu, before);
+    const unsigned word = w0 < nwords ? s_word[w0] : 0u, m = low_of(w0), lt = (1u << lane) - 1;
+    if (word >> lane & 1u) {
+      const int i = w0 * 32 + lane;
+      if (fresh) ids[before + __popc(word & lt)] = i;  // the prompt's order; st3_gather_kernel copies the rows
+      else if (m >> lane & 1u) s_hole[(before & 0xffff) + __popc(word & m & lt)] = i;
+      else s_mover[(before >> 16) + __popc(word & ~m & lt)] = i;
     }
   }
   if (fresh) {
@@ -443,12 +462,13 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
 #pragma unroll
     for (int j = 0; j < kMoveBatch; ++j)
       if (x0 + j * kPairs < npair) val[j] = *place(x0 + j * kPairs, s_mover);
+    if (x0 == tt / VPP)  // under the loads: the ids, each the low word of its key
+      for (int j = tt; j < nmove; j += kFinishThreads) ids[s_hole[j]] = (int)(0xffffffffu - (unsigned)s_key[s_mover[j]]);
 #pragma unroll
     for (int j = 0; j < kMoveBatch; ++j)
       if (x0 + j * kPairs < npair) *place(x0 + j * kPairs, s_hole) = val[j];
   }
   proxy_fence();  // the next attention launch reads the moved rows with bulk copies once it sees the flag
-  for (int j = tt; j < nmove; j += kFinishThreads) ids[s_hole[j]] = (int)(0xffffffffu - (unsigned)s_key[s_mover[j]]);  // the key's low word
   if (tt == 0) p.n_cur[lb] = k;
   done();
 }
