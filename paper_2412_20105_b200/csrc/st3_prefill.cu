@@ -176,6 +176,7 @@ struct PrefillParams {
   int fill_per_seq, num_heads;
   int T, sys_len, num_visual;
   int tile_major;       // grid (instance, tile) instead of (tile, instance)
+  int wide_out;         // out is aligned to 32 bytes
 };
 
 __global__ void __launch_bounds__(kPfThreads, 2)
@@ -445,6 +446,9 @@ st3_prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
       for (int i = tid; i < p.num_visual; i += 128) probs[i] = fast_exp2(probs[i] - rl) * il;
     }
     // ---- O / sum -> bf16 -> global ----
+    // A thread owns a row, so every store of a warp touches 32 rows: whole 32-byte sectors where the output allows it (half
+    // the store instructions, no sector written twice; 1024 x 675 positions 259 -> 247 us, 256 x 3043 in four layers 3.73
+    // -> 3.70 ms), 16 bytes otherwise.
     if (ok) {
       tc_fence_after();
       __nv_bfloat16* orow = p.out + ((size_t)row_base + qi) * kPfD;
@@ -453,16 +457,22 @@ st3_prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
         uint32_t v[32];
         tmem_ld32(tmem_O + lane_addr + cb * 32, v);
         if (live) {
+          uint32_t w[16];
 #pragma unroll
-          for (int c = 0; c < 32; c += 8) {
-            uint32_t w[4];
+          for (int e = 0; e < 16; ++e) {
+            const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(v[2 * e]) * inv_l, __uint_as_float(v[2 * e + 1]) * inv_l);
+            w[e] = *reinterpret_cast<const uint32_t*>(&b2);
+          }
+          if (p.wide_out) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(v[c + 2 * e]) * inv_l,
-                                                              __uint_as_float(v[c + 2 * e + 1]) * inv_l);
-              w[e] = *reinterpret_cast<const uint32_t*>(&b2);
-            }
-            *reinterpret_cast<uint4*>(orow + cb * 32 + c) = make_uint4(w[0], w[1], w[2], w[3]);
+            for (int e = 0; e < 16; e += 8)
+              asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(orow + cb * 32 + 2 * e), "r"(w[e]),
+                           "r"(w[e + 1]), "r"(w[e + 2]), "r"(w[e + 3]), "r"(w[e + 4]), "r"(w[e + 5]), "r"(w[e + 6]), "r"(w[e + 7])
+                           : "memory");
+          } else {
+#pragma unroll
+            for (int e = 0; e < 16; e += 4)
+              *reinterpret_cast<uint4*>(orow + cb * 32 + 2 * e) = make_uint4(w[e], w[e + 1], w[e + 2], w[e + 3]);
           }
         }
       }
@@ -562,6 +572,7 @@ static st3_status prefill_attend_impl(const void* q, const void* k, const void* 
   p.out = static_cast<__nv_bfloat16*>(out);
   p.head_probs = num_visual > 0 ? head_probs : nullptr;
   p.status = dev_status;
+  p.wide_out = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
   p.T = seq_len; p.sys_len = sys_len; p.num_visual = num_visual;
   p.fill = ids ? scores : nullptr;
   p.fill_per_seq = num_visual_total; p.num_heads = num_heads;

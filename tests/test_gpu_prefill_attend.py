@@ -234,3 +234,22 @@ def test_scores_by_original_index(H, nv, total):
         p = torch.softmax(torch.einsum("nd,ntd->nt", q[:, -1].double(), k.double()) / 128 ** 0.5, dim=1)[:, 2:2 + nv]
         want.scatter_(1, ids.long(), p.view(nb, H, nv).sum(1))
     assert torch.allclose(scores.double(), want, rtol=2e-3, atol=1e-7)
+
+
+@pytest.mark.parametrize("T", [1, 129, 200])
+def test_outputs_on_16_and_on_32_bytes_are_the_same(T):
+    """An output aligned to 32 bytes takes wider stores; the bytes are the same, and nothing is written around them."""
+    build()
+    g = torch.Generator().manual_seed(T)
+    q, k, v = (torch.randn(2, T, 128, generator=g).to(torch.bfloat16).cuda() for _ in range(3))
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    got = []
+    for shift in (0, 8):                                       # elements of 2 bytes
+        room = torch.full((2 * T * 128 + 32,), -7.0, dtype=torch.bfloat16, device="cuda")
+        assert room.data_ptr() % 32 == 0
+        B.st3_prefill_attend(q.data_ptr(), k.data_ptr(), v.data_ptr(), room.data_ptr() + 2 * shift, None, None,
+                             status.data_ptr(), 2, 2, T, 128, "bf16", 0, 0, torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        assert (room[:shift] == -7.0).all() and (room[shift + 2 * T * 128:] == -7.0).all()
+        got.append(room[shift:shift + 2 * T * 128].clone())
+    assert int(status.item()) == 0 and torch.equal(got[0], got[1]) and torch.isfinite(got[0].float()).all()
