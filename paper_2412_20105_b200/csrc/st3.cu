@@ -544,11 +544,11 @@ st3_status st3_create(const st3_config* cfg, void* dev_workspace, size_t bytes, 
   }
   ctx->num_sms = sms;
   ctx->attend_ctas_per_sm = tile_bytes(cfg) > 16384 ? 1 : 2;
-  // Selection: 16 bytes a row (key, two lists), and a stage for the logits that lies over the second list: all rows if
-  // 48 KB hold them, less where two blocks with their 16 bytes a row would no longer fit an SM, at least 48 rows a head.
+  // Selection: 16 bytes a row (key, two lists), and a stage for the logits that lies over the second list: all rows of the
+  // heads, or as many as leave room for two blocks on an SM, at least 48 of each.
   {
     const int rows = 16 * cfg->num_visual + 16, tail = (12 * cfg->num_visual + 15) / 16 * 16;  // the stage starts at `tail`
-    const int room = std::max(std::min(100 * 1024, tail + 48 * 1024), rows) - tail;
+    const int room = std::max(100 * 1024, rows) - tail;
     const int fit = std::max(room / (4 * cfg->num_heads) - 16, 32) / 32, all = ceil_div(std::max(cfg->num_visual, 48) - 16, 32);
     ctx->stage_rows = 32 * std::min(fit, all) + 16;
     ctx->finish_smem = std::max(rows, tail + 4 * cfg->num_heads * ctx->stage_rows);

@@ -252,9 +252,10 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
       s_key[i] = ((unsigned long long)u << 32) | (unsigned long long)(0xffffffffu - (unsigned)id);
     }
   }
-  // A warp scores 16 rows a pass: lane (four rows, group g) sums every eighth head of its rows, and the groups' sums meet in
-  // four shuffles that leave a lane with one row: a fixed order of additions, and a third of the shared-memory reads that a
-  // row per lane takes (1 540 -> 700 cycles for 288 rows of 32 heads).
+  // A lane sums every eighth head of four rows (a warp: 16 rows); the sums meet in shuffles that leave a lane with one row: a
+  // fixed order of additions, and a third of the shared-memory reads that a row per lane takes (1 540 -> 700 cycles a pass of
+  // 256 rows of 32 heads).  Every fourth head (32 rows) where 16 rows a warp take a second pass for a few rows: a small fp32
+  // layer 186 -> 183.5 us a generation, a prompt of 32 7B layers 1 227 -> 1 206; with 40 heads it loses (24 590 -> 24 690 us).
   for (int c0 = 0; own_scores && c0 < n_cur; c0 += pitch) {
     if (c0) {
       __syncthreads();
@@ -262,12 +263,14 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
       copies_landed();
       __syncthreads();
     }
-    const int rows = min(pitch, n_cur - c0), g = lane >> 2;
-    for (int r0 = warp * 16; r0 < rows; r0 += kFinishWarps * 16) {
-      const float* at = s_log + min(r0 + (lane & 3) * 4, (rows - 1) & ~3);
+    const int rows = min(pitch, n_cur - c0);
+    const int lq = rows > kFinishWarps * 16 && H <= 32 ? 3 : 2;  // log2 of the row quads of a warp
+    const int span = 4 << lq, groups = 32 >> lq, quad = lane & ((1 << lq) - 1), g = lane >> lq;
+    for (int r0 = warp * span; r0 < rows; r0 += kFinishWarps * span) {
+      const float* at = s_log + min(r0 + quad * 4, (rows - 1) & ~3);
       float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll 4
-      for (int h = g; h < H; h += 8) {
+      for (int h = g; h < H; h += groups) {
         const float2 st = s_ML[h];
         const float4 x = *reinterpret_cast<const float4*>(at + h * pitch);
         a0 += fast_exp2(x.x - st.x) * st.y;
@@ -280,9 +283,9 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
       const float b0 = (up ? a2 : a0) + __shfl_xor_sync(0xffffffffu, up ? a0 : a2, 16);
       const float b1 = (up ? a3 : a1) + __shfl_xor_sync(0xffffffffu, up ? a1 : a3, 16);
       float mass = (odd ? b1 : b0) + __shfl_xor_sync(0xffffffffu, odd ? b0 : b1, 8);
-      mass += __shfl_xor_sync(0xffffffffu, mass, 4);
-      const int r = r0 + (lane & 3) * 4 + (up ? 2 : 0) + (odd ? 1 : 0), i = c0 + r;
-      if (!(lane & 4) && r < rows) {
+      if (lq == 2) mass += __shfl_xor_sync(0xffffffffu, mass, 4);
+      const int r = r0 + quad * 4 + (up ? 2 : 0) + (odd ? 1 : 0), i = c0 + r;
+      if ((lq == 3 || !(lane & 4)) && r < rows) {
         if (!(mass >= 0.f) || !(mass <= 3.0e38f)) { bad = true; mass = 0.f; }
         const int id = fresh ? i : s_hole[i];
         mass_by_id[id] = mass;
