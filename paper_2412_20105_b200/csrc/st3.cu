@@ -244,8 +244,10 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
   };
   if (select_first) {  // prune by the caller's scores before the layer attends
     ctx->launches++;
-    if (launch(st3_finish_kernel<T, D, 1, kFinishThreads>, (unsigned)(2 * units), kFinishThreads, ctx->finish_smem, pdl, st,
-               *select_first) != cudaSuccess || !gather())
+    // nothing to merge yet: the first plane only
+    const dim3 grid((unsigned)c.batch, (unsigned)p.layer_count);
+    if (launch(st3_finish_kernel<T, D, 1, kFinishThreads>, grid, kFinishThreads, ctx->finish_smem, pdl, st, *select_first) !=
+            cudaSuccess || !gather())
       return ST3_ERR_CUDA;
   }
   cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr;
@@ -286,7 +288,12 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
     const bool many = units > ctx->num_sms, two = many && 2 * ctx->finish_smem <= 200 * 1024;
     auto kernel = two ? st3_finish_kernel<T, D, 2, kFinishThreads>
                   : many ? st3_finish_kernel<T, D, 1, 2 * kFinishThreads> : st3_finish_kernel<T, D, 1, kFinishThreads>;
-    if (launch(kernel, (unsigned)(2 * units), many && !two ? 2 * kFinishThreads : kFinishThreads, ctx->finish_smem, pdl, st,
+    // A warp merges one head after another, a round trip each: as many output blocks as give every warp one head, while the
+    // whole launch (a block to an SM) fits the GPU at once.  7B layers one a call 8 973 -> 8 694 us a generation, 13B layers
+    // of 16 sequences 24 585 -> 23 740, two NeXT sequences in four layers of 32 heads 3 760 -> 2 958.
+    const int out_blocks = std::max(1, std::min(ceil_div(c.num_heads, kFinishThreads / 32), ctx->num_sms / units - 1));
+    const dim3 grid((unsigned)c.batch, (unsigned)p.layer_count, (unsigned)(1 + out_blocks));
+    if (launch(kernel, grid, many && !two ? 2 * kFinishThreads : kFinishThreads, ctx->finish_smem, pdl, st,
                p) != cudaSuccess)
       return ST3_ERR_CUDA;
   }

@@ -131,13 +131,13 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
-// 4 or 16 bytes global -> shared without a register in between; copies_landed waits for all of the calling thread's
+// 4, 8 or 16 bytes global -> shared without a register in between; copies_landed waits for all of the calling thread's
 template <int N>
 __device__ __forceinline__ void copy_async(void* dst_smem, const void* src_gmem) {
   if constexpr (N == 16)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst_smem)), "l"(src_gmem) : "memory");
   else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst_smem)), "l"(src_gmem) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(dst_smem)), "l"(src_gmem), "n"(N) : "memory");
 }
 __device__ __forceinline__ void copies_landed() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 

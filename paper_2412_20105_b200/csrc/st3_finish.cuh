@@ -8,8 +8,8 @@ namespace {
 // ------------------------------------------------------------------------------------------
 // Merge partials, visual scores, top-k (Eq. 3), in-place compaction (Eq. 7's eviction)
 // ------------------------------------------------------------------------------------------
-// Two blocks per (layer, sequence), on different SMs, that never wait for each other:
-//   OUT block   merges the chunk partials of every head into the attention output (a warp per head);
+// Two or more blocks per (layer, sequence), on different SMs, that never wait for each other:
+//   OUT block   merges the chunk partials of its heads into the attention output (a warp per head);
 //   TRIM block  merges only the (max, sum) pairs, turns the raw logits into head-summed
 //               probabilities, selects the rows to keep, pairs holes with kept tail rows and
 //               moves the rows.
@@ -38,6 +38,9 @@ __device__ __forceinline__ void merge_stats(const float2* ml, long long item0, i
 constexpr int kSelBins = 256;   // bins of the selection's histogram, over the range of the scores; eight to a lane
 constexpr int kSelCand = 64;    // keys of the bin that the cut falls into that are ranked directly
 
+template <int N>
+struct Floats { static constexpr int value = N; };
+
 // BPS blocks of NT threads to an SM: one of 512 with 128 registers each, two of them when a launch has more (layer,
 // sequence) units than the GPU holds blocks (the work of a unit is a chain of round trips, and more units in flight end
 // sooner), or one of 1024 where two do not fit.
@@ -57,10 +60,10 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int B = p.B, H = p.H, Nv = p.Nv;
-  const int units = p.layer_count * B;  // blocks [0, units) trim, blocks [units, 2 units) write the output
-  const bool out_role = (int)blockIdx.x >= units;
-  const int unit = out_role ? blockIdx.x - units : blockIdx.x;
-  const int l_rel = unit / B, b = unit % B;
+  // grid (sequences, layers, 1 + output blocks): the first plane trims, the others write the output.  No division: a small
+  // launch starts little ahead of the end of its wait.
+  const int b = blockIdx.x, l_rel = blockIdx.y, out_part = (int)blockIdx.z - 1;
+  const bool out_role = out_part >= 0;
   const int l = p.layer_begin + l_rel;
   const long long lb = (long long)l * B + b;
   const LayerParams y = p.layer[l_rel];
@@ -79,7 +82,8 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
   // The parameters a block needs are read before it waits: they are cold in the constant cache (one 7B layer a call
   // 11.07 -> 10.88 us, a small fp32 layer 10.1 -> 9.7, a 13B layer of 16 sequences 44.6 -> 43.5).
   asm volatile("" ::"l"(ml), "l"(p.part_acc), "l"(p.out), "l"(p.logits_copy[y.src_copy]), "l"(p.ids), "l"(p.n_cur),
-               "l"(p.flags), "l"(p.ext_scores), "l"(item0 + item0_s), "l"(p.mass_by_id), "r"(p.fresh), "r"(nit + nit_s));
+               "l"(p.flags), "l"(p.ext_scores), "l"(item0 + item0_s), "l"(p.mass_by_id), "r"(p.fresh), "r"(nit + nit_s),
+               "r"(p.stage_rows));
   // This launch may have been set up while the attention launch before it was still running: wait for that
   // whole grid (and, through it, for everything earlier in the stream).  Then the next step's attention launch
   // may start; it waits on p.flags for what this launch changes.
@@ -87,10 +91,9 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (out_role) {
-    if (p.ext_scores) return;  // selection-only launch: nothing to merge yet
     // ===================== OUT block: attention output of every head =====================
     constexpr int kMergeBatch = 8 * 1024 / (BPS * NT);  // partials in flight per round trip, as the registers allow
-    for (int h = tid >> 5; h < H; h += kFinishWarps) {
+    for (int h = out_part * kFinishWarps + (tid >> 5); h < H; h += ((int)gridDim.z - 1) * kFinishWarps) {
       float a[kMergeBatch][DPL];
       auto load_batch = [&](int i0) {
 #pragma unroll
@@ -173,13 +176,15 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
   float* s_log = reinterpret_cast<float*>(smem + ((size_t)Nv * 12 + 15) / 16 * 16);  // [H][pitch], over the list of movers
   auto stage = [&](int c0) {
     const int rows = min(pitch, n_cur - c0);
-    if (Nv % 4 == 0) {  // every head's logits start on 16 bytes
+    auto copy = [&](auto floats) {  // that many at a time: every head's logits start on a multiple of them
+      constexpr int N = decltype(floats)::value;
       for (int h = warp; h < H; h += kFinishWarps)
-        for (int i = 4 * lane; i < rows; i += 128) copy_async<16>(s_log + h * pitch + i, logits + (h * Nv + c0 + i));
-    } else {
-      for (int h = warp; h < H; h += kFinishWarps)
-        for (int i = lane; i < rows; i += 32) copy_async<4>(s_log + h * pitch + i, logits + (h * Nv + c0 + i));
-    }
+#pragma unroll(N == 1 ? 4 : 1)
+        for (int i = N * lane; i < rows; i += N * 32) copy_async<4 * N>(s_log + h * pitch + i, logits + (h * Nv + c0 + i));
+    };
+    if (Nv % 4 == 0) copy(Floats<4>());
+    else if (Nv % 2 == 0) copy(Floats<2>());
+    else copy(Floats<1>());
   };
   if (own_scores) {
     // (max, sum) of the heads: a warp takes eight heads, four lanes to a head
@@ -226,8 +231,11 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
     } else if (!src_here) {  // the pruning layer ran in an earlier launch of this step: its statistics were kept
       for (int i = tt; i < H; i += kFinishThreads) s_ML[i] = *reinterpret_cast<const float2*>(p.head_stat + 2 * (lb_src * H + i));
     }
-    copies_landed();
+  } else {  // scores of the caller, of a new prompt: each thread fetches what it will read
+    const float* ext = p.ext_scores + ((long long)l_rel * B + b) * Nv;
+    for (int i = tt; i < n_cur; i += kFinishThreads) copy_async<4>(s_log + i, ext + i);
   }
+  copies_landed();
   __syncthreads();
   if (!fresh && n_dev != n_host) {  // host bookkeeping and device state disagree: flag, do not touch
     if (tt == 0) atomicOr(p.status, ST3_DEV_COUNT_MISMATCH);
@@ -240,16 +248,14 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
   unsigned lo = 0xffffffffu, hi = 0u;  // range of the keys' high words
   if (!own_scores) {
     // scores supplied by the caller (any finite float): order-preserving map of the bits to unsigned
-    const float* ext = p.ext_scores + ((long long)l_rel * B + b) * Nv;
     for (int i = tt; i < n_cur; i += kFinishThreads) {
-      const int id = fresh ? i : ids[i];
-      float sc = ext[id];
+      float sc = s_log[i];
       if (!(fabsf(sc) <= 3.0e38f)) { bad = true; sc = -3.0e38f; }
-      mass_by_id[id] = sc;
+      mass_by_id[i] = sc;
       unsigned u = __float_as_uint(sc);
       u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
       lo = min(lo, u); hi = max(hi, u);
-      s_key[i] = ((unsigned long long)u << 32) | (unsigned long long)(0xffffffffu - (unsigned)id);
+      s_key[i] = ((unsigned long long)u << 32) | (unsigned long long)(0xffffffffu - (unsigned)i);
     }
   }
   // A lane sums every eighth head of four rows (a warp: 16 rows); the sums meet in shuffles that leave a lane with one row: a

@@ -436,6 +436,44 @@ def test_selection_over_hard_score_distributions(nv, keep_bp):
         ctx.close()
 
 
+@pytest.mark.parametrize("H,nv", [(1, 17), (8, 256), (9, 257), (33, 511), (32, 513), (40, 576), (128, 700), (31, 1023),
+                                  (32, 1028)])
+def test_selection_by_own_scores_at_the_edges_of_its_passes(H, nv):
+    """Head counts and row counts around what a warp, a pass and the staged logits hold, rows on and off 16 bytes: the
+    scores against 64 bits, the kept rows against an exact sort of those scores, and the rows moved with their ids."""
+    D, sys_len, text, steps = 64, 2, 3, 4
+    cfg, ctx = _handmade(nv, H, D, sys_len, text, steps=steps, keep_bp=9000)
+    try:
+        g = torch.Generator().manual_seed(1000 * H + nv)
+        K, V = (torch.randn(1, 1, H, sys_len + nv + text, D, generator=g) for _ in range(2))
+        q, kn, vn = (torch.randn(steps + 1, 1, 1, H, D, generator=g) for _ in range(3))
+        out = torch.empty(1, 1, H, D, device="cuda")
+        keys = K[0, 0].double()
+        vis = list(range(nv))                                                       # rows held, in cache order
+        for t in range(steps):
+            if t == 0:
+                ctx.prefill_select(q[0].cuda(), K.cuda(), V.cuda(), [text], out)
+            else:
+                ctx.decode_step(t, q[t].cuda(), kn[t].cuda(), vn[t].cuda(), out)
+                keys = torch.cat([keys, kn[t, 0, 0].double()[:, None]], 1)
+            rest = list(range(sys_len)) + list(range(sys_len + nv, keys.shape[1]))
+            at = torch.tensor([sys_len + i for i in vis] + rest)
+            p = torch.softmax(torch.einsum("hd,htd->ht", q[t, 0, 0].double(), keys[:, at]) / D ** 0.5, dim=1)
+            want = p[:, :len(vis)].sum(0)
+            ids, cnt, mass = ctx.get_kept(0)
+            got = mass[0].cpu()[torch.tensor(vis)]
+            assert torch.allclose(got.double(), want, rtol=5e-4, atol=0)            # fp32 dot products and ex2.approx
+            k = B.st3_schedule_count(cfg, 0, t)
+            best = np.array(vis)[np.lexsort((np.array(vis), -got.numpy()))[:k]]     # ties: the lower original index
+            vis = ids[0, :k].tolist()
+            assert int(cnt[0]) == k and 0 < k < nv and sorted(vis) == sorted(best.tolist())
+            _, vv, _, _ = ctx.get_rows(0, 0, H - 1)
+            assert torch.equal(vv[:k].cpu(), V[0, 0, H - 1, sys_len + torch.tensor(vis)])
+        assert ctx.status() == 0
+    finally:
+        ctx.close()
+
+
 def test_more_heads_sequences_and_layers_than_a_grid_dimension_holds():
     """65 536 (layer, sequence, head) units in one call: 64 sequences of the same contents against one of them."""
     L, H, D, nv, text, nb = 32, 32, 64, 8, 3, 64
