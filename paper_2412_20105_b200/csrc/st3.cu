@@ -284,7 +284,10 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
     // Also a programmatic dependent launch: the attention kernel allows it at its start, the blocks become
     // resident as that grid drains, read their parameters and wait for all of it.
     // Two blocks per SM (with half the registers each) once the units outnumber the SMs (see st3_finish.cuh), as long as
-    // they fit: up to 6399 visual tokens; beyond, one of twice the threads.
+    // they fit: up to 6399 visual tokens; beyond, one of twice the threads.  Selection launches, the former blocks of up to
+    // 1024 threads with logits in registers / now: 296 units of 6399 tokens 31.7 / 27.9 us, 300 of 6400 48.7 / 43.5, 300 of
+    // 144 with 8 heads 16.0 / 14.4, 100 (one block an SM) of 2880 18.4 / 17.1; slower where rows are odd in number, many and
+    // of many heads (4-byte copies): 8 of 2877 with 40 heads 29.3 / 31.5.
     const bool many = units > ctx->num_sms, two = many && 2 * ctx->finish_smem <= 200 * 1024;
     auto kernel = two ? st3_finish_kernel<T, D, 2, kFinishThreads>
                   : many ? st3_finish_kernel<T, D, 1, 2 * kFinishThreads> : st3_finish_kernel<T, D, 1, kFinishThreads>;
