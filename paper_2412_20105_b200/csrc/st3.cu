@@ -12,7 +12,7 @@
 //                       leave one softmax partial (m, l, acc) per item, plus the raw logits of visual
 //                       rows for layers that evict at this step; the newest token's row is appended
 //                       on the way.
-//   st3_finish_kernel   per (layer, sequence) one block merges the partials of every head into the
+//   st3_finish_kernel   per (layer, sequence) one or more blocks merge the partials of the heads into the
 //                       attention output and one block scores the visual rows, selects the rows
 //                       to keep (ties toward the lower original index) and fills the holes among the
 //                       first n_new rows with the kept rows of the tail.
