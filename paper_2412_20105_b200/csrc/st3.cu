@@ -314,7 +314,9 @@ st3_status set_attrs_t(st3_ctx* ctx) {
       return ST3_ERR_CUDA;
   for (auto kernel : {st3_finish_kernel<T, D, 1, kFinishThreads>, st3_finish_kernel<T, D, 2, kFinishThreads>,
                       st3_finish_kernel<T, D, 1, 2 * kFinishThreads>})
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->finish_smem) != cudaSuccess)
+    // The attribute belongs to the kernel, which contexts of other sizes launch too: the most any of them may ask for, not
+    // what this one needs.  What a launch takes of an SM follows its own size.
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem) != cudaSuccess)
       return ST3_ERR_CUDA;
   return ST3_OK;
 }
@@ -563,7 +565,7 @@ st3_status st3_create(const st3_config* cfg, void* dev_workspace, size_t bytes, 
     ctx->stage_rows = 32 * std::min(fit, all) + 16;
     ctx->finish_smem = std::max(rows, tail + 4 * cfg->num_heads * ctx->stage_rows);
   }
-  if (ctx->attend_smem > 200 * 1024 || ctx->finish_smem > 200 * 1024) { delete ctx; return ST3_ERR_UNSUPPORTED; }
+  if (ctx->attend_smem > kMaxDynSmem || ctx->finish_smem > kMaxDynSmem) { delete ctx; return ST3_ERR_UNSUPPORTED; }
 #define ST3_ATTR(T, D) set_attrs_t<T, D>(ctx)
   st3_status s = ST3_DISPATCH(ctx, ST3_ATTR);
 #undef ST3_ATTR

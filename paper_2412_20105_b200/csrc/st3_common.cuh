@@ -18,6 +18,7 @@ constexpr int kMaxChunkRows = 128;  // upper bound on the rows of one work item
 constexpr int kMaxLayers = 64;
 constexpr int kMaxHeads = 128;
 constexpr int kMaxVisual = 8192;
+constexpr int kMaxDynSmem = 200 * 1024;  // dynamic shared memory a context may ask for in a launch
 constexpr long long kWaitCycles = 4000000000LL;  // ~2 s: bound on any wait for an async copy
 constexpr int kMaxFollow = 62;  // lazy layers whose values can follow one work item of the layer they inherit from
 

@@ -474,6 +474,39 @@ def test_selection_by_own_scores_at_the_edges_of_its_passes(H, nv):
         ctx.close()
 
 
+@pytest.mark.parametrize("heads", [(40, 8), (8, 40)])
+def test_contexts_of_different_sizes_used_in_turn(heads):
+    """Their selections take different amounts of shared memory: neither context may take anything from the other."""
+    nv, D, sys_len, text, steps = 576, 64, 2, 3, 3
+    g = torch.Generator().manual_seed(9)
+    data = {H: (torch.randn(steps + 1, 3, 1, 1, H, D, generator=g).cuda(),
+                *(torch.randn(1, 1, H, sys_len + nv + text, D, generator=g).cuda() for _ in range(2))) for H in heads}
+
+    def step(ctx, H, t):
+        x, K, V = data[H]
+        out = torch.empty(1, 1, H, D, device="cuda")
+        if t == 0:
+            ctx.prefill_select(x[0, 0], K, V, [text], out)
+        else:
+            ctx.decode_step(t, x[t, 0], x[t, 1], x[t, 2], out)
+        return out
+
+    alone = {}
+    for H in heads:
+        _, ctx = _handmade(nv, H, D, sys_len, text, steps=steps)
+        alone[H] = [step(ctx, H, t) for t in range(steps + 1)]
+        ctx.close()
+    ctxs = {H: _handmade(nv, H, D, sys_len, text, steps=steps)[1] for H in heads}
+    try:
+        for t in range(steps + 1):
+            for H in heads:
+                assert torch.equal(step(ctxs[H], H, t), alone[H][t]), (H, t)
+        assert all(c.status() == 0 for c in ctxs.values())
+    finally:
+        for c in ctxs.values():
+            c.close()
+
+
 def test_more_heads_sequences_and_layers_than_a_grid_dimension_holds():
     """65 536 (layer, sequence, head) units in one call: 64 sequences of the same contents against one of them."""
     L, H, D, nv, text, nb = 32, 32, 64, 8, 3, 64
