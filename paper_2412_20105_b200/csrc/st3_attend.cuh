@@ -669,10 +669,10 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
     const int grp = (warp - kSlots) / kGroupWarps;
     const int w = (warp - kSlots) % kGroupWarps;
     const int r8 = lane >> 2, c4 = lane & 3;
-    int rot;
-    if (CPL == 2) rot = r8 & 1;
-    else if (CPL == 4) rot = (c4 >> 1) + 2 * (r8 & 1);
-    else rot = lane & 7;
+    int flip;
+    if (CPL == 2) flip = r8 & 1;
+    else if (CPL == 4) flip = (c4 >> 1) + 2 * (r8 & 1);
+    else flip = lane & 7;
     const float sc = 1.4426950408889634f * rsqrtf((float)D);
     unsigned live = (1u << kSlots) - 1;  // slots that may still deliver work
     unsigned phf = 0;  // this warp's phase bits: bit 2s for tile area A of slot s, bit 2s+1 for area B
@@ -718,11 +718,11 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       }
       if (active) {
         const unsigned char* sQ = sV + kTileBytes;
-        // this lane's quarter of the query, in the rotated chunk order it reads rows in
+        // this lane's quarter of the query, in the chunk order it reads rows in
         u64 q2[CPL][EPL / 2];
 #pragma unroll
         for (int j = 0; j < CPL; ++j) {
-          const int jj = (j + rot) & (CPL - 1);
+          const int jj = j ^ flip;
           unpack16_pairs(*reinterpret_cast<const uint4*>(sQ + (c4 * CPL + jj) * 16), q2[j]);
         }
         // ---- K pass: four lanes per row, one logit per row ----
@@ -740,16 +740,23 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
             const unsigned char* row = sK + (size_t)min(r, nrows - 1) * ROWB + c4 * (CPL * 16);
 #pragma unroll
             for (int j = 0; j < CPL; ++j) {
-              const int jj = (j + rot) & (CPL - 1);
+              const int jj = j ^ flip;
               u64 k2[EPL / 2];
               unpack16_pairs(*reinterpret_cast<const uint4*>(row + jj * 16), k2);
 #pragma unroll
               for (int e = 0; e < EPL / 2; ++e) fma2(a2[j], q2[j][e], k2[e]);
             }
           }
-          float t = 0.f;
+          // Neighbours first, then pairs of pairs: the same additions for every `flip`, so that identical keys get identical
+          // logits wherever their rows stand (ties go by the original index).
+          float part[CPL];
 #pragma unroll
-          for (int j = 0; j < CPL; ++j) t += sum2(a2[j]);
+          for (int j = 0; j < CPL; ++j) part[j] = sum2(a2[j]);
+#pragma unroll
+          for (int o = 1; o < CPL; o <<= 1)
+#pragma unroll
+            for (int j = 0; j < CPL; j += 2 * o) part[j] += part[j + o];
+          float t = part[0];
           t += __shfl_xor_sync(0xffffffffu, t, 1);
           t += __shfl_xor_sync(0xffffffffu, t, 2);
           sl[g] = ok[g] ? t * sc : -INFINITY;  // log2-domain logit

@@ -228,8 +228,8 @@ def test_layer_by_layer_calls_match_one_call_for_all_layers():
         a.close(); b.close()
 
 
-def _handmade(nv, H=2, D=64, sys_len=2, text=3, steps=4, keep_bp=5000, **cfg_kw):
-    cfg = B.make_config(num_layers=1, num_heads=H, head_dim=D, dtype="f32", batch=1, sys_len=sys_len,
+def _handmade(nv, H=2, D=64, sys_len=2, text=3, steps=4, keep_bp=5000, dtype="f32", **cfg_kw):
+    cfg = B.make_config(num_layers=1, num_heads=H, head_dim=D, dtype=dtype, batch=1, sys_len=sys_len,
                         num_visual=nv, max_text_len=text, max_decode_steps=steps, stride=1, step_ratio_bp=0,
                         first_prune_layer=0, first_ratio_bp=10000 - keep_bp, tau=float(steps), **cfg_kw)
     return cfg, B.Context(cfg)
@@ -265,6 +265,47 @@ def test_equal_scores_keep_the_lowest_original_indices(static_rank):
             k = B.st3_schedule_count(cfg, 0, t)
             assert int(cnt[0]) == k and sorted(ids[0, :k].tolist()) == list(range(k))
         assert ctx.status() == 0
+    finally:
+        ctx.close()
+
+
+def _check_tied_classes(ctx, cfg, keys, q, dtype, sys_len, text, classes):
+    """Visual token i carries the key of class i % classes: tokens of a class must score alike to the last bit wherever
+    they stand in the prompt or (once holes have been filled) in the cache, and lose by their index only."""
+    H, D, nv = cfg.num_heads, cfg.head_dim, cfg.num_visual
+    t = dict(f32=torch.float32, bf16=torch.bfloat16)[dtype]
+    g = torch.Generator().manual_seed(nv)
+    K, V = (torch.randn(1, 1, H, sys_len + nv + text, D, generator=g) for _ in range(2))
+    K[0, 0, :, sys_len:sys_len + nv] = keys[:, torch.arange(nv) % classes]
+    kn = torch.randn(1, 1, H, D, generator=g).to(t).cuda()
+    out = torch.empty(1, 1, H, D, dtype=t, device="cuda")
+    vis = torch.arange(nv)
+    for step in range(4):
+        if step == 0:
+            ctx.prefill_select(q[0].to(t).cuda(), K.to(t).cuda(), V.to(t).cuda(), [text], out)
+        else:
+            ctx.decode_step(step, q[step].to(t).cuda(), kn, kn, out)
+        ids, cnt, mass = ctx.get_kept(0)
+        mass = mass[0].cpu()
+        k = B.st3_schedule_count(cfg, 0, step)
+        for c in range(classes):
+            m = mass[vis[vis % classes == c]]
+            assert (m == m[:1]).all(), (step, c, m.unique().tolist())
+        best = vis[np.lexsort((vis.numpy(), -mass[vis].numpy()))[:k]]
+        assert int(cnt[0]) == k < len(vis) and sorted(ids[0, :k].tolist()) == sorted(best.tolist()), step
+        vis = best.sort().values
+    assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("dtype,D", [("f32", 64), ("f32", 128), ("bf16", 64), ("bf16", 128)])
+@pytest.mark.parametrize("H", [1, 5])
+def test_identical_keys_score_alike_wherever_they_stand(dtype, D, H):
+    nv, sys_len, text = 333, 2, 3
+    cfg, ctx = _handmade(nv, H, D, sys_len, text, steps=8, keep_bp=9000, dtype=dtype)
+    try:
+        g = torch.Generator().manual_seed(D + H)
+        _check_tied_classes(ctx, cfg, torch.randn(H, 15, D, generator=g), torch.randn(4, 1, 1, H, D, generator=g), dtype,
+                            sys_len, text, 15)
     finally:
         ctx.close()
 
