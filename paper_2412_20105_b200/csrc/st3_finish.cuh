@@ -261,10 +261,12 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
       s_key[i] = ((unsigned long long)u << 32) | (unsigned long long)(0xffffffffu - (unsigned)i);
     }
   }
-  // A lane sums every eighth head of four rows (a warp: 16 rows); the sums meet in shuffles that leave a lane with one row: a
-  // fixed order of additions, and a third of the shared-memory reads that a row per lane takes (1 540 -> 700 cycles a pass of
-  // 256 rows of 32 heads).  Every fourth head (32 rows) where 16 rows a warp take a second pass for a few rows: a small fp32
-  // layer 186 -> 183.5 us a generation, a prompt of 32 7B layers 1 227 -> 1 206; with 40 heads it loses (24 590 -> 24 690 us).
+  // A lane sums every eighth head of four rows (a warp: 16 rows); the sums meet in shuffles that leave a lane with one row, and
+  // take a third of the shared-memory reads that a row per lane takes (1 540 -> 700 cycles a pass of 256 rows of 32 heads).
+  // Every fourth head (32 rows) where 16 rows a warp do not hold a stage: a small fp32 layer 186 -> 183.5 us a generation, a
+  // prompt of 32 7B layers 1 227 -> 1 206; with 40 heads it loses (24 590 -> 24 690 us).  One choice for all passes: it
+  // decides the order in which a row's heads are added, and rows with equal logits must get equal scores.
+  const int lq = min(pitch, n_cur) > kFinishWarps * 16 && H <= 32 ? 3 : 2;  // log2 of the row quads of a warp
   for (int c0 = 0; own_scores && c0 < n_cur; c0 += pitch) {
     if (c0) {
       __syncthreads();
@@ -273,7 +275,6 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
       __syncthreads();
     }
     const int rows = min(pitch, n_cur - c0);
-    const int lq = rows > kFinishWarps * 16 && H <= 32 ? 3 : 2;  // log2 of the row quads of a warp
     const int span = 4 << lq, groups = 32 >> lq, quad = lane & ((1 << lq) - 1), g = lane >> lq;
     for (int r0 = warp * span; r0 < rows; r0 += kFinishWarps * span) {
       const float* at = s_log + min(r0 + quad * 4, (rows - 1) & ~3);

@@ -515,6 +515,21 @@ def test_selection_by_own_scores_at_the_edges_of_its_passes(H, nv):
         ctx.close()
 
 
+@pytest.mark.parametrize("H,nv", [(32, 729), (32, 2880), (24, 1152), (40, 2880), (16, 576)])
+def test_ties_across_the_passes_over_the_staged_logits(H, nv):
+    """Logits of a class are equal to the last bit by construction (keys with one entry); the rows of a class fall into
+    several passes, the last of them short."""
+    sys_len, text = 2, 3
+    cfg, ctx = _handmade(nv, H, 64, sys_len, text, steps=8, keep_bp=9000)
+    try:
+        g = torch.Generator().manual_seed(nv + H)
+        keys = torch.zeros(H, 15, 64)
+        keys[:, :, 0] = torch.randn(H, 15, generator=g)
+        _check_tied_classes(ctx, cfg, keys, torch.randn(4, 1, 1, H, 64, generator=g), "f32", sys_len, text, 15)
+    finally:
+        ctx.close()
+
+
 @pytest.mark.parametrize("heads", [(40, 8), (8, 40)])
 def test_contexts_of_different_sizes_used_in_turn(heads):
     """Their selections take different amounts of shared memory: neither context may take anything from the other."""
