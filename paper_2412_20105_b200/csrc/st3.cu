@@ -133,7 +133,7 @@ Layout make_layout(const st3_config* c) {
   L.part_acc_bytes = align_up((size_t)L.max_items * c->num_heads * c->head_dim * sizeof(float), 256);
   L.part_ml = take(2 * L.part_ml_bytes);
   L.part_acc = take(2 * L.part_acc_bytes);
-  L.logits_bytes = align_up(lbh * (size_t)c->num_visual * sizeof(float), 256);
+  L.logits_bytes = align_up(lbh * (size_t)logit_pitch(c->num_visual) * sizeof(float), 256);
   L.logits = take(2 * L.logits_bytes);  // two copies, like the partials
   L.head_stat = take(lbh * 2 * sizeof(float));
   L.mass = take(lb * (size_t)c->num_visual * sizeof(float));

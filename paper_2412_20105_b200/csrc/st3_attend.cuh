@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(kAttendThreads, 2) st3_attend_kernel(const __g
       d.srcK = reinterpret_cast<const unsigned char*>(region_of(lk, b, h, is_vis, 0)) + (size_t)row0 * ROWB;
       d.srcV = reinterpret_cast<const unsigned char*>(region_of(l_rel, b, h, is_vis, 1)) + (size_t)row0 * ROWB;
       d.srcQ = reinterpret_cast<const T*>(p.q) + oidx_of(lk, b, h) * D;
-      d.glog = lbh_of(l_rel, b, h) * p.Nv + r0;
+      d.glog = lbh_of(l_rel, b, h) * logit_pitch(p.Nv) + r0;
       if (inputs_ready) fetch_new(d);
     };
     // Starts the copies of a decoded item into this (free) slot.

@@ -18,6 +18,8 @@ constexpr int kMaxChunkRows = 128;  // upper bound on the rows of one work item
 constexpr int kMaxLayers = 64;
 constexpr int kMaxHeads = 128;
 constexpr int kMaxVisual = 8192;
+// Floats from one head's logits to the next: every head's start on 16 bytes, for the copies of the selection.
+__host__ __device__ constexpr int logit_pitch(int num_visual) { return (num_visual + 3) & ~3; }
 constexpr int kMaxDynSmem = 200 * 1024;  // dynamic shared memory a context may ask for in a launch
 constexpr long long kWaitCycles = 4000000000LL;  // ~2 s: bound on any wait for an async copy
 constexpr int kMaxFollow = 62;  // lazy layers whose values can follow one work item of the layer they inherit from
@@ -72,7 +74,7 @@ struct alignas(64) StepParams {
   int* flags;            // [l][b] sequence number of the last finish launch that is done with (l, b)
   float* part_ml;        // [item*H + h][2]  (m, l) in the log2 domain
   float* part_acc;       // [item*H + h][D]  un-normalised output
-  float* logits;         // [l][b][h][Nv]    raw log2-domain logits of visual rows (this step's copy)
+  float* logits;         // [l][b][h][logit_pitch(Nv)]  raw log2-domain logits of visual rows (this step's copy)
   const float* logits_copy[2];  // both copies (a launch writes the one of its sequence parity)
   float* head_stat;      // [l][b][h][2]     (max, 1/sum) of a pruning layer's merged softmax
   float* mass_by_id;     // [l][b][Nv]
@@ -132,13 +134,14 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
-// 4, 8 or 16 bytes global -> shared without a register in between; copies_landed waits for all of the calling thread's
+// 4 or 16 bytes global -> shared without a register in between; copies_landed waits for all of the calling thread's
 template <int N>
 __device__ __forceinline__ void copy_async(void* dst_smem, const void* src_gmem) {
+  static_assert(N == 4 || N == 16, "4 or 16 bytes");
   if constexpr (N == 16)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst_smem)), "l"(src_gmem) : "memory");
   else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(dst_smem)), "l"(src_gmem), "n"(N) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst_smem)), "l"(src_gmem) : "memory");
 }
 __device__ __forceinline__ void copies_landed() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 

@@ -38,9 +38,6 @@ __device__ __forceinline__ void merge_stats(const float2* ml, long long item0, i
 constexpr int kSelBins = 256;   // bins of the selection's histogram, over the range of the scores; eight to a lane
 constexpr int kSelCand = 64;    // keys of the bin that the cut falls into that are ranked directly
 
-template <int N>
-struct Floats { static constexpr int value = N; };
-
 // BPS blocks of NT threads to an SM: one of 512 with 128 registers a thread, two of them when a launch has more (layer,
 // sequence) units than the GPU holds blocks (the work of a unit is a chain of round trips, and more units in flight end
 // sooner), or one of 1024 where two do not fit.  Bound by latency: two round trips, the flag, and dependent integer work in
@@ -166,7 +163,7 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
   int* ids = p.ids + lb * Nv;
   float* mass_by_id = p.mass_by_id + lb * Nv;
   const long long lb_src = (long long)src * B + b;
-  const float* logits = p.logits_copy[y.src_copy] + lb_src * H * Nv;
+  const float* logits = p.logits_copy[y.src_copy] + lb_src * H * logit_pitch(Nv);
   unsigned long long* s_key = reinterpret_cast<unsigned long long*>(smem);  // [Nv]
   int* s_hole = reinterpret_cast<int*>(smem + (size_t)Nv * 8);              // [Nv], the ids until the scores are known
   int* s_mover = s_hole + Nv;                                               // [Nv]
@@ -179,15 +176,8 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
   float* s_log = reinterpret_cast<float*>(smem + ((size_t)Nv * 12 + 15) / 16 * 16);  // [H][pitch], over the list of movers
   auto stage = [&](int c0) {
     const int rows = min(pitch, n_cur - c0);
-    auto copy = [&](auto floats) {  // that many at a time: every head's logits start on a multiple of them
-      constexpr int N = decltype(floats)::value;
-      for (int h = warp; h < H; h += kFinishWarps)
-#pragma unroll(N == 1 ? 4 : 1)
-        for (int i = N * lane; i < rows; i += N * 32) copy_async<4 * N>(s_log + h * pitch + i, logits + (h * Nv + c0 + i));
-    };
-    if (Nv % 4 == 0) copy(Floats<4>());
-    else if (Nv % 2 == 0) copy(Floats<2>());
-    else copy(Floats<1>());
+    for (int h = warp; h < H; h += kFinishWarps)
+      for (int i = 4 * lane; i < rows; i += 128) copy_async<16>(s_log + h * pitch + i, logits + (h * logit_pitch(Nv) + c0 + i));
   };
   if (own_scores) {
     // (max, sum) of the heads: a warp takes eight heads, four lanes to a head
