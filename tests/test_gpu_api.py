@@ -560,6 +560,38 @@ def test_rows_off_16_bytes_are_selected_as_fast_as_rows_on_them():
             ctx.close()
 
 
+@pytest.mark.parametrize("nb,nv,H", [(50, 6400, 16), (38, 1536, 32), (3, 333, 5)])
+def test_layers_of_a_stage_stay_alike_over_calls_of_different_sizes(nb, nv, H):
+    """The pruning layer in a call of its own, the other layers of its stage in the next one, which may take selection
+    blocks of another size: the same scores to the last bit, so the same tokens in the same order."""
+    L, D, text, steps = 4, 64, 3, 3
+    cfg = B.make_config(num_layers=L, num_heads=H, head_dim=D, dtype="bf16", batch=nb, sys_len=1, num_visual=nv,
+                        max_text_len=text, max_decode_steps=steps, stride=L, step_ratio_bp=0, first_prune_layer=0,
+                        first_ratio_bp=2000, tau=4.0, stage_shared=1)
+    ctx = B.Context(cfg)
+    try:
+        g = torch.Generator(device="cuda").manual_seed(nv)
+        rows = lambda *s: torch.empty(s, dtype=torch.bfloat16, device="cuda").normal_(generator=g)
+        K, V = (rows(1, nb, H, 1 + nv + text, D).expand(L, -1, -1, -1, -1).contiguous() for _ in range(2))
+        for t in range(steps + 1):
+            q, kn, vn = (rows(L, nb, H, D) for _ in range(3))
+            out = torch.empty_like(q)
+            for l0, l1 in ((0, 1), (1, L)):
+                if t == 0:
+                    ctx.prefill_select(q[l0:l1], K[l0:l1], V[l0:l1], [text] * nb, out[l0:l1], layer_begin=l0)
+                else:
+                    ctx.decode_step(t, q[l0:l1], kn[l0:l1], vn[l0:l1], out[l0:l1], layer_begin=l0)
+            n = B.st3_schedule_count(cfg, 0, t)
+            ids, cnt, mass = ctx.get_kept(0)
+            assert (cnt == n).all()
+            for l in range(1, L):
+                i, c, m = ctx.get_kept(l)
+                assert torch.equal(c, cnt) and torch.equal(i[:, :n], ids[:, :n]) and torch.equal(m, mass), (t, l)
+        assert ctx.status() == 0
+    finally:
+        ctx.close()
+
+
 @pytest.mark.parametrize("heads", [(40, 8), (8, 40)])
 def test_contexts_of_different_sizes_used_in_turn(heads):
     """Their selections take different amounts of shared memory: neither context may take anything from the other."""
