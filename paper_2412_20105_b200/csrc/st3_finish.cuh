@@ -414,18 +414,19 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
   const unsigned low_bits = (1u << (k & 31)) - 1;          // the border
   auto low_of = [&](int x) { return x < low_words ? 0xffffffffu : x == low_words ? low_bits : 0u; };
   const int nwords = (n_cur + 31) >> 5;
-  int total = 0;  // set bits: holes | movers << 16
-  for (int w0 = warp; w0 == warp || w0 < nwords; w0 += kFinishWarps) {
-    int all = 0, before = 0;  // of all words, and of the words below w0
-    for (int x = lane; x < nwords; x += 32) {
-      const unsigned word = s_word[x], m = low_of(x);
-      const int c = __popc(word & m) | __popc(word & ~m) << 16;
-      all += c;
-      before += x < w0 ? c : 0;
-    }
-    total = __reduce_add_sync(0xffffffffu, all);
-    before = __reduce_add_sync(0xffffffffu, before);
-    const unsigned word = w0 < nwords ? s_word[w0] : 0u, m = low_of(w0), lt = (1u << lane) - 1;
+  // A warp takes a run of words, so that it adds up those below only once.
+  const int run = (nwords + kFinishWarps - 1) / kFinishWarps, first = warp * run;
+  auto bits_of = [&](int x) { return __popc(s_word[x] & low_of(x)) | __popc(s_word[x] & ~low_of(x)) << 16; };
+  int total = 0, before = 0;  // set bits (holes | movers << 16) of all words, and of the words below w0
+  for (int x = lane; x < nwords; x += 32) {
+    const int c = bits_of(x);
+    total += c;
+    before += x < first ? c : 0;
+  }
+  total = __reduce_add_sync(0xffffffffu, total);
+  before = __reduce_add_sync(0xffffffffu, before);
+  for (int w0 = first; w0 < min(first + run, nwords); before += bits_of(w0++)) {
+    const unsigned word = s_word[w0], m = low_of(w0), lt = (1u << lane) - 1;
     if (word >> lane & 1u) {
       const int i = w0 * 32 + lane;
       if (fresh) ids[before + __popc(word & lt)] = i;  // the prompt's order; st3_gather_kernel copies the rows

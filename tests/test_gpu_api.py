@@ -455,7 +455,8 @@ def _score_sets(nv, g):
                 tiny=u * 1e-42)
 
 
-@pytest.mark.parametrize("nv,keep_bp", [(700, 5000), (700, 1), (2049, 3333), (8192, 5000), (65, 9999), (1, 5000), (300, 20)])
+@pytest.mark.parametrize("nv,keep_bp", [(700, 5000), (700, 1), (2049, 3333), (8192, 5000), (65, 9999), (1, 5000), (300, 20), (513, 5000),
+                                        (1025, 2000), (6401, 7777)])
 def test_selection_over_hard_score_distributions(nv, keep_bp):
     cfg, ctx = _handmade(nv, H=1, keep_bp=keep_bp)
     try:
