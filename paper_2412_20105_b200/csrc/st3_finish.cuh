@@ -414,25 +414,30 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
   const unsigned low_bits = (1u << (k & 31)) - 1;          // the border
   auto low_of = [&](int x) { return x < low_words ? 0xffffffffu : x == low_words ? low_bits : 0u; };
   const int nwords = (n_cur + 31) >> 5;
-  // A warp takes a run of words, so that it adds up those below only once.
+  // A warp takes a run of words, so that it adds up those below only once; its first one is requested together with them
+  // (after the sums: 7B layers one a call 8 746 -> 8 804 us a generation).
   const int run = (nwords + kFinishWarps - 1) / kFinishWarps, first = warp * run;
-  auto bits_of = [&](int x) { return __popc(s_word[x] & low_of(x)) | __popc(s_word[x] & ~low_of(x)) << 16; };
+  unsigned word = first < nwords ? s_word[first] : 0u;
+  auto bits_of = [&](unsigned x, unsigned m) { return __popc(x & m) | __popc(x & ~m) << 16; };
   int total = 0, before = 0;  // set bits (holes | movers << 16) of all words, and of the words below w0
   for (int x = lane; x < nwords; x += 32) {
-    const int c = bits_of(x);
+    const int c = bits_of(s_word[x], low_of(x));
     total += c;
     before += x < first ? c : 0;
   }
   total = __reduce_add_sync(0xffffffffu, total);
   before = __reduce_add_sync(0xffffffffu, before);
-  for (int w0 = first; w0 < min(first + run, nwords); before += bits_of(w0++)) {
-    const unsigned word = s_word[w0], m = low_of(w0), lt = (1u << lane) - 1;
+  for (int w0 = first;;) {
+    const unsigned m = low_of(w0), lt = (1u << lane) - 1;
     if (word >> lane & 1u) {
       const int i = w0 * 32 + lane;
       if (fresh) ids[before + __popc(word & lt)] = i;  // the prompt's order; st3_gather_kernel copies the rows
       else if (m >> lane & 1u) s_hole[(before & 0xffff) + __popc(word & m & lt)] = i;
       else s_mover[(before >> 16) + __popc(word & ~m & lt)] = i;
     }
+    if (++w0 >= min(first + run, nwords)) break;
+    before += bits_of(word, m);
+    word = s_word[w0];
   }
   if (fresh) {
     if (tt == 0) {
