@@ -191,7 +191,8 @@ struct st3_ctx {
   bool profiling;
   std::vector<cudaEvent_t> ev_pool;  // triples: before attend, after attend, after finish (and a prompt's gather)
   size_t ev_used;
-  int attend_smem, finish_smem, stage_rows, num_sms, attend_ctas_per_sm;
+  int attend_smem, num_sms, attend_ctas_per_sm;
+  struct { int smem, stage_rows; } sel[2];  // of a selection block: alone on an SM, or one of two
   int seq;                     // sequence number of the next step's launches (starts at 1)
   unsigned counter_base;       // what the device work counter will read when the next launch starts
   std::vector<int> flag_req;   // per layer: sequence number of the last finish launch over it (0: none)
@@ -231,7 +232,7 @@ cudaError_t launch(void (*kernel)(A...), dim3 grid, int threads, int smem, bool 
 // prefill: the layers' prompt rows stand in p.k_in / p.v_in; gathers: a launch copies (some of) them to the cache;
 // select_first: prune by the caller's scores, then attend.
 template <typename T, int D>
-st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, bool prefill, bool gathers,
+st3_status launch_step_t(st3_ctx* ctx, StepParams& p, cudaStream_t st, bool prefill, bool gathers,
                          const StepParams* select_first) {
   const st3_config& c = ctx->cfg;
   const int units = p.layer_count * c.batch;
@@ -246,7 +247,7 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
     ctx->launches++;
     // nothing to merge yet: the first plane only
     const dim3 grid((unsigned)c.batch, (unsigned)p.layer_count);
-    if (launch(st3_finish_kernel<T, D, 1, kFinishThreads>, grid, kFinishThreads, ctx->finish_smem, pdl, st, *select_first) !=
+    if (launch(st3_finish_kernel<T, D, 1, kFinishThreads>, grid, kFinishThreads, ctx->sel[1].smem, pdl, st, *select_first) !=
             cudaSuccess || !gather())
       return ST3_ERR_CUDA;
   }
@@ -288,7 +289,7 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
     // 1024 threads with logits in registers / now: 296 units of 6399 tokens 31.7 / 27.9 us, 300 of 6400 48.7 / 43.5, 300 of
     // 144 with 8 heads 16.0 / 14.4, 100 (one block an SM) of 2880 18.4 / 17.1; slower where rows are odd in number, many and
     // of many heads (4-byte copies): 8 of 2877 with 40 heads 29.3 / 31.5.
-    const bool many = units > ctx->num_sms, two = many && 2 * ctx->finish_smem <= 200 * 1024;
+    const bool many = units > ctx->num_sms, two = many && 2 * ctx->sel[1].smem <= kMaxDynSmem;
     auto kernel = two ? st3_finish_kernel<T, D, 2, kFinishThreads>
                   : many ? st3_finish_kernel<T, D, 1, 2 * kFinishThreads> : st3_finish_kernel<T, D, 1, kFinishThreads>;
     // A warp merges one head after another, a round trip each: as many output blocks as give every warp one head, while the
@@ -296,7 +297,8 @@ st3_status launch_step_t(st3_ctx* ctx, const StepParams& p, cudaStream_t st, boo
     // of 16 sequences 24 585 -> 23 740, two NeXT sequences in four layers of 32 heads 3 760 -> 2 958.
     const int out_blocks = std::max(1, std::min(ceil_div(c.num_heads, kFinishThreads / 32), ctx->num_sms / units - 1));
     const dim3 grid((unsigned)c.batch, (unsigned)p.layer_count, (unsigned)(1 + out_blocks));
-    if (launch(kernel, grid, many && !two ? 2 * kFinishThreads : kFinishThreads, ctx->finish_smem, pdl, st,
+    p.stage_rows = ctx->sel[two].stage_rows;
+    if (launch(kernel, grid, many && !two ? 2 * kFinishThreads : kFinishThreads, ctx->sel[two].smem, pdl, st,
                p) != cudaSuccess)
       return ST3_ERR_CUDA;
   }
@@ -355,7 +357,7 @@ st3_status run_step(st3_ctx* ctx, int step, int layer_begin, int layer_count, co
   p.lbh_stride = L.lbh_stride;
   p.layer_begin = layer_begin; p.layer_count = layer_count; p.B = c.batch; p.H = c.num_heads;
   p.sys_len = c.sys_len; p.Nv = c.num_visual; p.cap_txt = L.cap_txt; p.step = step; p.append = prefill ? 0 : 1;
-  p.static_rank = c.static_rank ? 1 : 0; p.stage_rows = ctx->stage_rows;
+  p.static_rank = c.static_rank ? 1 : 0;
   p.order = (prefill && !ext_scores) || !ctx->overlap;
   p.fresh = prefill && !ext_scores;
   p.k_in = prefill ? k : nullptr; p.v_in = prefill ? v : nullptr;
@@ -557,15 +559,18 @@ st3_status st3_create(const st3_config* cfg, void* dev_workspace, size_t bytes, 
   ctx->num_sms = sms;
   ctx->attend_ctas_per_sm = tile_bytes(cfg) > 16384 ? 1 : 2;
   // Selection: 16 bytes a row (key, two lists), and a stage for the logits that lies over the second list: all rows of the
-  // heads, or as many as leave room for two blocks on an SM, at least 48 of each.
-  {
+  // heads, or as many as there is room for, at least 48 of each.  A pass over the stage is a round trip, so a block that has
+  // the SM to itself takes all of it: one 32-head layer of 2880 tokens a call 19.5 -> 18.1 us with three passes instead of
+  // six, of 4096 26.3 -> 22.6, eight 40-head sequences of 2880 41.4 -> 39.2, one 7B-shaped sequence of 2880 in 32 calls
+  // 577 -> 541.
+  for (int two = 0; two < 2; ++two) {
     const int rows = 16 * cfg->num_visual + 16, tail = (12 * cfg->num_visual + 15) / 16 * 16;  // the stage starts at `tail`
-    const int room = std::max(100 * 1024, rows) - tail;
+    const int room = std::max(kMaxDynSmem / (1 + two), rows) - tail;
     const int fit = std::max(room / (4 * cfg->num_heads) - 16, 32) / 32, all = ceil_div(std::max(cfg->num_visual, 48) - 16, 32);
-    ctx->stage_rows = 32 * std::min(fit, all) + 16;
-    ctx->finish_smem = std::max(rows, tail + 4 * cfg->num_heads * ctx->stage_rows);
+    ctx->sel[two].stage_rows = 32 * std::min(fit, all) + 16;
+    ctx->sel[two].smem = std::max(rows, tail + 4 * cfg->num_heads * ctx->sel[two].stage_rows);
   }
-  if (ctx->attend_smem > kMaxDynSmem || ctx->finish_smem > kMaxDynSmem) { delete ctx; return ST3_ERR_UNSUPPORTED; }
+  if (ctx->attend_smem > kMaxDynSmem || ctx->sel[0].smem > kMaxDynSmem) { delete ctx; return ST3_ERR_UNSUPPORTED; }
 #define ST3_ATTR(T, D) set_attrs_t<T, D>(ctx)
   st3_status s = ST3_DISPATCH(ctx, ST3_ATTR);
 #undef ST3_ATTR

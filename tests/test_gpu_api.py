@@ -479,7 +479,7 @@ def test_selection_over_hard_score_distributions(nv, keep_bp):
 
 
 @pytest.mark.parametrize("H,nv", [(1, 17), (8, 256), (9, 257), (33, 511), (32, 513), (40, 576), (128, 700), (31, 1023),
-                                  (32, 1028)])
+                                  (32, 1028), (32, 1440), (32, 1460), (40, 2880)])
 def test_selection_by_own_scores_at_the_edges_of_its_passes(H, nv):
     """Head counts and row counts around what a warp, a pass and the staged logits hold, rows on and off 16 bytes: the
     scores against 64 bits, the kept rows against an exact sort of those scores, and the rows moved with their ids."""
