@@ -656,33 +656,58 @@ def test_more_heads_sequences_and_layers_than_a_grid_dimension_holds():
         assert (cb == c).all() and torch.equal(ia[:, :c].expand(nb, c), ib[:, :c])
 
 
-@pytest.mark.parametrize("nv,threads", [(6399, 512), (6400, 1024)])
-def test_half_size_selection_blocks_up_to_what_two_of_them_leave_of_an_sm(nv, threads):
-    """Many units: two selection blocks of 512 threads to an SM, as long as their shared memory fits twice."""
-    nb, D = 150, 64
-    cfg = B.make_config(num_layers=1, num_heads=1, head_dim=D, dtype="bf16", batch=nb, sys_len=1, num_visual=nv,
-                        max_text_len=2, max_decode_steps=1, stride=1, step_ratio_bp=0, first_prune_layer=0, tau=4.0)
+def _check_selection_launches(nb, nv, H, kernel):
+    """A prompt and two steps of `nb` sequences in one layer, through the named form of the selection kernel only: outputs
+    and scores against 64 bits, the kept rows against an exact sort of the scores, and the rows moved with their ids."""
+    D, sys_len, text, steps = 64, 1, 2, 2
+    cfg = B.make_config(num_layers=1, num_heads=H, head_dim=D, dtype="bf16", batch=nb, sys_len=sys_len, num_visual=nv,
+                        max_text_len=text, max_decode_steps=steps, stride=1, step_ratio_bp=0, first_prune_layer=0, tau=8.0)
     ctx = B.Context(cfg)
     try:
         g = torch.Generator(device="cuda").manual_seed(nv)
         rows = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
-        q, K, V = rows(1, nb, 1, D), rows(1, nb, 1, nv + 3, D), rows(1, nb, 1, nv + 3, D)
+        K, V = rows(nb, H, sys_len + nv + text, D), rows(nb, H, sys_len + nv + text, D)
+        q, kn, vn = (rows(steps + 1, 1, nb, H, D) for _ in range(3))
         out = torch.empty_like(q)
-        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA], acc_events=True) as prof:
-            ctx.prefill_select(q, K, V, [2] * nb, out)
-            torch.cuda.synchronize()
-        names = [e.key for e in prof.key_averages() if "st3_finish_kernel" in e.key]
-        assert len(names) == 1 and f", {threads}>" in names[0], names
-        p = torch.softmax(torch.einsum("bd,btd->bt", q[0, :, 0].double(), K[0, :, 0].double()) / D ** 0.5, dim=1)
-        ref = torch.einsum("bt,btd->bd", p, V[0, :, 0].double())
-        assert (out[0, :, 0].double() - ref).abs().max() <= 2e-2 * ref.abs().max()
-        ids, cnt, mass = ctx.get_kept(0)
-        n = nv // 2
-        assert (cnt == n).all() and ctx.status() == 0
-        cut = mass.sort(dim=1, descending=True).values[:, n - 1:n]                 # the kept are the n best
-        assert (mass.gather(1, ids[:, :n].long()) >= cut).all()
+        held = torch.ones(nb, nv, dtype=torch.bool, device="cuda")
+        keys, vals = K, V
+        for t in range(steps + 1):
+            with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA], acc_events=True) as prof:
+                if t == 0:
+                    ctx.prefill_select(q[0], K[None], V[None], [text] * nb, out[0])
+                else:
+                    ctx.decode_step(t, q[t], kn[t], vn[t], out[t])
+                torch.cuda.synchronize()
+            names = [e.key for e in prof.key_averages() if "st3_finish_kernel" in e.key]
+            assert len(names) == 1 and kernel in names[0], names
+            if t:
+                keys, vals = (torch.cat([x, n[t, 0][:, :, None]], 2) for x, n in ((keys, kn), (vals, vn)))
+            gone = torch.zeros(nb, keys.shape[2], dtype=torch.bool, device="cuda")
+            gone[:, sys_len:sys_len + nv] = ~held
+            x = torch.einsum("bhd,bhtd->bht", q[t, 0].double(), keys.double()) / D ** 0.5
+            p = torch.softmax(x.masked_fill(gone[:, None], float("-inf")), dim=2)
+            ref = torch.einsum("bht,bhtd->bhd", p, vals.double())
+            assert (out[t, 0].double() - ref).abs().max() <= 2e-2 * ref.abs().max()
+            ids, cnt, mass = ctx.get_kept(0)
+            want = p[:, :, sys_len:sys_len + nv].sum(1)
+            assert torch.allclose(mass[held].double(), want[held], rtol=5e-4, atol=0)   # fp32 dot products and ex2.approx
+            n = B.st3_schedule_count(cfg, 0, t)
+            best = mass.masked_fill(~held, -1.0).sort(dim=1, descending=True, stable=True).indices[:, :n]
+            assert (cnt == n).all() and torch.equal(ids[:, :n].sort(dim=1).values, best.sort(dim=1).values.int())
+            held = torch.zeros_like(held).scatter_(1, best, True)
+        for b, h in ((0, 0), (nb - 1, H - 1)):
+            kv, vv, _, _ = ctx.get_rows(0, b, h)
+            at = sys_len + ids[b, :n].long()
+            assert torch.equal(kv[:n], K[b, h, at]) and torch.equal(vv[:n], V[b, h, at])
+        assert ctx.status() == 0
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("nv,H,kernel", [(6399, 3, "64, 2, 512>"), (6400, 3, "64, 1, 1024>"), (700, 33, "64, 2, 512>")])
+def test_half_size_selection_blocks_up_to_what_two_of_them_leave_of_an_sm(nv, H, kernel):
+    """More units than SMs: two selection blocks of 512 threads to an SM, as long as their shared memory fits twice."""
+    _check_selection_launches(150, nv, H, kernel)
 
 
 def test_profile_counts_the_copy_of_a_prompts_kept_rows():
