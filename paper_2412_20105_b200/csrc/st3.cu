@@ -284,22 +284,26 @@ st3_status launch_step_t(st3_ctx* ctx, StepParams& p, cudaStream_t st, bool pref
   {
     // Also a programmatic dependent launch: the attention kernel allows it at its start, the blocks become
     // resident as that grid drains, read their parameters and wait for all of it.
-    // Two blocks per SM (with half the registers each) once the units outnumber the SMs (see st3_finish.cuh), as long as
-    // they fit: up to 6399 visual tokens; beyond, one of twice the threads.  Selection launches, the former blocks of up to
-    // 1024 threads with logits in registers / now: 296 units of 6399 tokens 31.7 / 27.9 us, 300 of 6400 48.7 / 43.5, 300 of
-    // 144 with 8 heads 16.0 / 14.4, 100 (one block an SM) of 2880 18.4 / 17.1; slower where rows are odd in number, many and
-    // of many heads (4-byte copies): 8 of 2877 with 40 heads 29.3 / 31.5.
-    const bool many = units > ctx->num_sms, two = many && 2 * ctx->sel[1].smem <= kMaxDynSmem;
+    // A unit is a (layer, sequence): one trimming block, and as many output blocks as give every warp one head (a warp merges
+    // one head after another, a round trip each) while the launch fits the GPU at once: 7B layers one a call 8.97 -> 8.69 ms a
+    // generation, 13B layers of 16 sequences 24.6 -> 23.7, two NeXT sequences in four layers of 32 heads 3.76 -> 2.96.
+    // Up to half as many units as SMs, blocks have an SM to themselves: 512 threads with 128 registers.  Beyond, output blocks
+    // come in waves after the others: 1024 threads, which merge 32 heads at a time, up to three quarters; from there two blocks
+    // to an SM (half the registers and the shared memory) where those stage all rows, or where even the trimming blocks
+    // outnumber the SMs, as long as two fit (up to 6399 tokens).  Decode steps of one layer, us, one block of 512 / of 1024 /
+    // two of 512: 75 units of 16 heads and 1152 tokens 41.9 / 40.8 / 42.2, 100 of 32 and 576 56.9 / 54.2 / 54.9, 115 of 32 and
+    // 576 64.9 / 62.1 / 61.4, 128 of 16 and 1152 64.3 / 62.0 / 61.8, 148 of 32 and 576 79.8 / 76.8 / 74.9, 148 of 32 and 2880
+    // (several passes) 286.4 / 281.9 / 286.2, 149 of 40 and 576 - / 96.0 / 91.3; units below half, 64 of 1 and 2880 16.0 / 16.5.
+    const int sms = ctx->num_sms;
+    const bool crowded = 2 * units > sms, one_pass = ctx->sel[1].stage_rows >= c.num_visual;
+    const bool two = (units > sms || (4 * units > 3 * sms && one_pass)) && 2 * ctx->sel[1].smem <= kMaxDynSmem;
     auto kernel = two ? st3_finish_kernel<T, D, 2, kFinishThreads>
-                  : many ? st3_finish_kernel<T, D, 1, 2 * kFinishThreads> : st3_finish_kernel<T, D, 1, kFinishThreads>;
-    // A warp merges one head after another, a round trip each: as many output blocks as give every warp one head, while the
-    // whole launch (a block to an SM) fits the GPU at once.  7B layers one a call 8 973 -> 8 694 us a generation, 13B layers
-    // of 16 sequences 24 585 -> 23 740, two NeXT sequences in four layers of 32 heads 3 760 -> 2 958.
-    const int out_blocks = std::max(1, std::min(ceil_div(c.num_heads, kFinishThreads / 32), ctx->num_sms / units - 1));
+                  : crowded ? st3_finish_kernel<T, D, 1, 2 * kFinishThreads> : st3_finish_kernel<T, D, 1, kFinishThreads>;
+    const int out_blocks =
+        std::max(1, std::min(ceil_div(c.num_heads, kFinishThreads / 32), (two ? 2 : 1) * sms / units - 1));
     const dim3 grid((unsigned)c.batch, (unsigned)p.layer_count, (unsigned)(1 + out_blocks));
     p.stage_rows = ctx->sel[two].stage_rows;
-    if (launch(kernel, grid, many && !two ? 2 * kFinishThreads : kFinishThreads, ctx->sel[two].smem, pdl, st,
-               p) != cudaSuccess)
+    if (launch(kernel, grid, crowded && !two ? 2 * kFinishThreads : kFinishThreads, ctx->sel[two].smem, pdl, st, p) != cudaSuccess)
       return ST3_ERR_CUDA;
   }
   ctx->launches += 2;

@@ -710,6 +710,15 @@ def test_half_size_selection_blocks_up_to_what_two_of_them_leave_of_an_sm(nv, H,
     _check_selection_launches(150, nv, H, kernel)
 
 
+@pytest.mark.parametrize("nb,nv,H,kernel", [(74, 300, 33, "64, 1, 512>"), (75, 300, 33, "64, 1, 1024>"),
+                                            (111, 577, 32, "64, 1, 1024>"), (112, 577, 32, "64, 2, 512>"),
+                                            (112, 1500, 32, "64, 1, 1024>"), (148, 300, 17, "64, 2, 512>")])
+def test_selection_blocks_of_a_crowded_launch(nb, nv, H, kernel):
+    """From half as many units as SMs, blocks of 1024 threads; from three quarters, two blocks to an SM if they hold all rows
+    at a time (148 SMs)."""
+    _check_selection_launches(nb, nv, H, kernel)
+
+
 def test_profile_counts_the_copy_of_a_prompts_kept_rows():
     """The select/compact time of a prompt holds the copy of the kept rows: it is no shorter than their bytes take at
     8 TB/s, less what the L2 cache (126 MB) may still hold of either side.  The selection alone is far shorter."""
