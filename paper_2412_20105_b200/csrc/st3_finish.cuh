@@ -38,9 +38,9 @@ __device__ __forceinline__ void merge_stats(const float2* ml, long long item0, i
 constexpr int kSelBins = 256;   // bins of the selection's histogram, over the range of the scores; eight to a lane
 constexpr int kSelCand = 64;    // keys of the bin that the cut falls into that are ranked directly
 
-// BPS blocks of NT threads to an SM: one of 512 with 128 registers a thread, two of them when a launch has more (layer,
-// sequence) units than the GPU holds blocks (the work of a unit is a chain of round trips, and more units in flight end
-// sooner), or one of 1024 where two do not fit.  Bound by latency: two round trips, the flag, and dependent integer work in
+// BPS blocks of NT threads to an SM: one of 512 with 128 registers a thread, one of 1024, or two of 512, as the launch has
+// more (layer, sequence) units (st3.cu has the rule: the work of a unit is a chain of round trips, and more units in flight
+// end sooner).  Bound by latency: two round trips, the flag, and dependent integer work in
 // between, which a warp issues at 6-10 cycles an instruction; threads that have no row only take issue slots.  The same code
 // with 1024 threads of 64 registers: 7B layers one a call 9 760 against 9 190 us a generation, 13B layers of 16 sequences
 // 26 680 against 25 670.
