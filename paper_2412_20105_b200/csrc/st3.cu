@@ -293,7 +293,7 @@ st3_status launch_step_t(st3_ctx* ctx, StepParams& p, cudaStream_t st, bool pref
     // outnumber the SMs, as long as two fit (up to 6399 tokens).  Decode steps of one layer, us, one block of 512 / of 1024 /
     // two of 512: 75 units of 16 heads and 1152 tokens 41.9 / 40.8 / 42.2, 100 of 32 and 576 56.9 / 54.2 / 54.9, 115 of 32 and
     // 576 64.9 / 62.1 / 61.4, 128 of 16 and 1152 64.3 / 62.0 / 61.8, 148 of 32 and 576 79.8 / 76.8 / 74.9, 148 of 32 and 2880
-    // (several passes) 286.4 / 281.9 / 286.2, 149 of 40 and 576 - / 96.0 / 91.3; units below half, 64 of 1 and 2880 16.0 / 16.5.
+    // (several passes) 286.4 / 281.9 / 286.2; below half, 64 of 1 and 2880 16.0 / 16.5.
     const int sms = ctx->num_sms;
     const bool crowded = 2 * units > sms, one_pass = ctx->sel[1].stage_rows >= c.num_visual;
     const bool two = (units > sms || (4 * units > 3 * sms && one_pass)) && 2 * ctx->sel[1].smem <= kMaxDynSmem;

@@ -253,9 +253,9 @@ __global__ void __launch_bounds__(NT, BPS) st3_finish_kernel(const __grid_consta
   }
   // A lane sums every eighth head of four rows (a warp: 16 rows); the sums meet in shuffles that leave a lane with one row, and
   // take a third of the shared-memory reads that a row per lane takes (1 540 -> 700 cycles a pass of 256 rows of 32 heads).
-  // Every fourth head (32 rows) where 16 warps of 16 rows do not hold all rows: a small fp32 layer 186 -> 183.5 us a generation, a
-  // prompt of 32 7B layers 1 227 -> 1 206; with 40 heads it loses (24 590 -> 24 690 us).  One choice for all passes and for
-  // every size of the block and its stage: it decides the order in which a row's heads are added, and rows with equal logits
+  // Every fourth head (32 rows) where 16 warps of 16 rows do not hold all rows: a small fp32 layer 186 -> 183.5 us a
+  // generation, a prompt of 32 7B layers 1 227 -> 1 206; with 40 heads, ten to a lane, it loses (24 590 -> 24 690 us).  One
+  // choice for all passes and for every size of the block and its stage: it decides the order in which a row's heads are added, and rows with equal logits
   // must get equal scores, also in two layers of a stage that are selected in different launches.
   const int lq = n_cur > 256 && H <= 32 ? 3 : 2;  // log2 of the row quads of a warp
   for (int c0 = 0; own_scores && c0 < n_cur; c0 += pitch) {
